@@ -269,6 +269,7 @@ lace_status pairconv_per_instance(lace_batch* b, cudaStream_t s, int* launches) 
                 tb.g2[a] = c->g2_f[a].as<float>();
             }
             tb.ktab = c->ktab_f.as<float>();
+            tb.klanes = c->klanes.as<float>();
             const size_t ng = c->g.ng;
             const int batch = (int)std::max<size_t>(
                 1, std::min<size_t>({(size_t)b->h_ngrids[q], part / ng, epart / (2 * (size_t)c->g.n[0]), (size_t)1024}));

@@ -128,6 +128,12 @@ lace_status build_tables(lace_ctx* c) {
             }
     CK(c->ktab_f.ensure(c->g.ng * sizeof(float)), "tables");
     CK(cudaMemcpy(c->ktab_f.p, kt.data(), c->g.ng * sizeof(float), cudaMemcpyHostToDevice), "tables");
+    if (c->prec != LACE_FP64 && lanes_ok(c->g.n)) {
+        CK(c->klanes.ensure(c->g.ng * sizeof(float)), "tables");
+        // on the stream of the copy above: it need not have reached the device yet
+        CK(lanes_ktab(c->g.n, c->ktab_f.as<float>(), c->klanes.as<float>(), nullptr), "tables");
+        CK(cudaStreamSynchronize(nullptr), "tables");
+    }
     CK(c->ktab_d.ensure(c->g.ng * sizeof(double)), "tables");
     CK(cudaMemcpy(c->ktab_d.p, ktd.data(), c->g.ng * sizeof(double), cudaMemcpyHostToDevice), "tables");
     return LACE_OK;
@@ -144,6 +150,7 @@ template <> FFTTables<float> tables<float>(lace_ctx* c) {
     FFTTables<float> t;
     for (int a = 0; a < 3; ++a) { t.tw[a] = c->tw_f[a].as<float2>(); t.g2[a] = c->g2_f[a].as<float>(); }
     t.ktab = c->ktab_f.as<float>();
+    t.klanes = lanes_ok(c->g.n) ? c->klanes.as<float>() : nullptr;
     return t;
 }
 
@@ -527,7 +534,7 @@ lace_status make_pairs(lace_ctx* c, bool use_S, double thr, Launch& L) {
         CK(cudaMemcpyAsync(c->pairs.p, hp.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, c->stream), "pairs");
         CK(cudaStreamSynchronize(c->stream), "pairs");
     }
-    CK(pack_pair_grids(c->pairs.as<int2>(), np, c->grids.as<PairGrid>(), c->stream, &L.n), "pack pairs");
+    CK(pack_pair_grids(c->pairs.as<int2>(), np, n, c->grids.as<PairGrid>(), c->stream, &L.n), "pack pairs");
     c->n_pairs = np;
     return LACE_OK;
 }
@@ -593,6 +600,7 @@ lace_status exchange_prepare_f(lace_ctx* c, MergedSys<float>* m, int* n_grids_ou
     m->psi = c->psi.as<float>();
     m->W = c->W.as<float>();
     m->ktab = c->ktab_f.as<float>();
+    m->klanes = c->klanes.as<float>();
     m->grids = c->grids.as<PairGrid>();
     m->scratch = c->scratch.as<float2>();
     m->epart = c->epart.as<double>();
@@ -912,6 +920,7 @@ lace_status lace_destroy(lace_ctx* c) {
     for (int a = 0; a < 3; ++a) { c->tw_d[a].release(); c->tw_f[a].release(); c->g2_d[a].release(); c->g2_f[a].release(); }
     c->ktab_f.release();
     c->ktab_d.release();
+    c->klanes.release();
     for (auto& e : c->ev) if (e) cudaEventDestroy(e);
     if (c->io_in) {
         cudaStreamSynchronize(c->io_in);
@@ -1349,7 +1358,7 @@ lace_status lace_get_device_bytes(lace_ctx* c, unsigned long long* bytes_out) {
     if (!c || !bytes_out) return LACE_ERR_ARG;
     const DevBuf* bufs[] = {&c->psi,   &c->canon, &c->W,      &c->xi,    &c->stage64, &c->scratch, &c->work,
                             &c->aux,   &c->mat,   &c->pairs,  &c->counts, &c->grids,  &c->epart,   &c->flag,
-                            &c->piv,   &c->pivfull, &c->exd,  &c->aceio, &c->ktab_f, &c->ktab_d, &c->ref,
+                            &c->piv,   &c->pivfull, &c->exd,  &c->aceio, &c->ktab_f, &c->ktab_d, &c->klanes, &c->ref,
                             &c->pw_idx, &c->pw_io,  &c->pw_real};
     unsigned long long b = 0;
     for (const DevBuf* d : bufs) b += d->bytes;

@@ -64,6 +64,7 @@ struct lace_ctx {
     DevBuf tw_d[3], tw_f[3], g2_d[3], g2_f[3];
     DevBuf ktab_f;  // K(G)/Ng rounded once from FP64 (FP32 path)
     DevBuf ktab_d;  // K(G)/Ng (FP64 path)
+    DevBuf klanes;  // -K(G)/Ng in the order of the lane passes (FP32 path)
     int kernel_kind = LACE_KERNEL_COULOMB;
     double kernel_omega = 0.0, kernel_alpha = 1.0;
 

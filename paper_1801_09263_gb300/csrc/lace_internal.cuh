@@ -26,11 +26,12 @@ template <typename T> struct FFTTables {
     cplx<T>* tw[3] = {nullptr, nullptr, nullptr};  // exp(-2 pi i m / n_a), m < n_a
     T* g2[3] = {nullptr, nullptr, nullptr};         // (2 pi m / L_a)^2 in FFT order
     T* ktab = nullptr;                              // optional K(G)/Ng table [n1][n2][n3]
+    T* klanes = nullptr;                            // FP32: -K(G)/Ng in the order of the lane passes (null: none)
 };
 
 // One complex FFT grid carries two real pair densities: slot a = (i1, j1),
 // slot b = (i2, j2); j2 < 0 marks an empty slot.  i is an occupied orbital
-// (row of Psi < n_occ), j any row of Psi.
+// (row of Psi < n_occ), j any row of Psi (below or above i).
 struct PairGrid {
     int i1, j1, i2, j2;
 };
@@ -47,6 +48,7 @@ template <typename T> struct MergedSys {
     const T* psi;
     T* W;
     const T* ktab;
+    const T* klanes;  // -K(G)/Ng in the order of the lane passes
     const PairGrid* grids;
     cplx<T>* scratch;
     double* epart;
@@ -62,6 +64,7 @@ template <typename T> struct ConvArgs {
     const T* g2[3];
     T kscale;         // 4 pi / Ng
     const T* ktab;    // K(G)/Ng per grid point, rounded once from FP64 (null: computed in T)
+    const T* klanes = nullptr;  // -K(G)/Ng in the order of the lane passes (pairconv_lanes.cuh)
     const T* psi;
     int n_occ;
     T* W;
@@ -78,15 +81,15 @@ template <typename T> struct ConvArgs {
     const MergedSys<T>* msys = nullptr;
 };
 
-// Size-specialised FP32 passes for cubic grids (pairconv_spec_*.cu): launch
-// pass 0/1/2 (A/B/C) for grid size n if a specialisation exists.
-bool spec_launch_s(int pass, int n, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s);
-bool spec_launch_m(int pass, int n, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s);
-bool spec_launch_l(int pass, int n, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s);
-bool spec_launch_x(int pass, int n, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s);
+// FP32 passes with two lines of a grid in the lanes of every packed
+// instruction (pairconv_lanes.cu): whether a grid takes them, the table
+// -K(G)/Ng in their order (Ng floats) from K(G)/Ng [n1][n2][n3], and the three
+// passes of nb complex grids.
+bool lanes_ok(const int n[3]);
+cudaError_t lanes_ktab(const int n[3], const float* d_ktab, float* d_out, cudaStream_t s);
+bool lanes_launch(const int n[3], int nb, const ConvArgs<float>& P, int g0, cudaStream_t s);
 
-// Grid sizes whose size-specialised passes take merged launches (one grid
-// per CTA, out of place) (pairconv_spec_*.cu).
+// Cubic grid sizes whose pair convolutions the request server merges.
 bool spec_merge_ok(int n);
 
 // The pair convolutions of several systems on one cubic grid size (n in
@@ -232,8 +235,10 @@ cudaError_t gather_columns(const T* psi, size_t ldpsi, int norb, const long long
 // followed by all (i, n_occ + e).  Returns the count in *n_pairs (host).
 cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double thr, bool use_S, int2* d_pairs,
                             int* d_counts, long long* n_pairs, cudaStream_t s, int* launches);
-// Pack pairs two by two into complex FFT grids.
-cudaError_t pack_pair_grids(const int2* d_pairs, long long n_pairs, PairGrid* d_grids, cudaStream_t s, int* launches);
+// Pack pairs two by two into complex FFT grids (an orbital shared by the two
+// pairs of a grid in both i slots).
+cudaError_t pack_pair_grids(const int2* d_pairs, long long n_pairs, int n_occ, PairGrid* d_grids, cudaStream_t s,
+                            int* launches);
 // Fixed-order FP64 sums over up to kSumBlocks blocks; part: kSumBlocks
 // doubles of scratch (one caller at a time per scratch).
 constexpr int kSumBlocks = 128;

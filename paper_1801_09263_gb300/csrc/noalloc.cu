@@ -227,7 +227,7 @@ extern "C" lace_status lace_exchange_pairs_noalloc(const double cell[3], int n1,
         tb.g2[a] = g2 + a * kMaxN;
     }
     if (n_grids > 0) {
-        if (pack_pair_grids(reinterpret_cast<const int2*>(d_pairs), n_pairs, grids, s, &launches) != cudaSuccess)
+        if (pack_pair_grids(reinterpret_cast<const int2*>(d_pairs), n_pairs, n_occ, grids, s, &launches) != cudaSuccess)
             return LACE_ERR_CUDA;
         if (pairconv_run<double>(g, tb, d_psi, n_occ, d_W, grids, (int)n_grids, grid_scratch, batch, epart,
                                  d_pair_e, s, &launches, nullptr, nullptr) != cudaSuccess)

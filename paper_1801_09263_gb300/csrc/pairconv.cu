@@ -158,6 +158,7 @@ cudaError_t pairconv_run(const GridGeom& g, const FFTTables<T>& tb, const T* psi
     }
     P.kscale = (T)(4.0 * M_PI / (double)g.ng);
     P.ktab = tb.ktab;
+    P.klanes = tb.klanes;
     P.psi = psi;
     P.n_occ = n_occ;
     P.W = W;
@@ -190,7 +191,7 @@ cudaError_t pairconv_run(const GridGeom& g, const FFTTables<T>& tb, const T* psi
         if (dev < 64) attr_done.fetch_or(1ull << dev);
     }
     {
-        // the out-of-place passes prefetch into L2 what the CTA two waves
+        // the lane passes prefetch into L2 what the CTA two waves
         // later (at two CTAs per SM) will read
         int nsm = 0;
         if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev))) return e;
@@ -201,20 +202,15 @@ cudaError_t pairconv_run(const GridGeom& g, const FFTTables<T>& tb, const T* psi
         P.pf_ahead = per_sm * nsm;
     }
     if (sm_plane > (size_t)INT32_MAX || sm_slab > (size_t)INT32_MAX) return cudaErrorInvalidValue;
-    // size-specialised FP32 kernels for even cubic grids of the specialised
-    // sizes (their planes start on 16-byte boundaries; LACE_GENERIC_FFT=1 to disable)
+    // FP32 grids that the lane passes take (LACE_GENERIC_FFT=1: the generic passes)
     const char* gen = getenv("LACE_GENERIC_FFT");
-    const bool spec_ok = !(gen && gen[0] == '1') && g.n[0] == g.n[1] && g.n[1] == g.n[2] && g.n[0] % 2 == 0;
+    const bool use_lanes = std::is_same<T, float>::value && tb.klanes && !(gen && gen[0] == '1') && lanes_ok(g.n);
     if (ev0) cudaEventRecord(ev0, s);
     for (int g0 = 0; g0 < n_grids; g0 += batch) {
         const int nb = std::min(batch, n_grids - g0);
         bool done = false;
         if constexpr (std::is_same<T, float>::value) {
-            if (spec_ok) {
-                for (int pass = 0; pass < 3; ++pass)
-                    done = spec_launch_s(pass, g.n[0], nb, P, g0, s) || spec_launch_m(pass, g.n[0], nb, P, g0, s) ||
-                           spec_launch_l(pass, g.n[0], nb, P, g0, s) || spec_launch_x(pass, g.n[0], nb, P, g0, s);
-            }
+            if (use_lanes) done = lanes_launch(g.n, nb, P, g0, s);
         }
         if (!done) {
             pass_a_kernel<T><<<dim3(g.n[0], nb), kThreads, sm_plane, s>>>(P, g0);
@@ -227,6 +223,11 @@ cudaError_t pairconv_run(const GridGeom& g, const FFTTables<T>& tb, const T* psi
     }
     if (ev1) cudaEventRecord(ev1, s);
     return cudaSuccess;
+}
+
+bool spec_merge_ok(int n) {
+    static const int sizes[] = {24, 32, 36, 40, 48, 50, 54, 60, 64, 72, 80, 96, 100};
+    return std::find(std::begin(sizes), std::end(sizes), n) != std::end(sizes);
 }
 
 cudaError_t pairconv_run_merged(int n, const FFTTables<float>& tb, const std::vector<MergedSys<float>>& sys,
@@ -274,6 +275,7 @@ cudaError_t pairconv_run_merged(int n, const FFTTables<float>& tb, const std::ve
     const size_t ng = (size_t)n * n * n;
     P.kscale = (float)(4.0 * M_PI / (double)ng);
     P.ktab = nullptr;
+    P.klanes = nullptr;
     P.psi = nullptr;
     P.W = nullptr;
     P.grids = nullptr;
@@ -289,11 +291,8 @@ cudaError_t pairconv_run_merged(int n, const FFTTables<float>& tb, const std::ve
     for (int r = 0; r < rounds; ++r) {
         const int g0 = start[r], nb = start[r + 1] - start[r];
         P.msys = d_sys + (size_t)r * nsys;
-        for (int pass = 0; pass < 3; ++pass) {
-            const bool ok = spec_launch_s(pass, n, nb, P, g0, s) || spec_launch_m(pass, n, nb, P, g0, s) ||
-                            spec_launch_l(pass, n, nb, P, g0, s) || spec_launch_x(pass, n, nb, P, g0, s);
-            if (!ok) return cudaErrorInvalidValue;
-        }
+        const int dims[3] = {n, n, n};
+        if (!lanes_launch(dims, nb, P, g0, s)) return cudaErrorInvalidValue;
         energy_collect_merged_kernel<<<(nb + 127) / 128, 128, 0, s>>>(d_refs, P.msys, g0, nb, n);
         *launches += 4;
         if ((e = cudaGetLastError())) return e;

@@ -154,7 +154,7 @@ __device__ __forceinline__ void spec_unit(int phase, const MultiArgs& A, const C
             V.dv = I.P.dv;                                                                 \
             const spec2::Sub<T> grp{(int)threadIdx.x - gi * T, 1 + gi};                    \
             float4* sm = reinterpret_cast<float4*>(smem + (size_t)gi * group_smem(NN));    \
-            if (phase == 0) spec2::body_a<NN, T>(I.P, V, w, sm, nullptr, grp);             \
+            if (phase == 0) spec2::body_a<NN, T>(I.P, V, w, sm, grp);                      \
             else if (phase == 1) spec2::body_b<NN, T>(I.P, V, w, sm, grp);                 \
             else spec2::body_c<NN, T>(I.P, V, w, sm, red + gi * 2 * (T / 32), grp);        \
         }                                                                                  \

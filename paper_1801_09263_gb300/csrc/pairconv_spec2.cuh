@@ -1,7 +1,6 @@
-// Size-specialised FP32 FFT passes of the pair convolutions, out-of-place
-// form.  Same three passes and the same arithmetic as pairconv_spec.cuh
-// (Eq. 2 evaluated with FFTs, Sec. 2; truncated by Eq. 5), laid out for
-// fewer barriers and more memory-level parallelism:
+// Size-specialised FP32 FFT pass bodies of the persistent multi-instance
+// kernel (pairconv_multi.cuh), out of place (Eq. 2 evaluated with FFTs,
+// Sec. 2; truncated by Eq. 5):
 //   * every radix stage reads one shared-memory plane and writes the other
 //     (ping-pong), so a thread keeps one butterfly live and a stage ends in
 //     one barrier instead of two;
@@ -18,9 +17,6 @@
 //     and a group of fixed k2 is one forward and one inverse butterfly.
 //     Pass B needs two barriers; its slab of the K(G)/Ng table is staged in
 //     shared memory by cp.async while the first stage runs;
-//   * passes A and C launch plane-major (the CTAs in flight share one plane
-//     of the orbitals and of W, which then stay in L2), and every CTA
-//     prefetches into L2 what the CTA one wave ahead will read;
 //   * each hand-off between two stages picks the row pitch (n or n + 1
 //     complex values) that keeps the 8-byte accesses of a half-warp on
 //     distinct banks for both stages, found with a bank model of every
@@ -32,9 +28,6 @@
 //     one register pair, so complex additions and products with real
 //     constants are single packed FP32 instructions (dft_packed.cuh).
 #pragma once
-
-#include <atomic>
-#include <cstdlib>
 
 #include "dft_packed.cuh"
 #include "pairconv_spec.cuh"
@@ -148,24 +141,7 @@ struct Sub {
     __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(NT) : "memory"); }
 };
 
-// Hint: fetch bytes (a multiple of 16, 16-byte aligned) at p into L2.
-__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// The CTA pf_ahead launch positions after this one, if any: its
-// blockIdx.x (fast) and blockIdx.y (slow).
-__device__ __forceinline__ bool ahead_cta(int pf_ahead, int& fast, int& slow) {
-    if (pf_ahead <= 0) return false;
-    const long lin = (long)blockIdx.y * gridDim.x + blockIdx.x + pf_ahead;
-    if (lin >= (long)gridDim.x * gridDim.y) return false;
-    fast = (int)(lin % gridDim.x);
-    slow = (int)(lin / gridDim.x);
-    return true;
-}
-
-// The buffers of grid g of a launch: its own system's in a merged launch
-// (the request server), the launch's otherwise.
+// The buffers of one complex grid.
 struct GridView {
     const float* psi;
     float* W;
@@ -176,32 +152,6 @@ struct GridView {
     int n_occ;
     double dv;
 };
-__device__ __forceinline__ GridView grid_view(const ConvArgs<float>& P, int g0, int g, int n1) {
-    GridView v;
-    if (P.refs) {
-        const GridRef r = P.refs[g0 + g];
-        const MergedSys<float>& m = P.msys[r.sys];
-        v.psi = m.psi;
-        v.W = m.W;
-        v.ktab = m.ktab;
-        v.d = m.grids[r.g];
-        v.scr = m.scratch + (size_t)(r.g - m.g0) * P.ng;
-        v.ep = m.epart + (size_t)(r.g - m.g0) * n1 * 2;
-        v.n_occ = m.n_occ;
-        v.dv = m.dv;
-    } else {
-        v.psi = P.psi;
-        v.W = P.W;
-        v.ktab = P.ktab;
-        v.d = P.grids[g0 + g];
-        v.scr = P.scratch + (size_t)g * P.ng;
-        v.ep = P.epart + (size_t)g * n1 * 2;
-        v.n_occ = P.n_occ;
-        v.dv = P.dv;
-    }
-    return v;
-}
-
 // One radix-R Stockham stage over LINES lines of length N, out of place, on
 // NT threads (tid: this thread's index among them): butterfly i of a line
 // reads elements i + t N/R through ld(line, e), multiplies by w_{P R}^{t k}
@@ -240,11 +190,10 @@ __device__ __forceinline__ void stage(int tid, const C* __restrict__ tw, Ld ld, 
 }
 
 // Pass A, one plane: rho of plane x of grid V, forward FFT along z then y,
-// on the NT threads of grp (the thread block, or a group of it).  pf_plane: an orbital plane to fetch into
-// L2 at the end (or null).
+// on the NT threads of grp (the thread block, or a group of it).
 template <int N, int NT, class G = Cta>
 __device__ __forceinline__ void body_a(const ConvArgs<float>& P, const GridView& V, int x, float4* smem_v4,
-                                       const float* pf_plane, G grp = G()) {
+                                       G grp = G()) {
     const int tid = grp.tid();
     static_assert(N % 2 == 0, "pass A reads orbital planes as 16-byte vectors");
     constexpr int NP = N * N;
@@ -302,23 +251,6 @@ __device__ __forceinline__ void body_a(const ConvArgs<float>& P, const GridView&
     C* out = V.scr + off;
     stage<N, pl.r2, pl.r1, -1, N, true, NT>(
         tid, tw, [&](int z, int y) { return b0[y * P23 + z]; }, [&](int z, int y, C v) { out[y * N + z] = v; });
-    if (pf_plane) prefetch_l2(pf_plane, NP * sizeof(float));
-}
-
-// Pass A: rho of plane x, forward FFT along z then y.
-template <int N>
-__global__ void __launch_bounds__(threads_for(N)) __maxnreg__(max_regs(N)) pass_a(ConvArgs<float> P, int g0) {
-    extern __shared__ float4 smem_v4[];
-    const int g = blockIdx.x, x = blockIdx.y;  // plane-major: the CTAs in flight share plane x
-    const GridView V = grid_view(P, g0, g, N);
-    int xa = 0, ga = 0;
-    const float* pf_plane = nullptr;  // orbital plane of the CTA ahead that this thread prefetches
-    if (threadIdx.x < 4 && ahead_cta(P.pf_ahead, ga, xa)) {
-        const GridView A = grid_view(P, g0, ga, N);
-        const int o = threadIdx.x == 0 ? A.d.i1 : threadIdx.x == 1 ? A.d.j1 : threadIdx.x == 2 ? A.d.i2 : A.d.j2;
-        if (o >= 0) pf_plane = A.psi + (size_t)o * P.ng + (size_t)xa * N * N;  // (j2 < 0: one pair)
-    }
-    body_a<N, threads_for(N)>(P, V, x, smem_v4, pf_plane);
 }
 
 // Pass B, one slab: slab ky of grid V: forward x-FFT (decimation in time),
@@ -419,20 +351,6 @@ __device__ __forceinline__ void body_b(const ConvArgs<float>& P, const GridView&
     }
 }
 
-// Pass B: slab ky: forward x-FFT, * K(G)/Ng, inverse x-FFT.
-template <int N>
-__global__ void __launch_bounds__(threads_for(N)) __maxnreg__(max_regs(N)) pass_b(ConvArgs<float> P, int g0) {
-    extern __shared__ float4 smem_v4[];
-    const int g = blockIdx.y, ky = blockIdx.x;
-    const GridView V = grid_view(P, g0, g, N);
-    {
-        int ka = 0, ga = 0;
-        if (threadIdx.x < N && ahead_cta(P.pf_ahead, ka, ga))
-            prefetch_l2(grid_view(P, g0, ga, N).scr + (size_t)threadIdx.x * N * N + (size_t)ka * N, N * sizeof(C));
-    }
-    body_b<N, threads_for(N)>(P, V, ky, smem_v4);
-}
-
 // Pass C, one plane: inverse FFT along y then z of plane x of grid V, then
 // the W updates (16-byte vector reductions) and the real-space pair
 // energies.  The NT threads of grp; red: 2 x (NT / 32) doubles of shared
@@ -455,16 +373,6 @@ __device__ __forceinline__ void body_c(const ConvArgs<float>& P, const GridView&
     const C* in = V.scr + off;
     stage<N, pl.r1, 1, +1, N, true, NT>(
         tid, tw, [&](int z, int y) { return in[y * N + z]; }, [&](int z, int y, C v) { b0[y * P01 + z] = v; });
-    if (P.pf_ahead > 0 && tid < 8) {
-        // the epilogue's orbital planes and W planes, fetched into L2 while
-        // the FFT stages run
-        const int q = tid & 3;
-        const int o = q == 0 ? d.i1 : q == 1 ? d.j1 : q == 2 ? d.i2 : d.j2;
-        if (o >= 0) {
-            const float* src = (tid < 4 ? V.psi : V.W) + (size_t)o * P.ng + off;
-            prefetch_l2(src, NP * sizeof(float));
-        }
-    }
     grp.sync();
     stage<N, pl.r2, pl.r1, +1, N, true, NT>(
         tid, tw, [&](int z, int y) { return b0[y * P01 + z]; }, [&](int z, int y, C v) { b1[y * P12 + z] = v; });
@@ -551,72 +459,5 @@ __device__ __forceinline__ void body_c(const ConvArgs<float>& P, const GridView&
     }
 }
 
-// Pass C: inverse FFT along y then z of plane x, W updates and pair energies.
-template <int N>
-__global__ void __launch_bounds__(threads_for(N)) __maxnreg__(max_regs(N)) pass_c(ConvArgs<float> P, int g0) {
-    extern __shared__ float4 smem_v4[];
-    __shared__ double red[2 * ((threads_for(N) + 31) / 32)];
-    const int g = blockIdx.x, x = blockIdx.y;  // plane-major: the CTAs in flight share plane x
-    const GridView V = grid_view(P, g0, g, N);
-    {
-        int xa = 0, ga = 0;
-        if (threadIdx.x == 32 && ahead_cta(P.pf_ahead, ga, xa))
-            prefetch_l2(grid_view(P, g0, ga, N).scr + (size_t)xa * N * N, N * N * sizeof(C));
-    }
-    body_c<N, threads_for(N)>(P, V, x, smem_v4, red);
-}
-
-// Launch pass 0/1/2 of a batch of nb complex grids.
-template <int N>
-bool launch_one(int pass, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
-    static std::atomic<unsigned long long> attr_done{0};  // one bit per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && !(attr_done.load() & (1ull << dev))) {
-        cudaFuncSetAttribute(pass_a<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(N, 0));
-        cudaFuncSetAttribute(pass_b<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(N, 1));
-        cudaFuncSetAttribute(pass_c<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(N, 2));
-        cudaFuncSetAttribute(pass_a<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(pass_b<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        cudaFuncSetAttribute(pass_c<N>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-        attr_done.fetch_or(1ull << dev);
-    }
-    const size_t sm = smem_bytes(N, pass);
-    constexpr int NT = threads_for(N);
-    if (pass == 0) pass_a<N><<<dim3(nb, N), NT, sm, s>>>(P, g0);
-    else if (pass == 1) pass_b<N><<<dim3(N, nb), NT, sm, s>>>(P, g0);
-    else pass_c<N><<<dim3(nb, N), NT, sm, s>>>(P, g0);
-    return true;
-}
-
-// LACE_FFT_INPLACE=1 selects the in-place passes of pairconv_spec.cuh (kept
-// for comparison and for grids whose two planes do not fit on chip).
-inline bool enabled() {
-    static const int on = [] {
-        const char* e = getenv("LACE_FFT_INPLACE");
-        return (e && e[0] == '1') ? 0 : 1;
-    }();
-    return on != 0;
-}
-
 }  // namespace spec2
-
-namespace spec {
-
-// The out-of-place passes where two planes fit in shared memory, else the
-// in-place ones.  A merged launch (several systems, P.refs) takes the
-// out-of-place passes or none.
-template <int N>
-bool launch_any(int pass, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
-    if constexpr (spec2::smem_max(N) <= 200 * 1024) {
-        // merged launches (P.refs) exist only in the one-grid out-of-place passes
-        if (spec2::enabled() || P.refs) return spec2::launch_one<N>(pass, nb, P, g0, s);
-    }
-    if (P.refs) return false;
-    // the in-place passes read rows as 16-byte vectors: n % 4 == 0 only
-    if constexpr (N % 4 == 0) return spec_launch_one<N>(pass, nb, P, g0, s);
-    return false;
-}
-
-}  // namespace spec
 }  // namespace lace

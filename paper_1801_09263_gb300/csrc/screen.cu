@@ -72,16 +72,30 @@ __global__ void write_pairs_kernel(int n_occ, int n_extra, const double* __restr
     for (int e = threadIdx.x; e < n_extra; e += blockDim.x) pairs[base + e] = make_int2(i, n_occ + e);
 }
 
-__global__ void pack_kernel(const int2* __restrict__ pairs, long long n_pairs, PairGrid* __restrict__ grids,
-                            long long n_grids) {
+// Two pairs of one grid that share an occupied orbital both take it as i (a
+// pair of occupied orbitals is symmetric): the passes then read it once and
+// add to its W once, three orbital reads and three W updates a grid instead
+// of four.
+__global__ void pack_kernel(const int2* __restrict__ pairs, long long n_pairs, int n_occ,
+                            PairGrid* __restrict__ grids, long long n_grids) {
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (g >= n_grids) return;
-    const int2 a = pairs[2 * g];
+    int2 a = pairs[2 * g];
     PairGrid d;
+    int2 b = make_int2(-1, -1);
+    if (2 * g + 1 < n_pairs) {
+        b = pairs[2 * g + 1];
+        const bool a_occ = a.y < n_occ, b_occ = b.y < n_occ;
+        const int shared = (a.x == b.x || (b_occ && a.x == b.y)) ? a.x
+                           : (a_occ && (a.y == b.x || (b_occ && a.y == b.y))) ? a.y : -1;
+        if (shared >= 0) {
+            if (a.x != shared) a = make_int2(a.y, a.x);
+            if (b.x != shared) b = make_int2(b.y, b.x);
+        }
+    }
     d.i1 = a.x;
     d.j1 = a.y;
     if (2 * g + 1 < n_pairs) {
-        const int2 b = pairs[2 * g + 1];
         d.i2 = b.x;
         d.j2 = b.y;
     } else {
@@ -161,11 +175,11 @@ cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double th
     return e;
 }
 
-cudaError_t pack_pair_grids(const int2* d_pairs, long long n_pairs, PairGrid* d_grids, cudaStream_t s,
+cudaError_t pack_pair_grids(const int2* d_pairs, long long n_pairs, int n_occ, PairGrid* d_grids, cudaStream_t s,
                             int* launches) {
     const long long n_grids = (n_pairs + 1) / 2;
     if (n_grids == 0) return cudaSuccess;
-    pack_kernel<<<(unsigned)((n_grids + 255) / 256), 256, 0, s>>>(d_pairs, n_pairs, d_grids, n_grids);
+    pack_kernel<<<(unsigned)((n_grids + 255) / 256), 256, 0, s>>>(d_pairs, n_pairs, n_occ, d_grids, n_grids);
     *launches += 1;
     return cudaGetLastError();
 }
