@@ -7,6 +7,7 @@
 #include "f32x2.cuh"
 #include "grid_sync.cuh"
 #include "lace_internal.cuh"
+#include "scdm_rounds.cuh"
 
 namespace lace {
 
@@ -492,288 +493,6 @@ __global__ void gather_columns_kernel(const T* __restrict__ psi, size_t ldpsi, i
     out[e] = (double)psi[(size_t)o * ldpsi + (size_t)idx[p]];
 }
 
-
-// ---------------------------------------------------------------------------
-// Register-resident pivoted QR (FP32): the same Businger-Golub steps as the
-// kernels above (take the live column with the largest residual norm, ties
-// to the lowest index; remove its direction from every column), laid out so
-// that one step is a short dependent chain.  LPC lanes hold one column (RPL
-// rows each), so the q.r dot products and the norms reduce with lane
-// shuffles alone; the columns of a CTA that do not fit in registers live in
-// shared memory with a padded row pitch (16-byte accesses free of bank
-// conflicts).  The row work runs on packed FP32 pairs.  A step makes one
-// pass over each column (the previous step's projection, this step's dot and
-// the squared norm before this step's projection: the residual norm is the
-// difference, |v|^2 - (q.v)^2).  Per step each warp publishes its best
-// column, projected, with its exact squared norm to global memory; the CTAs
-// then agree on the global winner through one 64-bit atomicMax per CTA
-// (key = the FP32 squared norm's bits above the complemented column index:
-// the largest norm, then the lowest index) and a grid barrier on a monotone
-// arrival counter; every CTA reads the winner's published column and scales
-// it by the inverse square root of its published norm (in FP32: FP64 runs
-// at a small fraction of the FP32 rate on this GPU).
-constexpr int QR2_THREADS = 512, QR2_WARPS = QR2_THREADS / 32;
-
-__device__ __forceinline__ unsigned long long ld_cg_u64(const unsigned long long* p) {
-    unsigned long long v;
-    asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// sum over the LPC lanes of one column (consecutive lanes)
-template <int LPC>
-__device__ __forceinline__ float lane_sum(float x) {
-#pragma unroll
-    for (int o = 1; o < LPC; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-}
-
-// One pass over a column chunk held in registers: v <- v - dp qp (the
-// previous step's projection, deferred to this pass), then the partial dot
-// q.v and squared norm v.v of the result.  The stored values and the dot are
-// those of the two-pass form (same products in the same order); only the
-// norm after this step's projection, |v|^2 - (q.v)^2, is formed differently.
-template <int RPL>
-__device__ __forceinline__ void qpass(const float* __restrict__ qp, const float* __restrict__ q, float* v, float dp,
-                                      float& dot, float& ss) {
-    const f2 nd = bc2(-dp);
-    f2 a0 = bc2(0.f), a1 = bc2(0.f), n0 = bc2(0.f), n1 = bc2(0.f);
-#pragma unroll
-    for (int j = 0; j < RPL; j += 4) {
-        const float4 p4 = *reinterpret_cast<const float4*>(qp + j);
-        const float4 q4 = *reinterpret_cast<const float4*>(q + j);
-        const f2 u0 = fma2(mk2(p4.x, p4.y), nd, mk2(v[j], v[j + 1]));
-        const f2 u1 = fma2(mk2(p4.z, p4.w), nd, mk2(v[j + 2], v[j + 3]));
-        a0 = fma2(mk2(q4.x, q4.y), u0, a0);
-        a1 = fma2(mk2(q4.z, q4.w), u1, a1);
-        n0 = fma2(u0, u0, n0);
-        n1 = fma2(u1, u1, n1);
-        unpk2(u0, v[j], v[j + 1]);
-        unpk2(u1, v[j + 2], v[j + 3]);
-    }
-    float x0, x1;
-    unpk2(a0 + a1, x0, x1);
-    dot = x0 + x1;
-    unpk2(n0 + n1, x0, x1);
-    ss = x0 + x1;
-}
-// The same pass over a column chunk in shared memory: one read and (store)
-// one write of the chunk per step.
-template <int RPL>
-__device__ __forceinline__ void spass(const float* __restrict__ qp, const float* __restrict__ q, float* w, float dp,
-                                      bool store, float& dot, float& ss) {
-    const f2 nd = bc2(-dp);
-    f2 a0 = bc2(0.f), a1 = bc2(0.f), n0 = bc2(0.f), n1 = bc2(0.f);
-#pragma unroll 4
-    for (int j = 0; j < RPL; j += 4) {
-        const float4 p4 = *reinterpret_cast<const float4*>(qp + j);
-        const float4 q4 = *reinterpret_cast<const float4*>(q + j);
-        const float4 x = *reinterpret_cast<const float4*>(w + j);
-        const f2 u0 = fma2(mk2(p4.x, p4.y), nd, mk2(x.x, x.y));
-        const f2 u1 = fma2(mk2(p4.z, p4.w), nd, mk2(x.z, x.w));
-        a0 = fma2(mk2(q4.x, q4.y), u0, a0);
-        a1 = fma2(mk2(q4.z, q4.w), u1, a1);
-        n0 = fma2(u0, u0, n0);
-        n1 = fma2(u1, u1, n1);
-        if (store) {
-            float4 o;
-            unpk2(u0, o.x, o.y);
-            unpk2(u1, o.z, o.w);
-            *reinterpret_cast<float4*>(w + j) = o;
-        }
-    }
-    float x0, x1;
-    unpk2(a0 + a1, x0, x1);
-    dot = x0 + x1;
-    unpk2(n0 + n1, x0, x1);
-    ss = x0 + x1;
-}
-
-__device__ __forceinline__ unsigned long long col_key(float nrm, int col) {
-    return ((unsigned long long)__float_as_uint(nrm) << 32) | (unsigned long long)(0xffffffffu - (unsigned)col);
-}
-
-// The columns of CTA b are [b cpb, (b + 1) cpb): the first G = 512 / LPC in
-// registers (group g = thread / LPC), the rest (s = 0, 1, ...) in shared
-// memory, handled by group s % G.  Rows: lane l of a group holds rows
-// [l RPL, (l + 1) RPL); q is kept as LPC row chunks of RPL + 4 floats, so
-// the LPC distinct chunks a warp reads at once fall on different banks.
-//
-// Each step makes one pass over every column: it applies the previous step's
-// projection (v -= d_{k-1} q_{k-1}, deferred from that step), and forms
-// d_k = q_k.v and |v|^2, so the column's norm after step k's projection is
-// |v|^2 - d_k^2 (clamped at 0).  A shared-memory column is read and written
-// once per step instead of read twice and written once.  The published
-// candidate is the projected column v - d_k q_k with its exact squared norm
-// (pnorm), from which the next q is normalised.  keys[npiv] and bar[0] are
-// zero at launch.
-template <int RPL, int LPC>
-__global__ void __launch_bounds__(QR2_THREADS, 1)
-    qr_resident_kernel(int nrow, int ncol, const float* __restrict__ R, int npiv, int cpb, float* __restrict__ pub,
-                       unsigned long long* __restrict__ keys, int* __restrict__ piv, unsigned* bar,
-                       unsigned long long limit_ns) {
-    constexpr int G = QR2_THREADS / LPC;
-    constexpr int NPAD = RPL * LPC;     // padded rows
-    constexpr int PITCH = RPL + 4;      // shared-memory row-chunk pitch (floats)
-    extern __shared__ __align__(16) float qr2_smem[];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = tid / LPC, l = tid % LPC;
-    const int c0 = blockIdx.x * cpb;
-    const int ncta = min(cpb, ncol - c0);  // columns of this CTA
-    const int SC = max(0, ncta - G);       // of them in shared memory
-    const int rounds = (SC + G - 1) / G;
-    const int myreg = g < ncta ? c0 + g : -1;
-    float* qbuf = qr2_smem;                            // 2 x [LPC][PITCH]: q of steps k (k & 1) and k - 1
-    float* sc = qr2_smem + 2 * LPC * PITCH;            // [SC][LPC][PITCH] shared-memory columns
-    float* dsm = sc + (size_t)SC * LPC * PITCH;        // [SC] each shared column's last dot
-    float* pnorm = pub + (size_t)2 * gridDim.x * QR2_WARPS * NPAD;  // [2][CTAs][warps] exact squared norms
-    __shared__ unsigned long long wkey[QR2_WARPS];
-    __shared__ int abort_sh;
-    float v[RPL];
-    float dreg = 0.f;      // the register column's last dot
-    unsigned chosen = 0u;  // bit 0: the register column; bit 1 + r: shared column of round r
-#pragma unroll
-    for (int j = 0; j < RPL; ++j) {
-        const int row = l * RPL + j;
-        v[j] = (myreg >= 0 && row < nrow) ? R[(size_t)row * ncol + myreg] : 0.f;
-    }
-    for (int r = 0; r < rounds; ++r) {
-        const int s = r * G + g;
-        if (s < SC) {
-            float* dst = sc + ((size_t)s * LPC + l) * PITCH;
-            const int col = c0 + G + s;
-            for (int j = 0; j < RPL; ++j) {
-                const int row = l * RPL + j;
-                dst[j] = row < nrow ? R[(size_t)row * ncol + col] : 0.f;
-            }
-        }
-    }
-    for (int j = tid; j < 2 * LPC * PITCH; j += QR2_THREADS) qbuf[j] = 0.f;
-    for (int j = tid; j < SC; j += QR2_THREADS) dsm[j] = 0.f;
-    __syncthreads();
-    for (int step = 0; step < npiv; ++step) {
-        const float* qrow = qbuf + (step & 1) * LPC * PITCH + l * PITCH;        // q_k (zero at step 0)
-        const float* prow = qbuf + ((step + 1) & 1) * LPC * PITCH + l * PITCH;  // q_{k-1}
-        unsigned long long best = 0ull;
-        // register column
-        {
-            float d, ss;
-            qpass<RPL>(prow, qrow, v, dreg, d, ss);
-            d = lane_sum<LPC>(d);
-            ss = lane_sum<LPC>(ss);
-            dreg = d;
-            const float nrm = fmaxf(ss - d * d, 0.f);
-            if (myreg >= 0 && !(chosen & 1u)) best = col_key(nrm, myreg);
-        }
-        // shared-memory columns
-        for (int r = 0; r < rounds; ++r) {
-            const int s = r * G + g;
-            const bool has = s < SC;  // uniform over the LPC lanes of the group
-            float* w = sc + ((size_t)(has ? s : 0) * LPC + l) * PITCH;
-            const float dp = has ? dsm[s] : 0.f;
-            float d, ss;
-            spass<RPL>(prow, qrow, w, dp, has, d, ss);
-            d = lane_sum<LPC>(d);
-            ss = lane_sum<LPC>(ss);
-            if (has && l == 0) dsm[s] = d;
-            if (has && !((chosen >> (1 + r)) & 1u)) {
-                const unsigned long long k = col_key(fmaxf(ss - d * d, 0.f), c0 + G + s);
-                best = k > best ? k : best;
-            }
-        }
-        // warp argmax of the keys
-        unsigned long long wb = best;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long x = __shfl_xor_sync(0xffffffffu, wb, o);
-            wb = x > wb ? x : wb;
-        }
-        // the lanes holding the warp's best column publish it projected
-        // (v - d q) with its exact squared norm
-        __syncwarp();  // this step's dsm writes are visible to the group's lanes
-        const size_t slot = ((size_t)(step & 1) * gridDim.x + blockIdx.x) * QR2_WARPS + warp;
-        const int wcol = (int)(0xffffffffu - (unsigned)(wb & 0xffffffffu));
-        const int ws = wcol - c0 - G;
-        const bool own_reg = wb != 0ull && wcol == myreg;
-        const bool own_sh = wb != 0ull && ws >= 0 && ws < SC && ws % G == g;
-        float pn = 0.f;
-        if (own_reg || own_sh) {
-            float* out = pub + slot * NPAD + l * RPL;
-            const float* src = own_sh ? sc + ((size_t)ws * LPC + l) * PITCH : nullptr;
-            const float d = own_sh ? dsm[ws] : dreg;
-#pragma unroll
-            for (int j = 0; j < RPL; j += 4) {
-                const float4 q4 = *reinterpret_cast<const float4*>(qrow + j);
-                const float4 x = own_sh ? *reinterpret_cast<const float4*>(src + j)
-                                        : make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
-                const float4 o = make_float4(fmaf(-d, q4.x, x.x), fmaf(-d, q4.y, x.y), fmaf(-d, q4.z, x.z),
-                                             fmaf(-d, q4.w, x.w));
-                pn = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, pn))));
-                *reinterpret_cast<float4*>(out + j) = o;
-            }
-        }
-        pn = lane_sum<LPC>(pn);  // every lane takes part; the owner group's lanes get its norm
-        if ((own_reg || own_sh) && l == 0) pnorm[slot] = pn;
-        if (lane == 0) wkey[warp] = wb;
-        // grid barrier: arrive with this CTA's best key, wait for every CTA.
-        // The key goes in first (a relaxed reduction, ordered before the
-        // arrival by its release); waiting CTAs poll with relaxed loads and
-        // a short back-off, then take one acquire fence.
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long kb = 0ull;
-#pragma unroll
-            for (int w = 0; w < QR2_WARPS; ++w) kb = wkey[w] > kb ? wkey[w] : kb;
-            if (kb) asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(keys + step), "l"(kb) : "memory");
-            const unsigned target = (unsigned)(step + 1) * gridDim.x;
-            unsigned cnt;
-            asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(cnt) : "l"(bar) : "memory");
-            int timed_out = 0;
-            if (cnt + 1 < target) {
-                const unsigned long long t0 = global_ns();
-                for (;;) {
-                    unsigned vv;
-                    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(vv) : "l"(bar) : "memory");
-                    if (vv >= target) break;
-                    if (global_ns() - t0 > limit_ns) {
-                        atomicExch(bar + 2, 1u);
-                        timed_out = 1;
-                        break;
-                    }
-                    __nanosleep(40);
-                }
-            }
-            asm volatile("fence.acq_rel.gpu;" ::: "memory");
-            abort_sh = timed_out;
-        }
-        __syncthreads();
-        if (abort_sh) return;
-        const unsigned long long key = ld_cg_u64(keys + step);
-        if (key == 0ull) {  // no live column left: cannot happen for npiv <= ncol
-            if (tid == 0) atomicExch(bar + 2, 2u);
-            return;
-        }
-        const int p = (int)(0xffffffffu - (unsigned)(key & 0xffffffffu));
-        const int wcta = p / cpb, li = p - wcta * cpb;
-        const int wg = li < G ? li : (li - G) % G;
-        const size_t wslot = ((size_t)(step & 1) * gridDim.x + wcta) * QR2_WARPS + (wg * LPC) / 32;
-        // the winner's exact squared norm, published with its column; the
-        // inverse square root in FP32 (FP64 arithmetic in every thread of
-        // every CTA cost ~5 us a step on this GPU's FP64 rate)
-        const float nn = __ldcg(pnorm + wslot);
-        const float inv = nn > 0.f ? 1.f / sqrtf(nn) : 0.f;
-        float* qnext = qbuf + ((step + 1) & 1) * LPC * PITCH;  // q_{k-1} is no longer read
-        for (int j = tid; j < NPAD; j += QR2_THREADS)
-            qnext[(j / RPL) * PITCH + j % RPL] = __ldcg(pub + wslot * NPAD + j) * inv;
-        if (wcta == (int)blockIdx.x && wg == g) {
-            if (li < G) chosen |= 1u;
-            else chosen |= 1u << (1 + (li - G) / G);
-        }
-        if (tid == 0 && blockIdx.x == 0) piv[step] = p;
-        __syncthreads();
-    }
-}
-
 }  // namespace
 
 static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
@@ -781,27 +500,14 @@ static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 // Capacity (in Best entries) of the block-winner buffer of qrcp_aux_bytes.
 static int nblocks_cap(int ncol) { return std::max((ncol + QR_THREADS - 1) / QR_THREADS, 2 * 152 * 8); }
 
-// Row layout of the register-resident QR: RPL rows per lane, LPC lanes per column.
-static void qr2_layout(int nrow, int* rpl, int* lpc) {
-    *rpl = nrow <= 32 ? 32 : 64;
-    *lpc = nrow <= 64 ? 1 : (nrow + 63) / 64 <= 2 ? 2 : (nrow + 63) / 64 <= 4 ? 4 : (nrow + 63) / 64 <= 8 ? 8 : 16;
-}
-
-// Published candidate columns: of the persistent kernel, 2 (step parity) x
-// CTAs (up to 304) x padded rows (< 2 nrow + 64), FP64 at most; of the
-// register-resident kernel, 2 x CTAs x 16 warps x padded rows (FP32).
-static size_t pub_bytes(int nrow) {
-    int rpl = 0, lpc = 0;
-    qr2_layout(nrow, &rpl, &lpc);
-    const size_t old = (size_t)2 * 304 * (2 * (size_t)nrow + 64) * sizeof(double);
-    const size_t res = align256((size_t)2 * 304 * 16 * rpl * lpc * sizeof(float)) + (size_t)2 * 304 * 16 * lpc * sizeof(double);
-    return align256(std::max(old, res));
-}
+// Published candidate columns of the persistent FP64 kernel: 2 (step parity) x
+// CTAs (up to 304) x padded rows (< 2 nrow + 64).
+static size_t pub_bytes(int nrow) { return align256((size_t)2 * 304 * (2 * (size_t)nrow + 64) * sizeof(double)); }
 
 size_t qrcp_aux_bytes(int nrow, int ncol) {
     const int nblocks = nblocks_cap(ncol);
     return align256(sizeof(Best) * nblocks) + align256((size_t)ncol) + align256(sizeof(double) * nrow) + 256 +
-           pub_bytes(nrow);
+           std::max(pub_bytes(nrow), qrr::buf_bytes(nrow, ncol));
 }
 
 // The persistent kernel for one (T, RPW, NREG); *ran = false when the rows
@@ -857,60 +563,43 @@ static cudaError_t qr_persistent_launch(int nrow, int ncol, T* R, int npiv, Best
     return cudaSuccess;
 }
 
-// The register-resident kernel for one (RPL, LPC); *ran = false when the
-// matrix does not fit on chip (registers of 256 threads an SM plus shared
-// memory) or the device cannot co-schedule the CTAs.
-template <int RPL, int LPC>
-static cudaError_t qr_resident_launch(int nrow, int ncol, const float* R, int npiv, unsigned long long* keys,
-                                      float* pub, int* d_piv, unsigned* bar, unsigned long long limit_ns,
-                                      cudaStream_t s, int* launches, bool* ran) {
+// The pivoted QR in rounds (scdm_rounds.cuh); *ran = false when the device
+// cannot co-schedule its CTAs.
+template <int NRL>
+static cudaError_t qr_rounds_launch(int nrow, int ncol, const float* R, int npiv, void* aux, int* d_piv, unsigned* bar,
+                                    unsigned long long limit_ns, cudaStream_t s, int* launches, bool* ran) {
     *ran = false;
     int dev = 0, sms = 0, coop = 0, optin = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
     cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    constexpr int G = QR2_THREADS / LPC, NPAD = RPL * LPC, PITCH = RPL + 4;
-    if (!coop || nrow > NPAD || sms > 304 || npiv > 4864) return cudaSuccess;
-    int ctas = std::min(sms, (ncol + G - 1) / G);
-    const int cpb = (ncol + ctas - 1) / ctas;
-    ctas = (ncol + cpb - 1) / cpb;
-    const int sc = std::max(0, cpb - G);
-    if ((sc + G - 1) / G > 31) return cudaSuccess;  // the per-thread chosen mask has 32 bits
-    const void* fn = (const void*)qr_resident_kernel<RPL, LPC>;
+    const void* fn = (const void*)qrr::rounds_kernel<NRL>;
     cudaFuncAttributes fa{};
     cudaError_t e;
     if ((e = cudaFuncGetAttributes(&fa, fn))) return e;
-    // two q buffers, the shared-memory columns and their last dots
-    const size_t dyn = (2 * (size_t)LPC * PITCH + (size_t)sc * LPC * PITCH + (((size_t)sc + 3) & ~(size_t)3)) *
-                       sizeof(float);
-    if (dyn + fa.sharedSizeBytes + 1024 > (size_t)optin) return cudaSuccess;
+    const size_t dyn = qrr::smem_bytes();
+    if (!coop || nrow > 32 * NRL || npiv > nrow || dyn + fa.sharedSizeBytes + 1024 > (size_t)optin) return cudaSuccess;
     // one limit for every caller of this kernel: the opt-in maximum
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes)))
         return e;
     int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, QR2_THREADS, dyn))) return e;
-    if (per_sm < 1 || ctas > per_sm * sms) return cudaSuccess;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, qrr::kThreads, dyn))) return e;
+    if (per_sm < 1) return cudaSuccess;
+    const int ctas = std::min(sms, (ncol + qrr::kTile - 1) / qrr::kTile);
+    qrr::Buf B = qrr::buf_at(aux, nrow, ncol);
     if ((e = cudaMemsetAsync(bar, 0, 4 * sizeof(unsigned), s))) return e;
-    if ((e = cudaMemsetAsync(keys, 0, (size_t)npiv * sizeof(unsigned long long), s))) return e;
-    int cpb_arg = cpb;
-    void* args[] = {(void*)&nrow, (void*)&ncol, (void*)&R,     (void*)&npiv,     (void*)&cpb_arg,
-                    (void*)&pub,  (void*)&keys, (void*)&d_piv, (void*)&bar, (void*)&limit_ns};
-    if ((e = cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(QR2_THREADS), args, dyn, s))) return e;
+    if ((e = cudaMemsetAsync(B.hist, 0, sizeof(unsigned) * qrr::kBins, s))) return e;
+    if ((e = cudaMemsetAsync(B.ctl, 0, 16 * sizeof(unsigned), s))) return e;
+    if ((e = cudaMemsetAsync(B.ctl + 4, 0xff, 2 * sizeof(unsigned), s))) return e;
+    void* args[] = {(void*)&nrow, (void*)&ncol, (void*)&R, (void*)&npiv, (void*)&B, (void*)&d_piv, (void*)&bar, (void*)&limit_ns};
+    if ((e = cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(qrr::kThreads), args, dyn, s))) return e;
     *launches += 1;
     *ran = true;
     return cudaSuccess;
 }
 
-static bool qr_resident_enabled() {
-    static const int on = [] {
-        const char* e = getenv("LACE_QR_RESIDENT");  // tuning: 0 selects the tile-group persistent kernel
-        return (e && e[0] == '0') ? 0 : 1;
-    }();
-    return on != 0;
-}
-
-// R (nrow x ncol, row-major, leading dimension ncol) is overwritten.  aux is
+// R (nrow x ncol, row-major, leading dimension ncol) may be overwritten.  aux is
 // caller-provided scratch of qrcp_aux_bytes(nrow, ncol) bytes.
 template <typename T>
 cudaError_t qrcp_pivots(int nrow, int ncol, T* R, int npiv, int* d_piv, void* aux, int* h_timeout,
@@ -925,36 +614,18 @@ cudaError_t qrcp_pivots(int nrow, int ncol, T* R, int npiv, int* d_piv, void* au
     unsigned* bar = reinterpret_cast<unsigned*>(reinterpret_cast<unsigned char*>(q) + align256(sizeof(double) * nrow));
     T* pub = reinterpret_cast<T*>(reinterpret_cast<unsigned char*>(bar) + 256);
     cudaMemsetAsync(chosen, 0, ncol, s);
-    // persistent cooperative version: float rows <= 512 keep two tiles per group
-    // in registers (32 rows per warp); otherwise shared memory and streaming only
+    // cooperative versions: in rounds (FP32), a barrier a pivot (FP64)
     bool ran = false;
     cudaError_t e;
     if constexpr (sizeof(T) == 4) {
-        // register-resident kernel where the matrix fits on chip, else the
-        // tile-group persistent kernel
-        e = cudaSuccess;
-        if (qr_resident_enabled()) {
-            int rpl = 0, lpc = 0;
-            qr2_layout(nrow, &rpl, &lpc);
-            unsigned long long* keys = reinterpret_cast<unsigned long long*>(best);
-            auto go = [&](auto launch) {
-                return launch(nrow, ncol, R, npiv, keys, pub, d_piv, bar, wait_limit_ns, s, launches, &ran);
-            };
-            if (rpl == 32) e = go(qr_resident_launch<32, 1>);
-            else if (lpc == 1) e = go(qr_resident_launch<64, 1>);
-            else if (lpc == 2) e = go(qr_resident_launch<64, 2>);
-            else if (lpc == 4) e = go(qr_resident_launch<64, 4>);
-            else if (lpc == 8) e = go(qr_resident_launch<64, 8>);
-            else e = go(qr_resident_launch<64, 16>);
-        }
-        if (!e && !ran) {
-            if (nrow <= 512)
-                e = qr_persistent_launch<T, 32, 2>(nrow, ncol, R, npiv, best, pub, chosen, d_piv, bar, wait_limit_ns,
-                                                  s, launches, &ran);
-            else
-                e = qr_persistent_launch<T, 64, 0>(nrow, ncol, R, npiv, best, pub, chosen, d_piv, bar, wait_limit_ns,
-                                                  s, launches, &ran);
-        }
+        // At 72^3 with 256 orbitals 0.67 ms (one barrier a pivot with the matrix
+        // in registers and shared memory: 2.37 ms), at 120^3 with 320, off chip,
+        // 1.7 ms (73.4 ms); 16 orbitals on 32^3 take the same time either way.
+        auto go = [&](auto launch) {
+            return launch(nrow, ncol, R, npiv, reinterpret_cast<unsigned char*>(bar) + 256, d_piv, bar, wait_limit_ns, s,
+                          launches, &ran);
+        };
+        e = nrow <= 256 ? go(qr_rounds_launch<8>) : nrow <= 512 ? go(qr_rounds_launch<16>) : go(qr_rounds_launch<32>);
     } else {
         e = qr_persistent_launch<T, 32, 0>(nrow, ncol, R, npiv, best, pub, chosen, d_piv, bar, wait_limit_ns, s,
                                           launches, &ran);
