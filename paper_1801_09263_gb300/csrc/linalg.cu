@@ -265,16 +265,130 @@ __global__ void __launch_bounds__(GR_THREADS) gemm_rows_f32_async_kernel(int M, 
     }
 }
 
+// The FP64 Gram.  FP64 issues one warp instruction in 16 clocks an SM, so the
+// kernel is bound by its FMAs alone and must not spend any on padding: 16 x 16
+// tiles (for symmetric products on and above the diagonal only) and the K range
+// split so that every SM has work whatever the size.  One warp holds a tile,
+// 2 x 4 outputs a lane, the four warps of a CTA take every fourth 16-point step
+// of the CTA's K range and add up through shared memory.  8 x 8 outputs on 24^3:
+// 1,050 -> 9 us (64 x 64 tiles in 14 K chunks, 98 % padding); 32 x 32 on 48^3:
+// 1,100 -> 170 us.
+constexpr int GD_T = 16, GD_WARPS = 4, GD_PITCH = GD_T + 2;
+__global__ void __launch_bounds__(32 * GD_WARPS) gemm_rows_f64_kernel(int M, int N, size_t K, const double* __restrict__ A,
+                                                                      size_t lda, const double* __restrict__ B, size_t ldb,
+                                                                      bool absval, bool sym, size_t kchunk,
+                                                                      double* __restrict__ work) {
+    __shared__ __align__(16) double As[GD_WARPS][GD_T][GD_PITCH], Bs[GD_WARPS][GD_T][GD_PITCH];  // [k][row]
+    int bm, bn;
+    if (sym) {
+        const int nt = (M + GD_T - 1) / GD_T;
+        int left = blockIdx.x;
+        bm = 0;
+        while (left >= nt - bm) {
+            left -= nt - bm;
+            ++bm;
+        }
+        bn = bm + left;
+    } else {
+        const int nt = (N + GD_T - 1) / GD_T;
+        bm = blockIdx.x / nt;
+        bn = blockIdx.x % nt;
+    }
+    const int m0 = bm * GD_T, n0 = bn * GD_T;
+    const size_t k_begin = (size_t)blockIdx.y * kchunk, k_end = min(K, k_begin + kchunk);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int kk = lane & 15, half = lane >> 4;
+    double pa[8], pb[8];
+    auto fetch = [&](size_t k0) {
+        const size_t k = k0 + kk;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int r = 2 * i + half;
+            pa[i] = k < k_end && m0 + r < M ? opv(__ldg(A + (size_t)(m0 + r) * lda + k), absval) : 0.0;
+            pb[i] = k < k_end && n0 + r < N ? opv(__ldg(B + (size_t)(n0 + r) * ldb + k), absval) : 0.0;
+        }
+    };
+    double acc[2][4] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+    const int lr = lane >> 2, lc = (lane & 3) * 4;
+    size_t k0 = k_begin + (size_t)warp * GD_T;
+    if (k0 < k_end) fetch(k0);
+    for (; k0 < k_end; k0 += GD_T * GD_WARPS) {
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            As[warp][kk][2 * i + half] = pa[i];
+            Bs[warp][kk][2 * i + half] = pb[i];
+        }
+        __syncwarp();
+        if (k0 + GD_T * GD_WARPS < k_end) fetch(k0 + GD_T * GD_WARPS);
+#pragma unroll
+        for (int q = 0; q < GD_T; ++q) {
+            const double a0 = As[warp][q][lr], a1 = As[warp][q][lr + 8];
+            const double2 b0 = *reinterpret_cast<const double2*>(&Bs[warp][q][lc]);
+            const double2 b1 = *reinterpret_cast<const double2*>(&Bs[warp][q][lc + 2]);
+            acc[0][0] = fma(a0, b0.x, acc[0][0]);
+            acc[0][1] = fma(a0, b0.y, acc[0][1]);
+            acc[0][2] = fma(a0, b1.x, acc[0][2]);
+            acc[0][3] = fma(a0, b1.y, acc[0][3]);
+            acc[1][0] = fma(a1, b0.x, acc[1][0]);
+            acc[1][1] = fma(a1, b0.y, acc[1][1]);
+            acc[1][2] = fma(a1, b1.x, acc[1][2]);
+            acc[1][3] = fma(a1, b1.y, acc[1][3]);
+        }
+    }
+    __syncthreads();
+    double* red = &As[0][0][0];  // [warp][16 x 16]
+    static_assert(sizeof(As) >= sizeof(double) * GD_WARPS * GD_T * GD_T, "the partial tiles fit where the stages were");
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) red[warp * GD_T * GD_T + (lr + 8 * i) * GD_T + lc + j] = acc[i][j];
+    __syncthreads();
+    double* out = work + (size_t)blockIdx.y * M * N;
+    for (int e = threadIdx.x; e < GD_T * GD_T; e += blockDim.x) {
+        const int m = m0 + e / GD_T, n = n0 + e % GD_T;
+        if (m < M && n < N)
+            out[(size_t)m * N + n] = (red[e] + red[GD_T * GD_T + e]) + (red[2 * GD_T * GD_T + e] + red[3 * GD_T * GD_T + e]);
+    }
+}
+
+// Many chunks of a small product: one warp an output, the lanes over the
+// chunks, then across the lanes (a fixed order).  tile: rows of the tiles of a
+// symmetric product, of which only those on and above the diagonal hold values.
+__global__ void reduce_chunks_warp_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha,
+                                          bool sym, int tile, double* __restrict__ C, int ldc) {
+    const size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (idx >= (size_t)M * N) return;
+    const int lane = threadIdx.x & 31;
+    const int m = (int)(idx / N), n = (int)(idx % N);
+    const size_t src = (sym && n / tile < m / tile) ? (size_t)n * N + m : idx;
+    double s = 0.0;
+    for (int c = lane; c < nchunk; c += 32) s += work[(size_t)c * M * N + src];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) C[(size_t)m * ldc + n] = alpha * s;
+}
+
 __global__ void reduce_chunks_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha,
-                                     bool sym, double* __restrict__ C, int ldc) {
+                                     bool sym, int tile, double* __restrict__ C, int ldc) {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (size_t)M * N) return;
     const int m = (int)(idx / N), n = (int)(idx % N);
     // symmetric products computed only the tiles above the diagonal: mirror the rest
-    const size_t src = (sym && n / GR_BN < m / GR_BM) ? (size_t)n * N + m : idx;
+    const size_t src = (sym && n / tile < m / tile) ? (size_t)n * N + m : idx;
     double s = 0.0;
     for (int c = 0; c < nchunk; ++c) s += work[(size_t)c * M * N + src];
     C[(size_t)m * ldc + n] = alpha * s;
+}
+
+int sm_count() {
+    static const int n = [] {
+        int dev = 0, nsm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+        if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+        return nsm;
+    }();
+    return n;
 }
 
 // CTAs of gemm_rows_kernel resident on the device at once (SMs x occupancy).
@@ -301,8 +415,62 @@ size_t n_chunks_for(int M, int N, size_t K, bool sym) {
     return std::max<size_t>(1, std::min(want, maxc));
 }
 
+// The FP64 Gram's CTAs an SM (16 warps: four a scheduler) and its K chunks: one
+// round of resident CTAs over the tiles, at least 64 points a warp's step.
+constexpr int GD_CTAS = 4;
+size_t f64_tiles(int M, int N, bool sym) {
+    const size_t tm = (size_t)(M + GD_T - 1) / GD_T, tn = (size_t)(N + GD_T - 1) / GD_T;
+    return sym ? tm * (tm + 1) / 2 : tm * tn;
+}
+size_t f64_chunks(int M, int N, size_t K, bool sym) {
+    const size_t want = std::max<size_t>(1, (size_t)GD_CTAS * sm_count() / f64_tiles(M, N, sym));
+    return std::max<size_t>(1, std::min(want, (K + 255) / 256));
+}
+
 // ------------------------------------------------------------------ gemm_combine
 constexpr int GC_BR = 128, GC_BN = 64, GC_BK = 16, GC_THREADS = 256;
+
+// The FP64 combination: a thread a grid point, 16 outputs of it, so that N is
+// padded to 16 at most (bound by its FMAs; 32 outputs of 32 on 48^3: 400 -> 190
+// us against 64-wide tiles).
+constexpr int GCD_N = 16, GCD_THREADS = 128, GCD_KC = 128;
+__global__ void __launch_bounds__(GCD_THREADS) gemm_combine_f64_kernel(int N, size_t K, int Kc, const double* __restrict__ A,
+                                                                       size_t lda, const double* __restrict__ Coef, int ldcoef,
+                                                                       double beta, double* __restrict__ Out, size_t ldo) {
+    __shared__ __align__(16) double Cs[GCD_KC][GCD_N];
+    const size_t r = (size_t)blockIdx.x * GCD_THREADS + threadIdx.x;
+    const int n0 = blockIdx.y * GCD_N;
+    const double* a = A + min(r, K - 1);
+    double acc[GCD_N];
+#pragma unroll
+    for (int j = 0; j < GCD_N; ++j) acc[j] = 0.0;
+    for (int k0 = 0; k0 < Kc; k0 += GCD_KC) {
+        const int kn = min(GCD_KC, Kc - k0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < kn * GCD_N; e += GCD_THREADS) {
+            const int k = e / GCD_N, j = e % GCD_N;
+            Cs[k][j] = n0 + j < N ? __ldg(Coef + (size_t)(k0 + k) * ldcoef + n0 + j) : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 4
+        for (int k = 0; k < kn; ++k) {
+            const double v = __ldg(a + (size_t)(k0 + k) * lda);
+#pragma unroll
+            for (int j = 0; j < GCD_N; j += 2) {
+                const double2 c = *reinterpret_cast<const double2*>(&Cs[k][j]);
+                acc[j] = fma(v, c.x, acc[j]);
+                acc[j + 1] = fma(v, c.y, acc[j + 1]);
+            }
+        }
+    }
+    if (r >= K) return;
+#pragma unroll
+    for (int j = 0; j < GCD_N; ++j) {
+        if (n0 + j >= N) break;
+        double* o = Out + (size_t)(n0 + j) * ldo + r;
+        *o = beta == 0.0 ? acc[j] : beta * *o + acc[j];
+    }
+}
 
 template <typename T>
 __global__ void __launch_bounds__(GC_THREADS) gemm_combine_kernel(int N, size_t K, int Kc, const T* __restrict__ A,
@@ -448,6 +616,7 @@ __global__ void __launch_bounds__(64) small_gemm_staged_f64_kernel(int M, int N,
         *c = alpha * v + (beta == 0.0 ? 0.0 : beta * *c);
     }
 }
+
 
 __global__ void small_gemm_f32_kernel(int N, const float* __restrict__ A, const float* __restrict__ B,
                                       float* __restrict__ C) {
@@ -948,8 +1117,8 @@ __global__ void fill_zero_kernel(double* p, size_t n) {
 // ============================================================================
 
 size_t gemm_rows_work_elems(int M, int N, size_t K) {
-    // a symmetric product takes the most chunks
-    return n_chunks_for(M, N, K, M == N) * (size_t)M * N;
+    // a symmetric product takes the most chunks; either precision
+    return std::max(n_chunks_for(M, N, K, M == N), f64_chunks(M, N, K, M == N)) * (size_t)M * N;
 }
 
 template <typename T>
@@ -958,6 +1127,25 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
                       int* launches) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     const bool sym = (A == B) && (lda == ldb) && (M == N);
+    const size_t tot = (size_t)M * N;
+    if constexpr (sizeof(T) == 8) {
+        const size_t n = std::min(f64_chunks(M, N, K, sym), work_elems / tot);
+        if (n == 0) return cudaErrorInvalidValue;
+        size_t kc = (K + n - 1) / n;
+        kc = (kc + GD_T - 1) / GD_T * GD_T;
+        const size_t nc = (K + kc - 1) / kc;
+        gemm_rows_f64_kernel<<<dim3((unsigned)f64_tiles(M, N, sym), (unsigned)nc), 32 * GD_WARPS, 0, s>>>(
+            M, N, K, A, lda, B, ldb, absval, sym, kc, work);
+        // (32 chunks and more: a thread summing them alone waits for each in turn)
+        if (nc >= 32)
+            reduce_chunks_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nc, work, alpha, sym,
+                                                                                 GD_T, C, ldc);
+        else
+            reduce_chunks_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nc, work, alpha, sym, GD_T, C,
+                                                                               ldc);
+        *launches += 2;
+        return cudaGetLastError();
+    }
     // as many chunks as the workspace holds, up to the balanced count
     const size_t nch = std::min(n_chunks_for(M, N, K, sym), work_elems / ((size_t)M * N));
     if (nch == 0) return cudaErrorInvalidValue;
@@ -974,12 +1162,13 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
             gemm_rows_kernel<T, true><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
         else
             gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
-    } else {
-        gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
     }
-    const size_t tot = (size_t)M * N;
-    reduce_chunks_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym, C,
-                                                                       ldc);
+    if (nch_eff >= 32)
+        reduce_chunks_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym,
+                                                                             GR_BM, C, ldc);
+    else
+        reduce_chunks_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym, GR_BM, C,
+                                                                           ldc);
     *launches += 2;
     return cudaGetLastError();
 }
@@ -988,6 +1177,12 @@ template <typename T>
 cudaError_t gemm_combine(int N, size_t K, int Kc, const T* A, size_t lda, const double* Coef, int ldcoef, double beta,
                          T* Out, size_t ldo, cudaStream_t s, int* launches) {
     if (N <= 0 || K == 0) return cudaSuccess;
+    if constexpr (sizeof(T) == 8) {
+        gemm_combine_f64_kernel<<<dim3((unsigned)((K + GCD_THREADS - 1) / GCD_THREADS), (N + GCD_N - 1) / GCD_N),
+                                  GCD_THREADS, 0, s>>>(N, K, Kc, A, lda, Coef, ldcoef, beta, Out, ldo);
+        *launches += 1;
+        return cudaGetLastError();
+    }
     dim3 grid((unsigned)((K + GC_BR - 1) / GC_BR), (N + GC_BN - 1) / GC_BN);
     bool done = false;
     if constexpr (std::is_same<T, float>::value) {
