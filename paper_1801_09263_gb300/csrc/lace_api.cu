@@ -183,7 +183,7 @@ lace_status lowdin_coeffs(lace_ctx* c, const T* src, int n, double* X, Launch& L
        "loewdin overlap");
     int ok = 0;
     if (c->prec == LACE_FP64) {
-        CK(inv_sqrt_spd(n, S, X, c->m(MS_NSWORK), c->flag.as<int>(), &ok, c->stream, &L.n), "loewdin inverse sqrt");
+        CK(inv_sqrt_spd(n, S, X, c->m(MS_NSWORK), &ok, c->stream, &L.n), "loewdin inverse sqrt");
     } else {
         // FP32 Newton-Schulz, then one FP64 first-order Loewdin step on X^T S X
         CK(inv_sqrt_spd_mixed(n, S, X, c->m(MS_NSWORK), &ok, c->stream, &L.n), "loewdin inverse sqrt");
@@ -372,7 +372,7 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
     CK(small_gemm_f64(n, n, n, phic, n, false, phic, n, true, 1.0, 0.0, B, n, c->stream, &L.n), "scdm B");
     int ok = 0;
     if (c->prec == LACE_FP64) {
-        CK(inv_sqrt_spd(n, B, Bmh, c->m(MS_NSWORK), c->flag.as<int>(), &ok, c->stream, &L.n), "scdm inverse sqrt");
+        CK(inv_sqrt_spd(n, B, Bmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "scdm inverse sqrt");
     } else {
         CK(inv_sqrt_spd_mixed(n, B, Bmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "scdm inverse sqrt");
     }
@@ -412,7 +412,7 @@ lace_status align_impl(lace_ctx* c) {
        "alignment overlap");
     CK(small_gemm_f64(n, n, n, Om, n, true, Om, n, false, 1.0, 0.0, P, n, c->stream, &L.n), "alignment");
     int ok = 0;
-    CK(inv_sqrt_spd(n, P, Pmh, c->m(MS_NSWORK), c->flag.as<int>(), &ok, c->stream, &L.n), "alignment");
+    CK(inv_sqrt_spd(n, P, Pmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "alignment");
     if (!ok) return fail(c, LACE_ERR_NOT_PD, "the orbitals are nearly orthogonal to the previous ones (no alignment)");
     CK(small_gemm_f64(n, n, n, Om, n, false, Pmh, n, false, 1.0, 0.0, Q, n, c->stream, &L.n), "alignment");
     // the SCDM rotation now includes Q

@@ -617,213 +617,10 @@ __global__ void __launch_bounds__(64) small_gemm_staged_f64_kernel(int M, int N,
     }
 }
 
-
-__global__ void small_gemm_f32_kernel(int N, const float* __restrict__ A, const float* __restrict__ B,
-                                      float* __restrict__ C) {
-    // C = A B for N x N row-major; 16 x 16 tiles, one output per thread
-    __shared__ float As[SG][SG + 1];
-    __shared__ float Bs[SG][SG + 1];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int m = blockIdx.y * SG + ty, n = blockIdx.x * SG + tx;
-    float acc = 0.f;
-    for (int k0 = 0; k0 < N; k0 += SG) {
-        As[ty][tx] = (m < N && k0 + tx < N) ? A[(size_t)m * N + k0 + tx] : 0.f;
-        Bs[ty][tx] = (n < N && k0 + ty < N) ? B[(size_t)(k0 + ty) * N + n] : 0.f;
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < SG; ++kk) acc = fmaf(As[ty][kk], Bs[kk][tx], acc);
-        __syncthreads();
-    }
-    if (m < N && n < N) C[(size_t)m * N + n] = acc;
-}
-
-// C = A B for N x N row-major, N <= 376: the block's 16 rows of A and 16
-// columns of B (transposed, so both are read along k) are staged in shared
-// memory with all loads in flight at once (the products are latency-bound at
-// N ~ 256), then one output per thread over the full K = N from 16-byte reads
-// (two shared-memory loads per four FMAs) into four partial sums.
-__host__ __device__ inline int sg_pitch(int N) { return ((N + 3) & ~3) + 4; }
-__global__ void small_gemm_f32_staged_kernel(int N, const float* __restrict__ A0, const float* __restrict__ B0,
-                                             float* __restrict__ C0, const float* __restrict__ A1,
-                                             const float* __restrict__ B1, float* __restrict__ C1) {
-    // blockIdx.z selects one of two independent products (C0 = A0 B0, C1 = A1 B1)
-    const float* __restrict__ A = blockIdx.z ? A1 : A0;
-    const float* __restrict__ B = blockIdx.z ? B1 : B0;
-    float* __restrict__ C = blockIdx.z ? C1 : C0;
-    extern __shared__ __align__(16) float sg_smem[];
-    const int lp = sg_pitch(N);       // 16-byte aligned rows, the pitch offsetting rows by 4 banks
-    float* As = sg_smem;              // [SG][lp]: A[m0 + r][k]
-    float* Bs = sg_smem + SG * lp;    // [SG][lp]: B[k][n0 + c]
-    const int tx = threadIdx.x, ty = threadIdx.y, t = ty * SG + tx;
-    const int m0 = blockIdx.y * SG, n0 = blockIdx.x * SG;
-    const int kpad = (N + 3) & ~3;
-    for (int q = t; q < SG * kpad; q += SG * SG) {
-        const int r = q / kpad, k = q % kpad;
-        As[r * lp + k] = (m0 + r < N && k < N) ? __ldg(A + (size_t)(m0 + r) * N + k) : 0.f;
-    }
-    for (int q = t; q < SG * kpad; q += SG * SG) {
-        const int k = q / SG, c = q % SG;
-        Bs[c * lp + k] = (n0 + c < N && k < N) ? __ldg(B + (size_t)k * N + n0 + c) : 0.f;
-    }
-    __syncthreads();
-    const int m = m0 + ty, n = n0 + tx;
-    const float* ar = As + ty * lp;
-    const float* br = Bs + tx * lp;
-    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-    for (int k = 0; k < kpad; k += 4) {
-        const float4 x = *reinterpret_cast<const float4*>(ar + k);
-        const float4 y = *reinterpret_cast<const float4*>(br + k);
-        a0 = fmaf(x.x, y.x, a0);
-        a1 = fmaf(x.y, y.y, a1);
-        a2 = fmaf(x.z, y.z, a2);
-        a3 = fmaf(x.w, y.w, a3);
-    }
-    if (m < N && n < N) C[(size_t)m * N + n] = (a0 + a1) + (a2 + a3);
-}
-
-void sgemm_f32_square(int N, const float* A, const float* B, float* C, cudaStream_t s) {
-    const dim3 gg((N + SG - 1) / SG, (N + SG - 1) / SG), bb(SG, SG);
-    const size_t smem = (size_t)2 * SG * sg_pitch(N) * sizeof(float);  // <= 48 KB for N <= 376
-    if (N <= 376) small_gemm_f32_staged_kernel<<<gg, bb, smem, s>>>(N, A, B, C, A, B, C);
-    else small_gemm_f32_kernel<<<gg, bb, 0, s>>>(N, A, B, C);
-}
-
-// C0 = A0 B0 and C1 = A1 B1 (independent N x N products) in one launch.
-void sgemm_f32_square_pair(int N, const float* A0, const float* B0, float* C0, const float* A1, const float* B1,
-                           float* C1, cudaStream_t s) {
-    if (N <= 376) {
-        const dim3 gg((N + SG - 1) / SG, (N + SG - 1) / SG, 2), bb(SG, SG);
-        const size_t smem = (size_t)2 * SG * sg_pitch(N) * sizeof(float);
-        small_gemm_f32_staged_kernel<<<gg, bb, smem, s>>>(N, A0, B0, C0, A1, B1, C1);
-    } else {
-        sgemm_f32_square(N, A0, B0, C0, s);
-        sgemm_f32_square(N, A1, B1, C1, s);
-    }
-}
-
-// T = (3 I - P) / 2 in place (FP32)
-__global__ void ns_t_f32_kernel(int N, float* P) {
+// y = b y + x
+__global__ void axpby_kernel(int n, const double* x, double b, double* y) {
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * N) return;
-    const float d = (idx / N == idx % N) ? 3.f : 0.f;
-    P[idx] = 0.5f * (d - P[idx]);
-}
-
-// out[0] = || I - A ||_F^2 (FP32 input, FP64 sum, fixed order)
-__global__ void scale_to_f32_kernel(int n, const double* in, float* out, double s) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < n) out[idx] = (float)(s * in[idx]);
-}
-
-__global__ void identity_f32_kernel(int N, float* X) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < N * N) X[idx] = (idx / N == idx % N) ? 1.f : 0.f;
-}
-
-// X = s * (Z + Z^T)/2 in FP64 from FP32 Z
-__global__ void sym_from_f32_kernel(int N, const float* Z, double* X, double s) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * N) return;
-    const int i = idx / N, j = idx % N;
-    X[idx] = s * 0.5 * ((double)Z[(size_t)i * N + j] + (double)Z[(size_t)j * N + i]);
-}
-
-// E := E - I (in place)
-__global__ void sub_identity_kernel(int N, double* E) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < N * N && idx / N == idx % N) E[idx] -= 1.0;
-}
-
-__global__ void axpy_kernel(int n, const double* x, double* y) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < n) y[idx] += x[idx];
-}
-
-__global__ void set_identity_kernel(int N, double* X, double scale) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * N) return;
-    X[idx] = (idx / N == idx % N) ? scale : 0.0;
-}
-
-__global__ void scale_copy_kernel(int n, const double* in, double* out, double s) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < n) out[idx] = s * in[idx];
-}
-
-// T = (3 I - P) / 2 in place on P
-__global__ void ns_t_kernel(int N, double* P) {
-    const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= N * N) return;
-    const double d = (idx / N == idx % N) ? 3.0 : 0.0;
-    P[idx] = 0.5 * (d - P[idx]);
-}
-
-// Frobenius norm squared (single block, fixed order) into out[0]; mode 1: of (I - A).
-// ||A||_F^2 (mode 0) or ||I - A||_F^2 (mode 1) of an N x N matrix: one block
-// per row (FP64 sums), then a fixed-order sum of the rows (deterministic).
-// part holds N doubles past out.
-template <typename TA>
-__global__ void frob_rows_kernel(int N, const TA* __restrict__ A, int mode, double* __restrict__ part) {
-    __shared__ double sh[32];
-    const int r = blockIdx.x;
-    double s = 0.0;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-        double v = (double)A[(size_t)r * N + c];
-        if (mode == 1) v = (r == c ? 1.0 : 0.0) - v;
-        s += mode == 2 ? fabs(v) : v * v;
-    }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-        part[r] = t;
-    }
-}
-
-__global__ void sum_rows_kernel(int N, const double* __restrict__ part, double* __restrict__ out) {
-    __shared__ double sh[256];
-    double s = 0.0;
-    for (int r = threadIdx.x; r < N; r += blockDim.x) s += part[r];
-    sh[threadIdx.x] = s;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] += sh[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[0] = sh[0];
-}
-
-__global__ void max_rows_kernel(int N, const double* __restrict__ part, double* __restrict__ out) {
-    __shared__ double sh[256];
-    double m = 0.0;
-    for (int r = threadIdx.x; r < N; r += blockDim.x) m = fmax(m, part[r]);
-    sh[threadIdx.x] = m;
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) sh[threadIdx.x] = fmax(sh[threadIdx.x], sh[threadIdx.x + o]);
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) out[0] = sh[0];
-}
-
-// scal[0] = ||A||_inf = max_i sum_j |a_ij|, an upper bound of the largest
-// eigenvalue of a symmetric A (Gershgorin) and usually far tighter than the
-// Frobenius norm: the Newton-Schulz iterations start with A's spectrum
-// scaled into (0, 1] close to 1 and need fewer steps.
-void norm_inf(int N, const double* A, double* scal, cudaStream_t s, int* launches) {
-    frob_rows_kernel<double><<<N, 128, 0, s>>>(N, A, 2, scal + 8);
-    max_rows_kernel<<<1, 256, 0, s>>>(N, scal + 8, scal);
-    *launches += 2;
-}
-
-template <typename TA>
-void frob(int N, const TA* A, int mode, double* scal, cudaStream_t s, int* launches) {
-    frob_rows_kernel<TA><<<N, 128, 0, s>>>(N, A, mode, scal + 8);
-    sum_rows_kernel<<<1, 256, 0, s>>>(N, scal + 8, scal);
-    *launches += 2;
+    if (idx < n) y[idx] = fma(b, y[idx], x[idx]);
 }
 
 // ------------------------------------------------------------------ Cholesky
@@ -1214,157 +1011,22 @@ cudaError_t small_gemm_f64(int M, int N, int K, const double* A, int lda, bool t
     return cudaGetLastError();
 }
 
-size_t inv_sqrt_work_elems(int N) { return 4 * (size_t)N * N + 8; }
-
-// Coupled Newton-Schulz iteration (Higham, "Functions of Matrices", Sec. 6.7):
-// Y_0 = A/c, Z_0 = I; T = (3I - Z Y)/2; Y <- Y T; Z <- T Z.  Z -> (A/c)^{-1/2}.
-// c = ||A||_F puts the spectrum of A/c in (0, 1], where the iteration converges.
-cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* d_flag, int* ok, cudaStream_t s,
-                         int* launches) {
-    (void)d_flag;
-    const size_t nn = (size_t)N * N;
-    double* Y = work;
-    double* Z = X;
-    double* T = work + nn;
-    double* Y2 = work + 2 * nn;
-    double* Z2 = work + 3 * nn;
-    double* scal = work + 4 * nn;
-    const int nb = (int)((nn + 255) / 256);
-    double h_norm2 = 0.0;
-    norm_inf(N, A, scal, s, launches);
-    cudaMemcpyAsync(&h_norm2, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e) return e;
-    if (!(h_norm2 > 0.0) || !std::isfinite(h_norm2)) { *ok = 0; return cudaSuccess; }
-    const double c = h_norm2;  // ||A||_inf >= lambda_max
-    scale_copy_kernel<<<nb, 256, 0, s>>>((int)nn, A, Y, 1.0 / c);
-    set_identity_kernel<<<nb, 256, 0, s>>>(N, Z, 1.0);
-    *launches += 2;
-    *ok = 0;
-    // Stop when ||I - Z Y||_F^2 is below 1e-24 N, or once it is below 1e-12 N
-    // and no longer falls by 4x between checks (rounding floor reached).
-    double prev = INFINITY;
-    for (int it = 0; it < 160; ++it) {
-        small_gemm_f64(N, N, N, Z, N, false, Y, N, false, 1.0, 0.0, T, N, s, launches);
-        ns_t_kernel<<<nb, 256, 0, s>>>(N, T);
-        small_gemm_f64(N, N, N, Y, N, false, T, N, false, 1.0, 0.0, Y2, N, s, launches);
-        small_gemm_f64(N, N, N, T, N, false, Z, N, false, 1.0, 0.0, Z2, N, s, launches);
-        cudaMemcpyAsync(Y, Y2, nn * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(Z, Z2, nn * sizeof(double), cudaMemcpyDeviceToDevice, s);
-        *launches += 1;
-        if (it >= 5 && (it % 2 == 1)) {
-            small_gemm_f64(N, N, N, Z, N, false, Y, N, false, 1.0, 0.0, T, N, s, launches);
-            frob<double>(N, T, 1, scal, s, launches);
-            cudaMemcpyAsync(&h_norm2, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-            if ((e = cudaStreamSynchronize(s))) return e;
-            if (!std::isfinite(h_norm2)) break;
-            if (h_norm2 < 1e-24 * N || (h_norm2 < 1e-12 * N && h_norm2 > 0.25 * prev)) { *ok = 1; break; }
-            prev = h_norm2;
-        }
-    }
-    if (!*ok) return cudaGetLastError();
-    // Reject ill-conditioned A: ||(A/c)^{-1/2}||_F^2 >= lambda_max/lambda_min.
-    frob<double>(N, Z, 0, scal, s, launches);
-    cudaMemcpyAsync(&h_norm2, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-    if ((e = cudaStreamSynchronize(s))) return e;
-    if (!(h_norm2 < 1e12)) { *ok = 0; return cudaSuccess; }
-    // A^{-1/2} = (A/c)^{-1/2} / sqrt(c)
-    scale_copy_kernel<<<nb, 256, 0, s>>>((int)nn, Z, X, 1.0 / std::sqrt(c));
-    *launches += 1;
-    return cudaGetLastError();
-}
-
-size_t inv_sqrt_mixed_work_elems(int N) { return 4 * (size_t)N * N + 8; }
-
-// FP32 coupled Newton-Schulz to ~1e-7 (same iteration as inv_sqrt_spd), then
-// X0 = sym(Z)/sqrt(c) in FP64.  X0 A X0 = I + O(1e-7); callers restore exact
-// orthonormality with one FP64 first-order Loewdin step (lowdin_refine).
-cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s,
-                               int* launches) {
-    const size_t nn = (size_t)N * N;
-    float* Y = reinterpret_cast<float*>(work);
-    float* Z = Y + nn;
-    float* T = Z + nn;
-    float* Y2 = T + nn;
-    float* Z2 = Y2 + nn;
-    double* scal = work + 3 * nn;  // past the five FP32 matrices (2.5 nn doubles)
-    const int nb = (int)((nn + 255) / 256);
-    double h = 0.0;
-    norm_inf(N, A, scal, s, launches);
-    cudaMemcpyAsync(&h, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
-    if (e) return e;
-    *ok = 0;
-    if (!(h > 0.0) || !std::isfinite(h)) return cudaSuccess;
-    const double c = h;  // ||A||_inf >= lambda_max
-    scale_to_f32_kernel<<<nb, 256, 0, s>>>((int)nn, A, Y, 1.0 / c);
-    identity_f32_kernel<<<nb, 256, 0, s>>>(N, Z);
-    *launches += 2;
-    // h = ||I - Z Y||_F^2 = sum_k (1 - x_k)^2 over the eigenvalues x_k of Z Y.
-    // Once h < 1e-6 N every |1 - x_k| < 0.016 and the iteration is in its
-    // quadratic regime (1 - x -> ~(3/4)(1 - x)^2): two more steps reach the
-    // FP32 rounding floor without another host-checked product.
-    // The check after every second step from the fourth on reads h from the
-    // next step's own first product P = Z Y, so it costs no product of its own.
-    double prev = INFINITY;
-    int extra = -1;
-    for (int it = 0; it < 160; ++it) {
-        sgemm_f32_square(N, Z, Y, T, s);  // P = Z Y of the current iterates
-        *launches += 1;
-        if (extra < 0 && it >= 4 && (it % 2 == 0)) {
-            frob<float>(N, T, 1, scal, s, launches);
-            cudaMemcpyAsync(&h, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-            if ((e = cudaStreamSynchronize(s))) return e;
-            if (!std::isfinite(h)) break;
-            if (h < 1e-11 * N || (h < 1e-6 * N && h > 0.25 * prev)) { *ok = 1; break; }
-            if (h < 1e-6 * N) extra = 2;
-            prev = h;
-        }
-        ns_t_f32_kernel<<<nb, 256, 0, s>>>(N, T);
-        sgemm_f32_square_pair(N, Y, T, Y2, T, Z, Z2, s);
-        std::swap(Y, Y2);
-        std::swap(Z, Z2);
-        *launches += 2;
-        if (extra > 0 && --extra == 0) {
-            *ok = 1;
-            break;
-        }
-    }
-    if (!*ok) return cudaGetLastError();
-    // ||(A/c)^{-1/2}||_F^2 >= lambda_max / lambda_min: reject ill-conditioned A
-    sym_from_f32_kernel<<<nb, 256, 0, s>>>(N, Z, X, 1.0);
-    frob<double>(N, X, 0, scal, s, launches);
-    cudaMemcpyAsync(&h, scal, sizeof(double), cudaMemcpyDeviceToHost, s);
-    *launches += 1;
-    if ((e = cudaStreamSynchronize(s))) return e;
-    if (!(h < 1e12)) { *ok = 0; return cudaSuccess; }
-    scale_copy_kernel<<<nb, 256, 0, s>>>((int)nn, X, X, 1.0 / std::sqrt(c));
-    *launches += 1;
-    return cudaGetLastError();
-}
-
-// First-order Loewdin correction making F^T G F = I to second order:
-// E = F^T G F - I (G = identity when G == nullptr), F <- F (I - E/2).
-// F is N x N FP64 (in place); work holds 3 N x N.
+// First-order Loewdin correction making F^T G F = I to second order (G =
+// identity when G == nullptr): F <- F (3 I - F^T G F) / 2.  F is N x N FP64 (in
+// place); work holds 3 N x N.
 cudaError_t lowdin_refine(int N, double* F, const double* G, double* work, cudaStream_t s, int* launches) {
     const size_t nn = (size_t)N * N;
     double* GF = work;
     double* E = work + nn;
     double* F2 = work + 2 * nn;
-    const int nb = (int)((nn + 255) / 256);
     const double* rhs = F;
     if (G) {
         small_gemm_f64(N, N, N, G, N, false, F, N, false, 1.0, 0.0, GF, N, s, launches);
         rhs = GF;
     }
-    small_gemm_f64(N, N, N, F, N, true, rhs, N, false, 1.0, 0.0, E, N, s, launches);
-    sub_identity_kernel<<<nb, 256, 0, s>>>(N, E);
-    *launches += 1;
-    small_gemm_f64(N, N, N, F, N, false, E, N, false, -0.5, 0.0, F2, N, s, launches);
-    // F += F2
-    cudaError_t e = cudaGetLastError();
-    if (e) return e;
-    axpy_kernel<<<nb, 256, 0, s>>>((int)nn, F2, F);
+    small_gemm_f64(N, N, N, F, N, true, rhs, N, false, -0.5, 0.0, E, N, s, launches);
+    small_gemm_f64(N, N, N, F, N, false, E, N, false, 1.0, 0.0, F2, N, s, launches);
+    axpby_kernel<<<(int)((nn + 255) / 256), 256, 0, s>>>((int)nn, F2, 1.5, F);
     *launches += 1;
     return cudaGetLastError();
 }
