@@ -639,6 +639,23 @@ __global__ void tc_reduce_kernel(int M, int N, int nchunk, const double* __restr
     C[(size_t)m * ldc + n] = alpha * s;
 }
 
+// The same for small products of many chunks: one warp an output, the lanes
+// over the chunks, then across the lanes (a thread alone would wait for one
+// chunk after the other).
+__global__ void tc_reduce_warp_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha, bool sym,
+                                      double* __restrict__ C, int ldc) {
+    const size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (idx >= (size_t)M * N) return;
+    const int lane = threadIdx.x & 31;
+    const int m = (int)(idx / N), n = (int)(idx % N);
+    const size_t src = (sym && n / TC_N < m / TC_M) ? (size_t)n * N + m : idx;
+    double s = 0.0;
+    for (int c = lane; c < nchunk; c += 32) s += work[(size_t)c * M * N + src];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) C[(size_t)m * ldc + n] = alpha * s;
+}
+
 // ---------------------------------------------------------------------------
 // Combination over orbitals: Out[n][r] = beta Out[n][r] + sum_k Coef[k][n] A[k][r]
 // (xi = W L^{-T}; K_ACE psi = -xi X).  As an MMA: D[r][n] = sum_k A^T[r][k]
@@ -1136,11 +1153,15 @@ size_t gram_tiles(int M, int N, bool sym) {
     return sym ? tm * (tm + 1) / 2 : tm * tn;
 }
 // K chunks: as many CTAs as fit one wave of 152 SMs (one CTA per SM), a
-// chunk at least 4096 points long.
+// chunk at least 256 points long.  A CTA's copies, splits and MMAs take ~0.8 us
+// a 32-point step and its set-up and last drain ~4 us, so small grids want many
+// short chunks: 16 orbitals on 32^3 take 98 us in 8 chunks of 4096 points, 15 us
+// in 128 of 256; 64 on 48^3 102 us in 27 of 4096, 29 us in 152.
+constexpr size_t kMinChunk = 256;
 size_t gram_chunks(int M, int N, size_t K, bool sym) {
     const size_t tiles = gram_tiles(M, N, sym);
     const size_t want = std::max<size_t>(1, 152 / tiles);
-    const size_t maxc = (K + 4095) / 4096;
+    const size_t maxc = (K + kMinChunk - 1) / kMinChunk;
     return std::max<size_t>(1, std::min(want, maxc));
 }
 }  // namespace
@@ -1187,7 +1208,11 @@ cudaError_t tc_gram(int M, int N, size_t K, const float* A, size_t lda, const fl
         kern<<<grid, TC_THREADS, TC_SMEM_BYTES, s>>>(M, N, K, A, lda, B, ldb, kchunk, work, d_err);
     }
     const size_t tot = (size_t)M * N;
-    tc_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, mirrored, C, ldc);
+    if (nch_eff >= 16 && tot <= 128 * 128)
+        tc_reduce_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, mirrored,
+                                                                         C, ldc);
+    else
+        tc_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, mirrored, C, ldc);
     *launches += 2;
     if (h_err) {
         cudaMemcpyAsync(h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
