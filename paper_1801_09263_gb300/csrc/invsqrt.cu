@@ -9,11 +9,15 @@
 // kernels between them and the host's waits for the norms were most of the time.
 // Up to 64 rows in FP32 (16 in FP64) one CTA keeps everything in shared memory;
 // beyond, a cooperative grid computes tiles and meets at a barrier after every
-// product.  Every iterate is a polynomial in A and so symmetric: only tiles on
-// and above the diagonal are computed, and both operands are read by rows.
+// product.  The iterates are symmetric but for rounding, and yet all products
+// are computed whole and read as they stand: the iteration damps the errors of
+// Z Y, Y T and T Z alone.  With T mirrored from its upper triangle they grow by
+// sqrt(lambda_max / lambda_min) a step (FP32 X A X - I of 2e-2 instead of 6e-5 at N = 400
+// and 2.5e3); with Y and Z mirrored, or a transpose read in place of either, matrices of
+// 1e7 that converge do not.
 //
-// Measured (FP32, both inverse square roots of a step, launches and waits
-// included): N = 256 650 -> 250 us, N = 64 480 -> 90 us.
+// Measured (FP32, both inverse square roots of a step): kernels 2 x 226 us at
+// N = 256 and 2 x 139 us at N = 64; separate launches with their waits took 650 and 480 us.
 #include <algorithm>
 #include <cmath>
 
@@ -65,48 +69,51 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 }
 
 // ------------------------------------------------------------------ one CTA
-// C = A B of symmetric matrices in shared memory (rows of pitch P, zero past
-// N), NB x NB outputs a thread of 16 x 16; f(m, n, value) for every output
-// with m <= n.
+// NB consecutive values.
+template <typename T, int NB> __device__ __forceinline__ void load_row(const T* p, T* v) {
+    if constexpr (sizeof(T) == 4 && NB == 4) {
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        v[0] = q.x, v[1] = q.y, v[2] = q.z, v[3] = q.w;
+    } else if constexpr (sizeof(T) == 4 && NB == 2) {
+        const float2 q = *reinterpret_cast<const float2*>(p);
+        v[0] = q.x, v[1] = q.y;
+    } else {
+#pragma unroll
+        for (int j = 0; j < NB; ++j) v[j] = p[j];
+    }
+}
+
+// C = A B of matrices in shared memory (rows of pitch P, zero past N), NB x NB
+// outputs a thread of 16 x 16 (rows ty + 16 i, columns NB tx + j); f(m, n, value)
+// for every output.
 template <typename T, int NB, int P, class F>
 __device__ __forceinline__ void one_product(int N, const T* A, const T* B, F f) {
     const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+    constexpr int KV = sizeof(T) == 4 ? 4 : 1;
     T acc[NB][NB];
 #pragma unroll
     for (int i = 0; i < NB; ++i)
 #pragma unroll
         for (int j = 0; j < NB; ++j) acc[i][j] = T(0);
-    if constexpr (sizeof(T) == 4) {
-        for (int k = 0; k < N; k += 4) {
-            float4 a[NB], b[NB];
+    for (int k = 0; k < N; k += KV) {
+        T a[NB][KV], b[KV][NB];
 #pragma unroll
-            for (int i = 0; i < NB; ++i) {
-                a[i] = *reinterpret_cast<const float4*>(A + (ty + 16 * i) * P + k);
-                b[i] = *reinterpret_cast<const float4*>(B + (tx + 16 * i) * P + k);
-            }
+        for (int i = 0; i < NB; ++i) load_row<T, KV>(A + (ty + 16 * i) * P + k, a[i]);
 #pragma unroll
-            for (int i = 0; i < NB; ++i)
+        for (int q = 0; q < KV; ++q) load_row<T, NB>(B + (k + q) * P + NB * tx, b[q]);
 #pragma unroll
-                for (int j = 0; j < NB; ++j) {
-                    acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-                    acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-                }
-        }
-    } else {
-        for (int k = 0; k < N; ++k)
+        for (int q = 0; q < KV; ++q)
 #pragma unroll
             for (int i = 0; i < NB; ++i)
 #pragma unroll
-                for (int j = 0; j < NB; ++j) acc[i][j] = fma(A[(ty + 16 * i) * P + k], B[(tx + 16 * j) * P + k], acc[i][j]);
+                for (int j = 0; j < NB; ++j) acc[i][j] = fma(a[i][q], b[q][j], acc[i][j]);
     }
 #pragma unroll
     for (int i = 0; i < NB; ++i)
 #pragma unroll
         for (int j = 0; j < NB; ++j) {
-            const int m = ty + 16 * i, n = tx + 16 * j;
-            if (m <= n && n < N) f(m, n, acc[i][j]);
+            const int m = ty + 16 * i, n = NB * tx + j;
+            if (m < N && n < N) f(m, n, acc[i][j]);
         }
 }
 
@@ -157,10 +164,8 @@ __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double*
         one_product<T, NB, P>(N, Z, Y, [&](int m, int n, T v) {
             const T d = m == n ? T(1) : T(0);
             const double x = (double)(d - v);
-            h += m == n ? x * x : 2.0 * x * x;
-            const T t = T(0.5) * (T(2) * d + (d - v));  // (3 delta - v) / 2
-            W[m * P + n] = t;
-            W[n * P + m] = t;
+            h += x * x;
+            W[m * P + n] = T(0.5) * (T(2) * d + (d - v));  // (3 delta - v) / 2
         });
         h = block_sum(h, sh);
         const int st = stop.test(h, N);
@@ -169,8 +174,8 @@ __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double*
             break;
         }
         __syncthreads();
-        one_product<T, NB, P>(N, Y, W, [&](int m, int n, T v) { Y2[m * P + n] = v; Y2[n * P + m] = v; });
-        one_product<T, NB, P>(N, W, Z, [&](int m, int n, T v) { Z2[m * P + n] = v; Z2[n * P + m] = v; });
+        one_product<T, NB, P>(N, Y, W, [&](int m, int n, T v) { Y2[m * P + n] = v; });
+        one_product<T, NB, P>(N, W, Z, [&](int m, int n, T v) { Z2[m * P + n] = v; });
         __syncthreads();
         T* t = Y;
         Y = Y2;
@@ -182,13 +187,14 @@ __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double*
     // ||(A/c)^{-1/2}||_F^2 >= lambda_max / lambda_min: reject ill-conditioned A
     double f = 0.0;
     for (int e = tid; e < N * N; e += kNsThreads) {
-        const double z = (double)Z[(e / N) * P + e % N];
+        const double z = 0.5 * ((double)Z[(e / N) * P + e % N] + (double)Z[(e % N) * P + e / N]);
         f += z * z;
     }
     f = block_sum(f, sh);
     if (!ok || !(f < 1e12)) return;
     const double s = 1.0 / sqrt(c);
-    for (int e = tid; e < N * N; e += kNsThreads) X[e] = s * (double)Z[(e / N) * P + e % N];
+    for (int e = tid; e < N * N; e += kNsThreads) 
+        X[e] = s * 0.5 * ((double)Z[(e / N) * P + e % N] + (double)Z[(e % N) * P + e / N]);
     if (tid == 0) *status = 1;
 }
 
@@ -214,15 +220,14 @@ template <typename T> struct NsArgs {
     int* status;               // 1 converged, 0 failed, -1 a barrier wait ran out (preset)
 };
 
-// One tile (bm, bn) of A B (B symmetric, both read by rows); f(m, n, value) for
-// its outputs with m <= n < N, each by one thread.
+// One tile (bm, bn) of A B; f(m, n, value) for its outputs, each by one thread.
 template <typename T, class F>
 __device__ __forceinline__ void grid_product(int N, int ld, const T* A, const T* B, int bm, int bn, T* smem, F f) {
     using C = NsTile<T>;
-    constexpr int S = C::S, P = C::P, E = C::E;
-    T* As = smem;
-    T* Bs = smem + S * P;
-    T* red = smem + 2 * S * P;  // [4][S][S]
+    constexpr int S = C::S, P = C::P, E = C::E, KV = sizeof(T) == 4 ? 4 : 1;
+    T* As = smem;          // [S][P]
+    T* Bs = smem + S * P;  // [KC][S]
+    T* red = Bs + C::KC * S;  // [4][S][S]
     const int tid = threadIdx.x, group = tid >> 6, t = tid & 63, ti = t >> 3, tj = t & 7;
     T acc[E][E];
 #pragma unroll
@@ -230,80 +235,69 @@ __device__ __forceinline__ void grid_product(int N, int ld, const T* A, const T*
 #pragma unroll
         for (int j = 0; j < E; ++j) acc[i][j] = T(0);
     for (int k0 = 0; k0 < N; k0 += C::KC) {
+        const int len = min(C::KC, N - k0), per = ((len + 3) / 4 + 3) / 4 * 4;  // (past len: zeros)
         __syncthreads();
         if constexpr (sizeof(T) == 4) {
-            constexpr int Q = C::KC / 4;
+            constexpr int Q = C::KC / 4, SQ = S / 4;
             const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int e = tid; e < 2 * S * Q; e += kNsThreads) {
-                const int r = e / Q, q = e % Q, row = r < S ? bm * S + r : bn * S + r - S;
-                const T* M = r < S ? A : B;
-                const bool in = row < N && k0 + 4 * q < ld;
-                *reinterpret_cast<float4*>(smem + r * P + 4 * q) =
-                    in ? __ldcg(reinterpret_cast<const float4*>(M + (size_t)row * ld + k0) + q) : z;
+            for (int e = tid; e < S * Q; e += kNsThreads) {
+                const int r = e / Q, q = e % Q, row = bm * S + r;
+                *reinterpret_cast<float4*>(As + r * P + 4 * q) =
+                    row < N && k0 + 4 * q < ld ? __ldcg(reinterpret_cast<const float4*>(A + (size_t)row * ld + k0) + q) : z;
+            }
+            for (int e = tid; e < 4 * per * SQ; e += kNsThreads) {
+                const int k = e / SQ, q = e % SQ, col = bn * S + 4 * q;
+                *reinterpret_cast<float4*>(Bs + k * S + 4 * q) =
+                    k < len && col < ld ? __ldcg(reinterpret_cast<const float4*>(B + (size_t)(k0 + k) * ld + col)) : z;
             }
         } else {
-            for (int e = tid; e < 2 * S * C::KC; e += kNsThreads) {
-                const int r = e / C::KC, q = e % C::KC, row = r < S ? bm * S + r : bn * S + r - S;
-                const T* M = r < S ? A : B;
-                smem[r * P + q] = row < N && k0 + q < N ? __ldcg(M + (size_t)row * ld + k0 + q) : T(0);
+            for (int e = tid; e < S * C::KC; e += kNsThreads) {
+                const int r = e / C::KC, q = e % C::KC, row = bm * S + r;
+                As[r * P + q] = row < N && q < len ? __ldcg(A + (size_t)row * ld + k0 + q) : T(0);
+            }
+            for (int e = tid; e < S * C::KC; e += kNsThreads) {
+                const int k = e / S, col = bn * S + e % S;
+                Bs[e] = k < len && col < N ? __ldcg(B + (size_t)(k0 + k) * ld + col) : T(0);
             }
         }
         __syncthreads();
-        const int len = min(C::KC, N - k0), per = ((len + 3) / 4 + 3) / 4 * 4;  // (past len: zeros)
         const int kb = group * per, ke = min(kb + per, C::KC);
-        if constexpr (sizeof(T) == 4) {
-            for (int k = kb; k < ke; k += 4) {
-                float4 a[E], b[E];
+        for (int k = kb; k < ke; k += KV) {
+            T a[E][KV], b[KV][E];
 #pragma unroll
-                for (int i = 0; i < E; ++i) {
-                    a[i] = *reinterpret_cast<const float4*>(As + (ti + 8 * i) * P + k);
-                    b[i] = *reinterpret_cast<const float4*>(Bs + (tj + 8 * i) * P + k);
-                }
+            for (int i = 0; i < E; ++i) load_row<T, KV>(As + (ti + 8 * i) * P + k, a[i]);
+#pragma unroll
+            for (int q = 0; q < KV; ++q) load_row<T, E>(Bs + (k + q) * S + E * tj, b[q]);
+#pragma unroll
+            for (int q = 0; q < KV; ++q)
 #pragma unroll
                 for (int i = 0; i < E; ++i)
 #pragma unroll
-                    for (int j = 0; j < E; ++j) {
-                        acc[i][j] = fmaf(a[i].x, b[j].x, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].y, b[j].y, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].z, b[j].z, acc[i][j]);
-                        acc[i][j] = fmaf(a[i].w, b[j].w, acc[i][j]);
-                    }
-            }
-        } else {
-            for (int k = kb; k < min(ke, len); ++k) acc[0][0] = fma(As[ti * P + k], Bs[tj * P + k], acc[0][0]);
+                    for (int j = 0; j < E; ++j) acc[i][j] = fma(a[i][q], b[q][j], acc[i][j]);
         }
     }
 #pragma unroll
     for (int i = 0; i < E; ++i)
 #pragma unroll
-        for (int j = 0; j < E; ++j) red[(group * S + ti + 8 * i) * S + tj + 8 * j] = acc[i][j];
+        for (int j = 0; j < E; ++j) red[(group * S + ti + 8 * i) * S + E * tj + j] = acc[i][j];
     __syncthreads();
     if (tid < S * S) {
         const int m = bm * S + tid / S, n = bn * S + tid % S;
         const T v = (red[tid] + red[S * S + tid]) + (red[2 * S * S + tid] + red[3 * S * S + tid]);
-        if (m <= n && n < N) f(m, n, v);
+        if (m < N && n < N) f(m, n, v);
     }
     __syncthreads();
-}
-
-__device__ __forceinline__ void tile_of(int t, int nt, int& bm, int& bn) {
-    bm = 0;
-    while (t >= nt - bm) {
-        t -= nt - bm;
-        ++bm;
-    }
-    bn = bm + t;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     using C = NsTile<T>;
-    __shared__ __align__(16) T smem[2 * C::S * C::P + 4 * C::S * C::S];
+    __shared__ __align__(16) T smem[C::S * (C::P + C::KC) + 4 * C::S * C::S];
     __shared__ double sh[kNsThreads / 32];
     __shared__ int abort_sh;
     unsigned gen = 0;
     const int N = a.N, ld = a.ld, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nt = (N + C::S - 1) / C::S, tiles = nt * (nt + 1) / 2;
+    const int nt = (N + C::S - 1) / C::S, tiles = nt * nt;
     const size_t all = (size_t)gridDim.x * kNsThreads, me = (size_t)blockIdx.x * kNsThreads + tid;
     // c = largest row sum
     for (int r = blockIdx.x * (kNsThreads / 32) + warp; r < N; r += gridDim.x * (kNsThreads / 32)) {
@@ -336,10 +330,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     }
     if (!grid_barrier(a.bar, gen, &abort_sh)) return;
     T *Y = a.Y, *Z = a.Z, *Y2 = a.Y2, *Z2 = a.Z2;
-    auto put = [&](T* M, int m, int n, T v) {
-        __stcg(M + (size_t)m * ld + n, v);
-        __stcg(M + (size_t)n * ld + m, v);
-    };
+    auto put = [&](T* M, int m, int n, T v) { __stcg(M + (size_t)m * ld + n, v); };
     // sum over the CTAs in a fixed order: every CTA decides alike
     auto total = [&]() {
         double s = 0.0;
@@ -363,16 +354,13 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         }
         if (it > 0) {
             double h = 0.0;
-            for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
-                int bm, bn;
-                tile_of(t, nt, bm, bn);
-                grid_product<T>(N, ld, Z, Y, bm, bn, smem, [&](int m, int n, T v) {
+            for (int t = blockIdx.x; t < tiles; t += gridDim.x)
+                grid_product<T>(N, ld, Z, Y, t / nt, t % nt, smem, [&](int m, int n, T v) {
                     const T d = m == n ? T(1) : T(0);
                     const double x = (double)(d - v);
-                    h += m == n ? x * x : 2.0 * x * x;
+                    h += x * x;
                     put(a.W, m, n, T(0.5) * (T(2) * d + (d - v)));
                 });
-            }
             h = block_sum(h, sh);
             if (tid == 0) __stcg(a.part + blockIdx.x, h);
             if (!grid_barrier(a.bar, gen, &abort_sh)) return;
@@ -383,8 +371,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
             }
         }
         for (int t = blockIdx.x; t < (it > 0 ? 2 : 1) * tiles; t += gridDim.x) {
-            int bm, bn;
-            tile_of(t < tiles ? t : t - tiles, nt, bm, bn);
+            const int bm = t % tiles / nt, bn = t % nt;
             if (t < tiles) grid_product<T>(N, ld, Y, a.W, bm, bn, smem, [&](int m, int n, T v) { put(Y2, m, n, v); });
             else grid_product<T>(N, ld, a.W, Z, bm, bn, smem, [&](int m, int n, T v) { put(Z2, m, n, v); });
         }
@@ -400,7 +387,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     double f = 0.0;
     const double s = 1.0 / sqrt(c);
     for (size_t e = me; e < (size_t)N * N; e += all) {
-        const double z = (double)__ldcg(Z + (e / N) * ld + e % N);
+        const double z = 0.5 * ((double)__ldcg(Z + (e / N) * ld + e % N) + (double)__ldcg(Z + (e % N) * ld + e / N));
         f += z * z;
         if (ok) a.X[e] = s * z;
     }
@@ -466,7 +453,8 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, c
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kNsThreads, 0))) return e;
         if (per_sm < 1 || sms > kNsMaxCtas) return cudaErrorCooperativeLaunchTooLarge;
         const int nt = (N + NsTile<T>::S - 1) / NsTile<T>::S;
-        const int ctas = std::min(sms, nt * (nt + 1));  // the two products of a step side by side
+        // the two products of a step side by side
+        const int ctas = std::min({sms * std::min(per_sm, 2), kNsMaxCtas, 2 * nt * nt});
         void* args[] = {(void*)&a};
         if ((e = cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(kNsThreads), args, 0, s))) return e;
     }
