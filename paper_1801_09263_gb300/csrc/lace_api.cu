@@ -166,21 +166,137 @@ lace_status ensure_orbital_buffers(lace_ctx* c, int n_occ, int n_extra) {
     CK(c->mat.ensure(c->mslot * kMatSlots * sizeof(double)), "alloc matrices");
     const size_t wk = std::max(gemm_rows_work_elems(n_p, n_p, ng), (size_t)1);
     CK(c->work.ensure(wk * sizeof(double)), "alloc work");
+    CK(c->rowmax.ensure(sizeof(unsigned) * 4 * (size_t)n_p), "alloc row maxima");
     CK(c->flag.ensure(64), "alloc flag");
     CK(c->exd.ensure((8 + 2 * kSumBlocks) * sizeof(double)), "alloc exd");  // [0] E_x, [1] ACE energy, sum scratch
     CK(c->counts.ensure(sizeof(int) * (2 * (size_t)n_occ + 2)), "alloc counts");
     return LACE_OK;
 }
 
+// Timeout flags of the tensor-core calls (see lace_ctx::hflags): a call
+// takes slot s of the device flags (or, with none left, waits for its own,
+// h_err != nullptr), and tc_flag_copy queues the slot's copy to the pinned
+// host flags; tc_timed_out, after the API call's stream synchronisation,
+// reports whether any of them gave up.
+struct TcFlag {
+    int* d = nullptr;  // device slot
+    int* h = nullptr;  // host word to wait on (synchronous mode) or nullptr
+    int s = -1;
+    int herr = 0;
+};
+TcFlag tc_flag(lace_ctx* c) {
+    TcFlag f;
+    if (c->hflags && c->tc_next < kFlagSlots) {
+        f.s = c->tc_next++;
+        c->hflags[f.s] = 0;
+        f.d = c->flag.as<int>() + f.s;
+    } else {
+        f.d = c->flag.as<int>() + 1;
+        f.h = &f.herr;
+    }
+    return f;
+}
+cudaError_t tc_flag_copy(lace_ctx* c, const TcFlag& f) {
+    if (f.s < 0) return cudaSuccess;
+    return cudaMemcpyAsync(c->hflags + f.s, f.d, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
+}
+bool tc_timed_out(lace_ctx* c) {
+    bool any = false;
+    for (int k = 2; k < c->tc_next; ++k) any |= c->hflags[k] != 0;
+    c->tc_next = 2;
+    return any;
+}
+
+// Row maxima of the contractions below: raw occupied orbitals, extras, and
+// the two sets of an alignment.
+unsigned* max_occ(lace_ctx* c) { return c->rowmax.as<unsigned>(); }
+unsigned* max_extra(lace_ctx* c) { return c->rowmax.as<unsigned>() + c->n_occ; }
+unsigned* max_w(lace_ctx* c) { return c->rowmax.as<unsigned>() + c->n_p; }
+unsigned* max_ref(lace_ctx* c) { return c->rowmax.as<unsigned>() + 2 * (size_t)c->n_p; }
+
+// M x N x K contractions of orbital rows from here on take the tensor-core
+// kernels of tc_exact.cu, whose tiles are 128 wide and which need the rows'
+// maxima and cut coefficients.  Load and localisation, CUDA cores -> tensor cores:
+// 1.0e9 at 96 orbitals 0.86 -> 0.78 ms and at 128 0.93 -> 0.91, 5.4e8 at 128 even;
+// half-filled tiles 1.1e9 at 64 orbitals 0.79 -> 0.81 and 2.0e9 at 48 0.99 -> 1.00,
+// 4.5e8 and less slower by 0.03-0.04.
+bool exact_size(size_t M, size_t N, size_t K) {
+    return (double)M * (double)N * (double)K >= (std::min(M, N) > 64 ? 1e9 : 2e9);
+}
+bool tc_off() {  // LACE_NO_TC=1: the CUDA cores
+    const char* e = getenv("LACE_NO_TC");
+    return e && e[0] == '1';
+}
+// Whether any contraction of the loaded rows can be one of those (decides at
+// the load whether their maxima are taken: lace_ctx::rows_max).
+bool wants_row_max(lace_ctx* c) {
+    const size_t n = std::max(c->n_occ, c->n_extra);
+    return c->prec != LACE_FP64 && !tc_off() && exact_size(n, n, c->g.ng) && exact_ok(c->g.ng, c->canon.p);
+}
+template <typename T> bool use_exact(lace_ctx* c, size_t M, size_t N, size_t K, const T* a) {
+    return std::is_same<T, float>::value && c->rows_max && !tc_off() && exact_size(M, N, K) && exact_ok(K, a);
+}
+lace_status exact_done(lace_ctx* c, TcFlag& f, const char* where) {
+    if (f.h) {  // no slot left: wait for this call's own flag
+        CK(cudaMemcpyAsync(f.h, f.d, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "flags");
+        CK(cudaStreamSynchronize(c->stream), "flags");
+        if (f.herr) return fail(c, LACE_ERR_TIMEOUT, std::string(where) + ": an mbarrier wait timed out");
+    }
+    CK(tc_flag_copy(c, f), "flags");
+    return LACE_OK;
+}
+// The largest |x| of each row of X for the two calls below.
+template <typename T>
+lace_status orbital_max(lace_ctx* c, const T* X, int rows, size_t K, unsigned* mx, Launch& L) {
+    if constexpr (std::is_same<T, float>::value)
+        if (c->rows_max && exact_ok(K, X)) CK(row_max(X, rows, K, mx, c->stream, &L.n), "row maxima");
+    return LACE_OK;
+}
+// C = alpha A B^T over rows of K values.
+template <typename T>
+lace_status orbital_gram(lace_ctx* c, int M, int N, size_t K, const T* A, const unsigned* ma, const T* B, const unsigned* mb,
+                         double alpha, double* C, int ldc, Launch& L, const char* where) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (use_exact(c, M, N, K, A) && exact_ok(K, B)) {
+            CK(c->work.ensure(std::max(c->work.bytes, gram_exact_work_elems(M, N, K, A == B && M == N) * sizeof(double))),
+               "alloc work");
+            TcFlag f = tc_flag(c);
+            CK(gram_exact(M, N, K, A, ma, B, mb, alpha, C, ldc, c->work.as<double>(), c->work.bytes / sizeof(double), f.d,
+                          c->stream, &L.n),
+               where);
+            return exact_done(c, f, where);
+        }
+    }
+    CK(gemm_rows<T>(M, N, K, A, K, B, K, alpha, false, C, ldc, c->work.as<double>(), c->work.bytes / sizeof(double),
+                    c->stream, &L.n),
+       where);
+    return LACE_OK;
+}
+// Out[n] = (add ? Out[n] : 0) + sum_k Coef[k][n] A[k] over rows of K values.
+template <typename T>
+lace_status orbital_combine(lace_ctx* c, int N, size_t K, int Kc, const T* A, const unsigned* ma, const double* Coef, int ldcoef,
+                            bool add, T* Out, Launch& L, const char* where) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (use_exact(c, N, Kc, K, A) && exact_ok(K, Out)) {
+            CK(c->slices.ensure(combine_exact_scratch_bytes(N, Kc)), "alloc slices");
+            TcFlag f = tc_flag(c);
+            CK(combine_exact(N, K, Kc, A, ma, Coef, ldcoef, add, Out, K, c->slices.p, f.d, c->stream, &L.n), where);
+            return exact_done(c, f, where);
+        }
+    }
+    CK(gemm_combine<T>(N, K, Kc, A, K, Coef, ldcoef, add ? 1.0 : 0.0, Out, K, c->stream, &L.n), where);
+    return LACE_OK;
+}
+
 // Loewdin coefficients: X = S^{-1/2}, S = dV src src^T (FP64 Newton-Schulz;
 // mixed path: FP32 Newton-Schulz and one FP64 first-order refinement).
 template <typename T>
-lace_status lowdin_coeffs(lace_ctx* c, const T* src, int n, double* X, Launch& L) {
-    const size_t ng = c->g.ng;
+lace_status lowdin_coeffs(lace_ctx* c, const T* src, const unsigned* mx, int n, double* X, Launch& L) {
     double* S = c->m(MS_A);
-    CK(gemm_rows<T>(n, n, ng, src, ng, src, ng, c->g.dv, false, S, n, c->work.as<double>(),
-                    c->work.bytes / sizeof(double), c->stream, &L.n),
-       "loewdin overlap");
+    {
+        lace_status st = orbital_gram<T>(c, n, n, c->g.ng, src, mx, src, mx, c->g.dv, S, n, L, "loewdin overlap");
+        if (st) return st;
+    }
     int ok = 0;
     if (c->prec == LACE_FP64) {
         CK(inv_sqrt_spd(n, S, X, c->m(MS_NSWORK), &ok, c->stream, &L.n), "loewdin inverse sqrt");
@@ -195,12 +311,26 @@ lace_status lowdin_coeffs(lace_ctx* c, const T* src, int n, double* X, Launch& L
 
 // Loewdin: dst[n] = sum_k src[k] X[k][n], X = S^{-1/2}, S = dV src src^T.
 template <typename T>
-lace_status lowdin_rows(lace_ctx* c, const T* src, int n, T* dst, Launch& L) {
+lace_status lowdin_rows(lace_ctx* c, const T* src, const unsigned* mx, int n, T* dst, Launch& L) {
     double* X = c->m(MS_B);
-    lace_status st = lowdin_coeffs<T>(c, src, n, X, L);
+    lace_status st = lowdin_coeffs<T>(c, src, mx, n, X, L);
     if (st) return st;
-    CK(gemm_combine<T>(n, c->g.ng, n, src, c->g.ng, X, n, 0.0, dst, c->g.ng, c->stream, &L.n), "loewdin combine");
-    return LACE_OK;
+    return orbital_combine<T>(c, n, c->g.ng, n, src, mx, X, n, false, dst, L, "loewdin combine");
+}
+
+// FP64 orbitals to the working precision, with the row maxima of the
+// tensor-core contractions in the same pass.
+template <typename T>
+lace_status load_rows(lace_ctx* c, const double* src, T* dst, int rows, unsigned* mx, Launch& L) {
+    const size_t ng = c->g.ng;
+    if constexpr (std::is_same<T, float>::value) {
+        if (c->rows_max && exact_ok(ng, dst) && (uintptr_t)src % 16 == 0) {
+            CK(convert_row_max(src, dst, rows, ng, mx, c->stream, &L.n), "load convert");
+            return LACE_OK;
+        }
+    }
+    CK(convert<double, T>(src, dst, (size_t)rows * ng, c->stream, &L.n), "load convert");
+    return orbital_max<T>(c, dst, rows, ng, mx, L);
 }
 
 // The occupied orbitals stay raw (canon buffer) with their Loewdin
@@ -213,36 +343,41 @@ lace_status load_impl(lace_ctx* c, const double* d_phi64, int n_occ, int n_extra
     T* psi = c->psi.as<T>();
     T* raw = c->canon.as<T>();
     double* X = c->m(MS_X);
-    CK(convert<double, T>(d_phi64, raw, (size_t)n_occ * ng, c->stream, &L.n), "load convert");
+    c->rows_max = wants_row_max(c);
+    {
+        lace_status st = load_rows<T>(c, d_phi64, raw, n_occ, max_occ(c), L);
+        if (st) return st;
+    }
     c->x_identity = !ortho;
     c->psi_occ_ready = false;
     if (ortho) {
-        lace_status st = lowdin_coeffs<T>(c, raw, n_occ, X, L);
+        lace_status st = lowdin_coeffs<T>(c, raw, max_occ(c), n_occ, X, L);
         if (st) return st;
     }
     if (n_extra > 0) {
         T* ex_raw = c->W.as<T>();  // staging
-        CK(convert<double, T>(d_phi64 + (size_t)n_occ * ng, ex_raw, (size_t)n_extra * ng, c->stream, &L.n),
-           "load convert");
+        lace_status st = load_rows<T>(c, d_phi64 + (size_t)n_occ * ng, ex_raw, n_extra, max_extra(c), L);
+        if (st) return st;
         if (ortho) {
             // extra -= canon (dV canon^T extra), canon = raw X:  coefficients -X X^T G,
             // G = dV raw^T extra
             double* G = c->m(MS_A);
             double* T1 = c->m(MS_B);
             double* D = c->m(MS_LINV);
-            CK(gemm_rows<T>(n_occ, n_extra, ng, raw, ng, ex_raw, ng, c->g.dv, false, G, n_extra, c->work.as<double>(),
-                            c->work.bytes / sizeof(double), c->stream, &L.n),
-               "extras projection");
+            if ((st = orbital_gram<T>(c, n_occ, n_extra, ng, raw, max_occ(c), ex_raw, max_extra(c), c->g.dv, G, n_extra, L,
+                                      "extras projection")))
+                return st;
             CK(small_gemm_f64(n_occ, n_extra, n_occ, X, n_occ, true, G, n_extra, false, 1.0, 0.0, T1, n_extra,
                               c->stream, &L.n),
                "extras projection");
             CK(small_gemm_f64(n_occ, n_extra, n_occ, X, n_occ, false, T1, n_extra, false, -1.0, 0.0, D, n_extra,
                               c->stream, &L.n),
                "extras projection");
-            CK(gemm_combine<T>(n_extra, ng, n_occ, raw, ng, D, n_extra, 1.0, ex_raw, ng, c->stream, &L.n),
-               "extras projection");
-            lace_status st = lowdin_rows<T>(c, ex_raw, n_extra, psi + (size_t)n_occ * ng, L);
-            if (st) return st;
+            if ((st = orbital_combine<T>(c, n_extra, ng, n_occ, raw, max_occ(c), D, n_extra, true, ex_raw, L,
+                                         "extras projection")) ||
+                (st = orbital_max<T>(c, ex_raw, n_extra, ng, max_extra(c), L)) ||
+                (st = lowdin_rows<T>(c, ex_raw, max_extra(c), n_extra, psi + (size_t)n_occ * ng, L)))
+                return st;
         } else {
             CK(cudaMemcpyAsync(psi + (size_t)n_occ * ng, ex_raw, (size_t)n_extra * ng * sizeof(T),
                                cudaMemcpyDeviceToDevice, c->stream),
@@ -262,17 +397,23 @@ lace_status materialize_impl(lace_ctx* c) {
         CK(cudaMemcpyAsync(c->psi.p, c->canon.p, (size_t)n * ng * sizeof(T), cudaMemcpyDeviceToDevice, c->stream),
            "orbitals");
     } else {
-        CK(gemm_combine<T>(n, ng, n, c->canon.as<T>(), ng, c->m(MS_X), n, 0.0, c->psi.as<T>(), ng, c->stream, &L.n),
-           "loewdin combine");
+        return orbital_combine<T>(c, n, ng, n, c->canon.as<T>(), max_occ(c), c->m(MS_X), n, false, c->psi.as<T>(), L,
+                                  "loewdin combine");
     }
     return LACE_OK;
 }
 
 lace_status materialize_psi(lace_ctx* c) {
     if (c->psi_occ_ready) return LACE_OK;
+    c->tc_next = 2;
     lace_status st = c->prec == LACE_FP64 ? materialize_impl<double>(c) : materialize_impl<float>(c);
-    if (st == LACE_OK) c->psi_occ_ready = true;
-    return st;
+    if (st) return st;
+    if (c->hflags && c->tc_next > 2) {
+        CK(cudaStreamSynchronize(c->stream), "loewdin combine");
+        if (tc_timed_out(c)) return fail(c, LACE_ERR_TIMEOUT, "loewdin combine: an mbarrier wait timed out");
+    }
+    c->psi_occ_ready = true;
+    return LACE_OK;
 }
 
 lace_status load_common(lace_ctx* c, const double* phi, bool dev, int n_occ, int n_extra, int ortho) {
@@ -292,6 +433,7 @@ lace_status load_common(lace_ctx* c, const double* phi, bool dev, int n_occ, int
     c->n_extra = n_extra;
     c->n_p = n_occ + n_extra;
     ev_begin(c, ST_LOAD);
+    c->tc_next = 2;
     const size_t bytes = (size_t)c->n_p * c->g.ng * sizeof(double);
     const double* src = phi;
     if (!dev) {
@@ -303,6 +445,8 @@ lace_status load_common(lace_ctx* c, const double* phi, bool dev, int n_occ, int
     ev_end(c, ST_LOAD);
     if (st) return st;
     CK(cudaStreamSynchronize(c->stream), "load");
+    if (c->hflags && tc_timed_out(c))
+        return fail(c, LACE_ERR_TIMEOUT, "orthonormalisation: an mbarrier wait timed out");
     c->loaded = true;
     return LACE_OK;
 }
@@ -334,8 +478,8 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
         } else {
             T* tmp = c->W.as<T>();
             CK(gather_subsample<T>(c->g, stride, raw, n, tmp, &ncol, c->stream, &L.n), "subsample");
-            CK(gemm_combine<T>(n, (size_t)ncol, n, tmp, (size_t)ncol, X, n, 0.0, R, (size_t)ncol, c->stream, &L.n),
-               "subsample");
+            lace_status st = orbital_combine<T>(c, n, (size_t)ncol, n, tmp, max_occ(c), X, n, false, R, L, "subsample");
+            if (st) return st;
         }
         int timeout = 0;
         CK(qrcp_pivots<T>(n, ncol, R, n, c->piv.as<int>(), c->aux.p, &timeout, c->wait_limit_ns, c->stream, &L.n),
@@ -388,7 +532,10 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
         CK(small_gemm_f64(n, n, n, X, n, false, U, n, false, 1.0, 0.0, XU, n, c->stream, &L.n), "scdm rotate");
         Cf = XU;
     }
-    CK(gemm_combine<T>(n, ng, n, raw, ng, Cf, n, 0.0, c->psi.as<T>(), ng, c->stream, &L.n), "scdm rotate");
+    {
+        lace_status st = orbital_combine<T>(c, n, ng, n, raw, max_occ(c), Cf, n, false, c->psi.as<T>(), L, "scdm rotate");
+        if (st) return st;
+    }
     c->psi_occ_ready = true;
     return LACE_OK;
 }
@@ -407,9 +554,10 @@ lace_status align_impl(lace_ctx* c) {
     double* P = c->m(MS_B);
     double* Pmh = c->m(MS_LINV);
     double* Q = c->m(MS_LINVT);
-    CK(gemm_rows<T>(n, n, ng, w, ng, ref, ng, c->g.dv, false, Om, n, c->work.as<double>(),
-                    c->work.bytes / sizeof(double), c->stream, &L.n),
-       "alignment overlap");
+    lace_status st;
+    if ((st = orbital_max<T>(c, w, n, ng, max_w(c), L)) || (st = orbital_max<T>(c, ref, n, ng, max_ref(c), L)) ||
+        (st = orbital_gram<T>(c, n, n, ng, w, max_w(c), ref, max_ref(c), c->g.dv, Om, n, L, "alignment overlap")))
+        return st;
     CK(small_gemm_f64(n, n, n, Om, n, true, Om, n, false, 1.0, 0.0, P, n, c->stream, &L.n), "alignment");
     int ok = 0;
     CK(inv_sqrt_spd(n, P, Pmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "alignment");
@@ -421,46 +569,12 @@ lace_status align_impl(lace_ctx* c) {
     CK(small_gemm_f64(n, n, n, U, n, false, Q, n, false, 1.0, 0.0, UQ, n, c->stream, &L.n), "alignment");
     CK(cudaMemcpyAsync(U, UQ, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, c->stream), "alignment");
     T* tmp = c->W.as<T>();
-    CK(gemm_combine<T>(n, ng, n, w, ng, Q, n, 0.0, tmp, ng, c->stream, &L.n), "alignment");
+    if ((st = orbital_combine<T>(c, n, ng, n, w, max_w(c), Q, n, false, tmp, L, "alignment"))) return st;
     CK(cudaMemcpyAsync(w, tmp, (size_t)n * ng * sizeof(T), cudaMemcpyDeviceToDevice, c->stream), "alignment");
     return LACE_OK;
 }
 
 // ------------------------------------------------------------------ screening
-// Timeout flags of the tensor-core calls (see lace_ctx::hflags): a call
-// takes slot s of the device flags (or, with none left, waits for its own,
-// h_err != nullptr), and tc_flag_copy queues the slot's copy to the pinned
-// host flags; tc_timed_out, after the API call's stream synchronisation,
-// reports whether any of them gave up.
-struct TcFlag {
-    int* d = nullptr;  // device slot
-    int* h = nullptr;  // host word to wait on (synchronous mode) or nullptr
-    int s = -1;
-    int herr = 0;
-};
-TcFlag tc_flag(lace_ctx* c) {
-    TcFlag f;
-    if (c->hflags && c->tc_next < kFlagSlots) {
-        f.s = c->tc_next++;
-        c->hflags[f.s] = 0;
-        f.d = c->flag.as<int>() + f.s;
-    } else {
-        f.d = c->flag.as<int>() + 1;
-        f.h = &f.herr;
-    }
-    return f;
-}
-cudaError_t tc_flag_copy(lace_ctx* c, const TcFlag& f) {
-    if (f.s < 0) return cudaSuccess;
-    return cudaMemcpyAsync(c->hflags + f.s, f.d, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
-}
-bool tc_timed_out(lace_ctx* c) {
-    bool any = false;
-    for (int k = 2; k < c->tc_next; ++k) any |= c->hflags[k] != 0;
-    c->tc_next = 2;
-    return any;
-}
-
 // S_ik = dV sum_r |psi_i(r)| |psi_k(r)| (Eq. 4).  Mixed path: tcgen05 3xBF16
 // (S only decides which pairs pass the threshold; the Gram's periodic
 // compensated drains keep it ~1e-7 relative), symmetric tiles only; FP64 and
@@ -472,8 +586,7 @@ lace_status screen_impl(lace_ctx* c, double thr) {
     const int n = c->n_occ;
     const T* psi = c->psi.as<T>();
     if constexpr (std::is_same<T, float>::value) {
-        const char* notc = getenv("LACE_NO_TC");
-        if (!(notc && notc[0] == '1') && ng % 4 == 0 && (uintptr_t)psi % 16 == 0) {
+        if (!tc_off() && ng % 4 == 0 && (uintptr_t)psi % 16 == 0) {
             CK(c->work.ensure(std::max(c->work.bytes, tc_gram_work_elems(n, n, ng, true) * sizeof(double))),
                "alloc work");
             TcFlag f = tc_flag(c);
@@ -629,9 +742,8 @@ template <typename T>
 lace_status ace_contract(lace_ctx* c, int M, int N, const T* A, const T* B, double alpha, double* C, Launch& L) {
     const size_t ng = c->g.ng;
     if constexpr (std::is_same<T, float>::value) {
-        const char* notc = getenv("LACE_NO_TC");
         const bool aligned = ng % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0;
-        if (!(notc && notc[0] == '1') && aligned) {
+        if (!tc_off() && aligned) {
             CK(c->work.ensure(std::max(c->work.bytes, tc_gram_work_elems(M, N, ng) * sizeof(double))), "alloc work");
             TcFlag f = tc_flag(c);
             CK(tc_gram(M, N, ng, A, ng, B, ng, alpha, C, N, c->work.as<double>(), c->work.bytes / sizeof(double),
@@ -658,8 +770,7 @@ template <typename T, typename TO>
 lace_status ace_combine(lace_ctx* c, int N, int Kc, const T* A, const double* Coef, TO* Out, Launch& L) {
     const size_t ng = c->g.ng;
     if constexpr (std::is_same<T, float>::value) {
-        const char* notc = getenv("LACE_NO_TC");
-        if (!(notc && notc[0] == '1')) {
+        if (!tc_off()) {
             CK(c->work.ensure(std::max(c->work.bytes, tc_combine_scratch_bytes(N, Kc))), "alloc work");
             TcFlag f = tc_flag(c);
             CK(tc_combine(N, ng, Kc, A, ng, Coef, N, 0.0, Out, ng, c->work.p, f.d, f.h, c->stream, &L.n),
@@ -840,6 +951,11 @@ size_t predict_ctx_bytes(int prec, const int n[3], int n_occ, int n_extra, int n
         work = std::max(work, tc_gram_work_elems((int)n_p, (int)n_p, ng) * sizeof(double));
         work = std::max(work, tc_gram_work_elems(n_occ, n_occ, ng, true) * sizeof(double));
         work = std::max(work, tc_combine_scratch_bytes((int)n_p, (int)n_p));
+        work = std::max(work, gram_exact_work_elems(n_occ, n_occ, ng, true) * sizeof(double));
+        if (n_extra) {
+            work = std::max(work, gram_exact_work_elems(n_occ, n_extra, ng, false) * sizeof(double));
+            work = std::max(work, gram_exact_work_elems(n_extra, n_extra, ng, true) * sizeof(double));
+        }
         if (na) {
             work = std::max(work, tc_gram_work_elems((int)n_p, (int)na, ng) * sizeof(double));
             work = std::max(work, tc_combine_scratch_bytes((int)na, (int)n_p));
@@ -848,6 +964,8 @@ size_t predict_ctx_bytes(int prec, const int n[3], int n_occ, int n_extra, int n
     if (na) work = std::max(work, gemm_rows_work_elems((int)n_p, (int)na, ng) * sizeof(double));
     const size_t mslot = n_p * n_p + 64 * n_p + 64;
     size_t b = 0;
+    if (prec != LACE_FP64)  // coefficient slices and row maxima
+        b += combine_exact_scratch_bytes(std::max(n_occ, n_extra), std::max(n_occ, n_extra)) + 4 * n_p * sizeof(unsigned);
     b += 3 * n_p * ng * eb;        // psi, W, xi
     b += (size_t)n_occ * ng * eb;  // canonical orbitals
     b += n_p * ng * 8;             // FP64 staging
@@ -915,7 +1033,7 @@ lace_status lace_destroy(lace_ctx* c) {
     cudaStreamSynchronize(c->stream);
     DevBuf* bufs[] = {&c->psi, &c->canon, &c->W, &c->xi, &c->stage64, &c->scratch, &c->work, &c->aux, &c->mat,
                       &c->pairs, &c->counts, &c->grids, &c->epart, &c->flag, &c->piv, &c->pivfull, &c->exd,
-                      &c->aceio, &c->ref, &c->pw_idx, &c->pw_io, &c->pw_real};
+                      &c->aceio, &c->rowmax, &c->slices, &c->ref, &c->pw_idx, &c->pw_io, &c->pw_real};
     for (DevBuf* b : bufs) b->release();
     for (int a = 0; a < 3; ++a) { c->tw_d[a].release(); c->tw_f[a].release(); c->g2_d[a].release(); c->g2_f[a].release(); }
     c->ktab_f.release();
@@ -1008,11 +1126,13 @@ static lace_status localize_common(lace_ctx* c, int stride, const long long* imp
     cudaSetDevice(c->device);
     c->localized = c->screened = c->applied = false;
     ev_begin(c, ST_LOCALIZE);
+    c->tc_next = 2;
     lace_status st = c->prec == LACE_FP64 ? localize_impl<double>(c, stride, imposed)
                                           : localize_impl<float>(c, stride, imposed);
     ev_end(c, ST_LOCALIZE);
     if (st) return st;
     CK(cudaStreamSynchronize(c->stream), "localize");
+    if (c->hflags && tc_timed_out(c)) return fail(c, LACE_ERR_TIMEOUT, "rotation: an mbarrier wait timed out");
     if (pivots_out) std::copy(c->pivots_host.begin(), c->pivots_host.end(), pivots_out);
     c->localized = true;
     return LACE_OK;
@@ -1042,6 +1162,7 @@ lace_status lace_align_to_previous(lace_ctx* c, int* aligned_out) {
     if (aligned_out) *aligned_out = 0;
     if (c->have_ref && c->ref_n == c->n_occ && c->ref.bytes >= bytes) {
         c->screened = c->applied = false;
+        c->tc_next = 2;
         lace_status st = c->prec == LACE_FP64 ? align_impl<double>(c) : align_impl<float>(c);
         if (st) return st;
         if (aligned_out) *aligned_out = 1;
@@ -1049,6 +1170,7 @@ lace_status lace_align_to_previous(lace_ctx* c, int* aligned_out) {
     CK(c->ref.ensure(bytes), "alloc alignment reference");
     CK(cudaMemcpyAsync(c->ref.p, c->psi.p, bytes, cudaMemcpyDeviceToDevice, c->stream), "alignment");
     CK(cudaStreamSynchronize(c->stream), "alignment");
+    if (c->hflags && tc_timed_out(c)) return fail(c, LACE_ERR_TIMEOUT, "alignment: an mbarrier wait timed out");
     c->have_ref = true;
     c->ref_n = c->n_occ;
     return LACE_OK;
@@ -1358,8 +1480,8 @@ lace_status lace_get_device_bytes(lace_ctx* c, unsigned long long* bytes_out) {
     if (!c || !bytes_out) return LACE_ERR_ARG;
     const DevBuf* bufs[] = {&c->psi,   &c->canon, &c->W,      &c->xi,    &c->stage64, &c->scratch, &c->work,
                             &c->aux,   &c->mat,   &c->pairs,  &c->counts, &c->grids,  &c->epart,   &c->flag,
-                            &c->piv,   &c->pivfull, &c->exd,  &c->aceio, &c->ktab_f, &c->ktab_d, &c->klanes, &c->ref,
-                            &c->pw_idx, &c->pw_io,  &c->pw_real};
+                            &c->piv,   &c->pivfull, &c->exd,  &c->aceio, &c->ktab_f, &c->ktab_d, &c->klanes, &c->rowmax,
+                            &c->slices, &c->ref, &c->pw_idx, &c->pw_io,  &c->pw_real};
     unsigned long long b = 0;
     for (const DevBuf* d : bufs) b += d->bytes;
     for (int a = 0; a < 3; ++a) b += c->tw_d[a].bytes + c->tw_f[a].bytes + c->g2_d[a].bytes + c->g2_f[a].bytes;

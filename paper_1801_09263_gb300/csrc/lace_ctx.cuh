@@ -86,6 +86,9 @@ struct lace_ctx {
     DevBuf mat;     // small FP64 matrices (see offsets below)
     DevBuf pairs, counts, grids, epart, flag, piv, pivfull, exd;
     DevBuf aceio;   // FP64 device copies of a host ACE apply's input and output
+    DevBuf rowmax;  // largest |x| of orbital rows (FP32 bits): raw occupied, extras, alignment
+    bool rows_max = false;  // rowmax holds the loaded rows' maxima
+    DevBuf slices;  // coefficient slices of a rotation
     DevBuf ref;     // [n_occ][ng] localised orbitals of the previous alignment
     DevBuf pw_idx, pw_io, pw_real;  // plane-wave front end: G offsets, coefficients, FP64 orbitals
     double ecut = 0.0;              // orbital cutoff of lace_set_cell (Ha)

@@ -184,6 +184,24 @@ cudaError_t tc_combine(int N, size_t K, int Kc, const float* A, size_t lda, cons
                        int* launches);
 size_t tc_combine_scratch_bytes(int N, int Kc);
 
+// FP32-accurate contractions on the tensor cores (tc_exact.cu; rows of K values,
+// contiguous, K % 4 == 0, 16-byte aligned: exact_ok).  max_*: the bits of the
+// largest |x| of each row (a bound will do), from row_max or, with the rounding
+// of FP64 rows to FP32, convert_row_max (16-byte aligned input).  d_err: set
+// when a bounded mbarrier wait gave up.
+bool exact_ok(size_t K, const void* a);
+cudaError_t convert_row_max(const double* in, float* out, int rows, size_t n, unsigned* d_max, cudaStream_t s, int* launches);
+cudaError_t row_max(const float* in, int rows, size_t n, unsigned* d_max, cudaStream_t s, int* launches);
+// C[m][n] = alpha sum_r A[m][r] B[n][r] (A == B: symmetric).
+cudaError_t gram_exact(int M, int N, size_t K, const float* A, const unsigned* max_a, const float* B, const unsigned* max_b,
+                       double alpha, double* C, int ldc, double* work, size_t work_elems, int* d_err, cudaStream_t s,
+                       int* launches);
+size_t gram_exact_work_elems(int M, int N, size_t K, bool sym);
+// Out[n][r] = (add ? Out[n][r] : 0) + sum_k Coef[k][n] A[k][r].
+cudaError_t combine_exact(int N, size_t K, int Kc, const float* A, const unsigned* max_a, const double* Coef, int ldcoef,
+                          bool add, float* Out, size_t ldo, void* scratch, int* d_err, cudaStream_t s, int* launches);
+size_t combine_exact_scratch_bytes(int N, int Kc);
+
 // Small FP64 dense kernels (N x N).
 cudaError_t small_gemm_f64(int M, int N, int K, const double* A, int lda, bool ta, const double* B, int ldb, bool tb,
                            double alpha, double beta, double* C, int ldc, cudaStream_t s, int* launches);

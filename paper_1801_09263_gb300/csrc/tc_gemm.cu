@@ -34,84 +34,17 @@
 #include <algorithm>
 
 #include "lace_internal.cuh"
+#include "tc_util.cuh"
 
 namespace lace {
 
 namespace {
 
-constexpr int TC_M = 128, TC_N = 128, TC_BK = 64, TC_THREADS = 512;
+constexpr int TC_BK = 64, TC_THREADS = 512;
 constexpr int TC_VPT = (TC_M * TC_BK / 4) / TC_THREADS;  // float4 vectors per thread per tile
 constexpr int TC_TILE_BYTES = TC_M * TC_BK * 2;      // 16 KB per BF16 tile
 constexpr int TC_STAGE_BYTES = 4 * TC_TILE_BYTES;    // A_hi, A_lo, B_hi, B_lo
 constexpr int TC_SMEM_BYTES = 2 * TC_STAGE_BYTES + 1024;  // + alignment slack
-constexpr long long TC_WAIT_LIMIT = 1LL << 26;       // bounded mbarrier polls
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
-}
-
-// Bounded wait for the completion of the phase with the given parity.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    const uint32_t a = smem_u32(bar);
-    for (long long it = 0; it < TC_WAIT_LIMIT; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\n"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            "selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
-// 128-byte swizzled K-major shared-memory descriptor (SBO = 1024 B between
-// 8-row groups, version 1, layout type 2 = SWIZZLE_128B).
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;                  // leading byte offset (unused for swizzled K-major)
-    d |= (uint64_t)(1024 >> 4) << 32;        // stride byte offset
-    d |= (uint64_t)1 << 46;                  // descriptor version
-    d |= (uint64_t)2 << 61;                  // SWIZZLE_128B
-    return d;
-}
-
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, M = 128, N = 128.
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_N >> 3) << 17) |
-                            ((uint32_t)(TC_M >> 4) << 24);
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(kIdesc), "r"(accumulate));
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-
-// Byte offset of BF16 element (row r, k) in a 128-byte swizzled K-major tile of 64 columns.
-__device__ __forceinline__ uint32_t sw128_off(int r, int k) {
-    return (uint32_t)(r * 128 + ((((k >> 3) ^ (r & 7)) & 7) << 4) + (k & 7) * 2);
-}
-
-// Two FP32 values rounded to BF16 (round to nearest even) and packed: x0 in
-// the low half (the lower address), x1 in the high half.
-__device__ __forceinline__ uint32_t bf16x2_rn(float x0, float x1) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
-    return r;
-}
 
 // hi = bf16(x), lo = bf16(x - hi) for four values, packed in element order
 // (one conversion instruction per two values; a BF16 value widens to FP32
@@ -290,22 +223,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
-// ---------------------------------------------------------------------------
-// TMA helpers.
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-// 2D tile load: box at element coordinates (x = column, y = row) of the map.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-        "[%4];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-
 // Geometry of the TMA-fed Gram (tc_gram_ws_kernel): 32-wide K steps, so that
 // two BF16 stages fit beside a deep FP32 pipeline: TG2_STAGES steps of 128 x
 // 32 FP32 tiles of A and B in flight (plain row-major, 16 KB each), and two
@@ -320,24 +237,6 @@ constexpr int TG2_BF_TILE = TC_M * TG2_BK * 2;        // 8 KB
 constexpr int TG2_BF_STAGE = 4 * TG2_BF_TILE;         // A_hi, A_lo, B_hi, B_lo
 constexpr int TG2_SMEM_BYTES = TG2_STAGES * TG2_F32_STAGE + 2 * TG2_BF_STAGE + 1024;
 constexpr int TG2_VPT = (TC_M * TG2_BK / 4) / TC_THREADS;  // float4 per thread per tile
-
-// 64-byte swizzled K-major shared-memory descriptor (SBO = 512 B between
-// 8-row groups, version 1, layout type 4 = SWIZZLE_64B).
-__device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
-
-// Byte offset of BF16 element (row r, k) in a 64-byte swizzled K-major tile
-// of 32 columns (16-byte chunk c of row r at chunk c ^ ((r / 2) mod 4)).
-__device__ __forceinline__ uint32_t sw64_off(int r, int k) {
-    return (uint32_t)(r * 64 + ((((k >> 3) ^ (r >> 1)) & 3) << 4) + (k & 7) * 2);
-}
 
 template <bool ABS>
 __device__ __forceinline__ void split_tile32(const unsigned char* f32, unsigned char* hi_tile, unsigned char* lo_tile) {
@@ -382,38 +281,6 @@ constexpr int TW_THREADS = (TW_SPLIT_WARPS + 2) * 32;
 constexpr int TG2_DRAIN = 4;  // steps per accumulation period
 static_assert(TG2_DRAIN >= 2, "a period's drain follows the split of the next period's second step");
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Bounded wait that also gives up when *abort is set.
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, volatile int* abort) {
-    const uint32_t a = smem_u32(bar);
-    for (long long it = 0; it < TC_WAIT_LIMIT; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\n"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            "selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if ((it & 63) == 63 && *abort) return false;
-    }
-    *abort = 1;
-    return false;
-}
-
-// 16 FP32 accumulator columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* v) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr));
-}
-
 // Add one period's accumulator (32 columns at taddr) into the Kahan sums.
 // The compensations are kept as BF16 pairs (comp2[j] holds columns 2j and
 // 2j + 1): a compensation is below half an ulp of its sum, so its own 8-bit
@@ -437,22 +304,6 @@ __device__ __forceinline__ void drain_period(uint32_t taddr, float* fold, uint32
             fold[q + 1] = t1;
         }
     }
-}
-
-// Output tile of a CTA: tile_m fastest over all tiles, or, for a symmetric
-// product (A = B), the tiles on and above the diagonal only, column by column.
-__device__ __forceinline__ void gram_tile(int idx, int tiles_m, bool sym, int& tm, int& tn) {
-    if (!sym) {
-        tm = idx % tiles_m;
-        tn = idx / tiles_m;
-        return;
-    }
-    tn = 0;
-    while (idx > tn) {
-        idx -= tn + 1;
-        ++tn;
-    }
-    tm = idx;
 }
 
 template <bool ABS>
@@ -669,17 +520,6 @@ constexpr int CB_A_BYTES = TC_M * TC_BK * 2;   // 16 KB
 constexpr int CB_B_BYTES = CB_N * TC_BK * 2;   // 32 KB
 constexpr int CB_STAGE_BYTES = 2 * CB_A_BYTES + 2 * CB_B_BYTES;
 constexpr int CB_SMEM_BYTES = 2 * CB_STAGE_BYTES + 1024;
-constexpr uint32_t kIdescN256 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(CB_N >> 3) << 17) |
-                                ((uint32_t)(TC_M >> 4) << 24);
-
-__device__ __forceinline__ void mma_bf16_n256(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(kIdescN256), "r"(accumulate));
-}
-
 // hiT[n][k], loT[n][k] (BF16, rows of kpad, zero padded) from Coef[k][n] (FP64)
 __global__ void coef_split_kernel(int Kc, int N, const double* __restrict__ coef, int ldcoef, int kpad, int npad,
                                   __nv_bfloat16* __restrict__ hiT, __nv_bfloat16* __restrict__ loT) {
@@ -1033,46 +873,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }  // namespace
 
 namespace {
-
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// The driver's tensor-map encoder (through the runtime's entry-point query,
-// so no link against the driver library), or null.  LACE_TC_TMA=0 turns the
-// TMA-fed Gram kernel off (tuning: the register-staged kernel then runs).
-EncodeTiledFn encode_tiled() {
-    static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-        const char* e = getenv("LACE_TC_TMA");
-        if (e && e[0] == '0') return nullptr;
-        void* f = nullptr;
-        cudaDriverEntryPointQueryResult q{};
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return reinterpret_cast<EncodeTiledFn>(f);
-    }();
-    return fn;
-}
-
-// Tensor map of a row-major matrix [rows][cols] (row pitch ld elements of
-// esize bytes; 16-byte aligned base and pitch) in boxes of box_rows x
-// box_cols; reads outside the matrix return zeros.
-bool make_map(CUtensorMap* m, CUtensorMapDataType type, size_t esize, const void* base, size_t rows, size_t cols,
-              size_t ld, int box_cols, int box_rows, CUtensorMapSwizzle swz) {
-    const EncodeTiledFn enc = encode_tiled();
-    if (!enc || rows == 0 || cols == 0 || rows > 0xffffffffull || cols > 0xffffffffull) return false;
-    if (((uintptr_t)base % 16) || ((ld * esize) % 16)) return false;
-    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)(ld * esize)};
-    const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    const cuuint32_t estr[2] = {1, 1};
-    return enc(m, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
 
 // FP32 [rows][cols] in boxes of 128 rows x bk columns (the Gram's A and B tiles).
 bool make_tile_map(CUtensorMap* m, const float* base, size_t rows, size_t cols, size_t ld, int bk) {
