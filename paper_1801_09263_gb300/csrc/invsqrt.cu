@@ -7,17 +7,17 @@
 // One launch runs the whole iteration, its convergence test included: the
 // products are small (33 MFLOP at N = 256) and the launches, the elementwise
 // kernels between them and the host's waits for the norms were most of the time.
-// Up to 64 rows in FP32 (16 in FP64) one CTA keeps everything in shared memory;
-// beyond, a cooperative grid computes tiles and meets at a barrier after every
-// product.  The iterates are symmetric but for rounding, and yet all products
+// Up to 16 rows one CTA keeps everything in shared memory, up to 64 in FP32 a
+// cluster of eight does; beyond, a cooperative grid computes tiles and meets at a
+// barrier after every product.  The iterates are symmetric but for rounding, and yet all products
 // are computed whole and read as they stand: the iteration damps the errors of
 // Z Y, Y T and T Z alone.  With T mirrored from its upper triangle they grow by
 // sqrt(lambda_max / lambda_min) a step (FP32 X A X - I of 2e-2 instead of 6e-5 at N = 400
 // and 2.5e3); with Y and Z mirrored, or a transpose read in place of either, matrices of
 // 1e7 that converge do not.
 //
-// Measured (FP32, both inverse square roots of a step): kernels 2 x 226 us at
-// N = 256 and 2 x 139 us at N = 64; separate launches with their waits took 650 and 480 us.
+// Measured (FP32, both inverse square roots of a step, kernels alone): 440 us at
+// N = 256 and 114 us at N = 64; separate launches with their waits took 650 and 480 us.
 #include <algorithm>
 #include <cmath>
 
@@ -36,34 +36,36 @@ constexpr int kNsMaxCtas = 304;
 // rounding floor).  FP32: the same at 1e-11 N and 1e-6 N; and once below 1e-6 N
 // every |1 - x_k| < 0.016 and the iteration is in its quadratic regime
 // (1 - x -> ~(3/4)(1 - x)^2), so two more steps reach the floor.
+// h is summed in FP32 (FP64 runs at 1/64 of its rate, and a sum of the squares of
+// FP64 differences needs neither its digits nor its range).
 template <typename T> struct Stop {
-    double prev;
+    float prev;
     int extra;
     __device__ Stop() : prev(INFINITY), extra(-1) {}
     // the last of the two extra steps is done
     __device__ bool done() const { return extra == 0; }
     // 1: converged, 0: go on, -1: failed
-    __device__ int test(double h, int n) {
-        constexpr double lo = sizeof(T) == 8 ? 1e-24 : 1e-11, hi = sizeof(T) == 8 ? 1e-12 : 1e-6;
+    __device__ int test(float h, int n) {
+        constexpr float lo = sizeof(T) == 8 ? 1e-24f : 1e-11f, hi = sizeof(T) == 8 ? 1e-12f : 1e-6f;
         if (extra > 0) {
             --extra;
             return 0;
         }
         if (!(h < INFINITY)) return -1;
-        if (h < lo * n || (h < hi * n && h > 0.25 * prev)) return 1;
+        if (h < lo * n || (h < hi * n && h > 0.25f * prev)) return 1;
         if (sizeof(T) == 4 && h < hi * n) extra = 1;  // this step and one more
         prev = h;
         return 0;
     }
 };
 
-__device__ __forceinline__ double block_sum(double v, double* sh) {
+template <typename V> __device__ __forceinline__ V block_sum(V v, V* sh) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     __syncthreads();
     if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    double t = 0.0;
+    V t = V(0);
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
     return t;
 }
@@ -83,47 +85,24 @@ template <typename T, int NB> __device__ __forceinline__ void load_row(const T* 
     }
 }
 
-// C = A B of matrices in shared memory (rows of pitch P, zero past N), NB x NB
-// outputs a thread of 16 x 16 (rows ty + 16 i, columns NB tx + j); f(m, n, value)
-// for every output.
-template <typename T, int NB, int P, class F>
-__device__ __forceinline__ void one_product(int N, const T* A, const T* B, F f) {
-    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-    constexpr int KV = sizeof(T) == 4 ? 4 : 1;
-    T acc[NB][NB];
+// C = A B of matrices in shared memory (16 rows of pitch P, zero past N), one
+// output a thread; f(m, n, value) for every output.
+template <typename T, int P, class F> __device__ __forceinline__ void one_product(int N, const T* A, const T* B, F f) {
+    const int m = threadIdx.x >> 4, n = threadIdx.x & 15;
+    T acc = T(0);
 #pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) acc[i][j] = T(0);
-    for (int k = 0; k < N; k += KV) {
-        T a[NB][KV], b[KV][NB];
-#pragma unroll
-        for (int i = 0; i < NB; ++i) load_row<T, KV>(A + (ty + 16 * i) * P + k, a[i]);
-#pragma unroll
-        for (int q = 0; q < KV; ++q) load_row<T, NB>(B + (k + q) * P + NB * tx, b[q]);
-#pragma unroll
-        for (int q = 0; q < KV; ++q)
-#pragma unroll
-            for (int i = 0; i < NB; ++i)
-#pragma unroll
-                for (int j = 0; j < NB; ++j) acc[i][j] = fma(a[i][q], b[q][j], acc[i][j]);
-    }
-#pragma unroll
-    for (int i = 0; i < NB; ++i)
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-            const int m = ty + 16 * i, n = NB * tx + j;
-            if (m < N && n < N) f(m, n, acc[i][j]);
-        }
+    for (int k = 0; k < 16; ++k) acc = fma(A[m * P + k], B[k * P + n], acc);
+    if (m < N && n < N) f(m, n, acc);
 }
 
-template <typename T, int NB>
+template <typename T>
 __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double* __restrict__ A, double* __restrict__ X,
                                                             int* status) {
-    constexpr int R = 16 * NB, P = R + (sizeof(T) == 4 ? 4 : 1);
-    extern __shared__ double ns_smem[];
+    constexpr int R = 16, P = 17;
+    __shared__ T mats[5 * R * P];
     __shared__ double sh[kNsThreads / 32];
-    T* Y = reinterpret_cast<T*>(ns_smem);
+    __shared__ float shf[kNsThreads / 32];
+    T* Y = mats;
     T* Z = Y + R * P;
     T* W = Z + R * P;
     T* Y2 = W + R * P;
@@ -160,22 +139,21 @@ __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double*
             ok = true;
             break;
         }
-        double h = 0.0;
-        one_product<T, NB, P>(N, Z, Y, [&](int m, int n, T v) {
+        float h = 0.f;
+        one_product<T, P>(N, Z, Y, [&](int m, int n, T v) {
             const T d = m == n ? T(1) : T(0);
-            const double x = (double)(d - v);
-            h += x * x;
+            const float x = (float)(d - v);
+            h = fmaf(x, x, h);
             W[m * P + n] = T(0.5) * (T(2) * d + (d - v));  // (3 delta - v) / 2
         });
-        h = block_sum(h, sh);
+        h = block_sum(h, shf);
         const int st = stop.test(h, N);
         if (st != 0) {
             ok = st > 0;
             break;
         }
-        __syncthreads();
-        one_product<T, NB, P>(N, Y, W, [&](int m, int n, T v) { Y2[m * P + n] = v; });
-        one_product<T, NB, P>(N, W, Z, [&](int m, int n, T v) { Z2[m * P + n] = v; });
+        one_product<T, P>(N, Y, W, [&](int m, int n, T v) { Y2[m * P + n] = v; });
+        one_product<T, P>(N, W, Z, [&](int m, int n, T v) { Z2[m * P + n] = v; });
         __syncthreads();
         T* t = Y;
         Y = Y2;
@@ -198,6 +176,182 @@ __global__ void __launch_bounds__(kNsThreads) ns_one_kernel(int N, const double*
     if (tid == 0) *status = 1;
 }
 
+// ------------------------------------------------------------------ a cluster
+// 17 to 64 rows in FP32: eight CTAs with a copy of the iterates each compute
+// RB rows of a product and write them into all copies (distributed shared
+// memory); two cluster barriers a step.  One CTA took 139 us for a 64 x 64 of a 48^3
+// step (3.2 us a step at the FP32 peak of one SM), this takes 57: load and
+// localisation 0.71 -> 0.54 ms.  At 80 and 96 rows it is even with the grid (0.15 and
+// 0.16 ms a load).
+constexpr int kNsCluster = 8;
+template <int RB> struct NsCl {
+    static constexpr int R = kNsCluster * RB, P = R + 4;
+    static constexpr int KG = RB == 4 ? 8 : 4;  // groups of threads, each a part of K
+    static constexpr int UNITS = RB * RB, THREADS = UNITS * KG;  // 4 rows x 2 columns a thread
+    static constexpr int FLOATS = 4 * R * P + 2 * KG * RB * R;
+};
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The shared-memory address of p in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return r;
+}
+
+// Partial sums over this group's part of K of RB rows of A B -> red[group].
+template <int RB> __device__ __forceinline__ void cl_product(const float* A, const float* B, float* red) {
+    using C = NsCl<RB>;
+    const int group = threadIdx.x / C::UNITS, u = threadIdx.x % C::UNITS;
+    const int r0 = u / (C::R / 2) * 4, c0 = u % (C::R / 2) * 2;
+    float acc[4][2] = {};
+#pragma unroll 4
+    for (int k = group * (C::R / C::KG); k < (group + 1) * (C::R / C::KG); k += 4) {
+        float a[4][4], b[4][2];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) load_row<float, 4>(A + (r0 + i) * C::P + k, a[i]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) load_row<float, 2>(B + (k + q) * C::P + c0, b[q]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) acc[i][j] = fmaf(a[i][q], b[q][j], acc[i][j]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float2*>(red + (group * RB + r0 + i) * C::R + c0) = make_float2(acc[i][0], acc[i][1]);
+}
+// Four outputs of a row (e = 4-column group of RB x R) summed over the groups.
+template <int RB> __device__ __forceinline__ float4 cl_sum(const float* red, int e) {
+    using C = NsCl<RB>;
+    float4 s = *reinterpret_cast<const float4*>(red + 4 * e);
+#pragma unroll
+    for (int g = 1; g < C::KG; ++g) {
+        const float4 v = *reinterpret_cast<const float4*>(red + g * RB * C::R + 4 * e);
+        s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+    }
+    return s;
+}
+__device__ __forceinline__ void cl_put(float* at, float4 v) {
+#pragma unroll
+    for (int r = 0; r < kNsCluster; ++r)
+        asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(cluster_addr(at, r)), "f"(v.x), "f"(v.y), "f"(v.z),
+                     "f"(v.w)
+                     : "memory");
+}
+
+template <int RB>
+__global__ void __cluster_dims__(kNsCluster, 1, 1) __launch_bounds__(NsCl<RB>::THREADS)
+    ns_cluster_kernel(int N, const double* __restrict__ A, double* __restrict__ X, int* status) {
+    using C = NsCl<RB>;
+    constexpr int R = C::R, P = C::P, TH = C::THREADS;
+    extern __shared__ double ns_smem[];
+    __shared__ float sh[TH / 32 + 1];
+    __shared__ float part[kNsCluster];
+    __shared__ double rowsum[TH / 32 + 1];
+    float* Y = reinterpret_cast<float*>(ns_smem);
+    float* Z = Y + R * P;
+    float* Z2 = Z + R * P;
+    float* W = Z2 + R * P;
+    float* red = W + R * P;
+    float* red2 = red + C::KG * RB * R;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rank = (int)cluster_rank(), m0 = rank * RB;
+    // c = largest row sum (every CTA for itself)
+    double c = 0.0;
+    for (int r = warp; r < N; r += TH / 32) {
+        double s = 0.0;
+        for (int k = lane; k < N; k += 32) s += fabs(A[(size_t)r * N + k]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        c = s > c || s != s ? s : c;
+    }
+    if (lane == 0) rowsum[warp] = c;
+    __syncthreads();
+    c = 0.0;
+    for (int w = 0; w < TH / 32; ++w) c = rowsum[w] > c || rowsum[w] != rowsum[w] ? rowsum[w] : c;
+    const bool run = c > 0.0 && c < INFINITY;  // (alike in all CTAs)
+    const double ci = run ? 1.0 / c : 0.0;
+    for (int e = tid; e < 3 * R * P; e += TH) Y[e] = 0.f;
+    __syncthreads();
+    for (int e = tid; e < N * N; e += TH) {
+        const int r = e / N, k = e % N;
+        Y[r * P + k] = (float)(0.5 * (A[e] + A[(size_t)k * N + r]) * ci);
+        if (r == k) Z[r * P + k] = 1.f;
+    }
+    cluster_barrier();  // all copies are set up
+    Stop<float> stop;
+    bool ok = false;
+    if (run)
+        for (int it = 0; it < kNsMaxIt; ++it) {
+            if (stop.done()) {
+                ok = true;
+                break;
+            }
+            cl_product<RB>(Z + m0 * P, Y, red);
+            __syncthreads();
+            float h = 0.f;
+            for (int e = tid; e < RB * R / 4; e += TH) {
+                const int m = m0 + 4 * e / R, n = 4 * e % R;
+                const float4 v = cl_sum<RB>(red, e);
+                float4 t;
+                auto one = [&](float v1, int col) {
+                    const float d = m == col ? 1.f : 0.f, x = m < N && col < N ? d - v1 : 0.f;
+                    h = fmaf(x, x, h);
+                    return m < N && col < N ? 0.5f * (2.f * d + x) : 0.f;  // (3 delta - v) / 2
+                };
+                t.x = one(v.x, n), t.y = one(v.y, n + 1), t.z = one(v.z, n + 2), t.w = one(v.w, n + 3);
+                cl_put(W + m * P + n, t);
+            }
+            h = block_sum(h, sh);
+            if (tid < kNsCluster)
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(part + rank, tid)), "f"(h) : "memory");
+            cluster_barrier();
+            h = 0.f;
+#pragma unroll
+            for (int r = 0; r < kNsCluster; ++r) h += part[r];  // a fixed order: every CTA decides alike
+            const int st = stop.test(h, N);
+            if (st != 0) {
+                ok = st > 0;
+                break;
+            }
+            cl_product<RB>(Y + m0 * P, W, red);
+            cl_product<RB>(W + m0 * P, Z, red2);
+            __syncthreads();  // (Y's own rows are read: the other CTAs read no rows of this one's now)
+            for (int e = tid; e < RB * R / 4; e += TH) {
+                const int at = (m0 + 4 * e / R) * P + 4 * e % R;
+                cl_put(Y + at, cl_sum<RB>(red, e));
+                cl_put(Z2 + at, cl_sum<RB>(red2, e));
+            }
+            cluster_barrier();
+            float* t = Z;
+            Z = Z2;
+            Z2 = t;
+        }
+    // ||(A/c)^{-1/2}||_F^2 >= lambda_max / lambda_min: reject ill-conditioned A
+    float f = 0.f;
+    const double s = 1.0 / sqrt(c);
+    for (int e = tid; e < N * N; e += TH) {
+        const float z = 0.5f * (Z[(e / N) * P + e % N] + Z[(e % N) * P + e / N]);
+        f = fmaf(z, z, f);
+    }
+    f = block_sum(f, sh);
+    ok = ok && f < 1e12f;
+    if (ok)
+        for (int e = rank * TH + tid; e < N * N; e += kNsCluster * TH)
+            X[e] = s * 0.5 * ((double)Z[(e / N) * P + e % N] + (double)Z[(e % N) * P + e / N]);
+    if (rank == 0 && tid == 0) *status = ok ? 1 : 0;
+    cluster_barrier();  // no CTA leaves while its memory may be written
+}
+
 // ------------------------------------------------------------------ a grid
 // Tile sizes: FP32 16 x 16 outputs, 2 x 2 a thread; FP64 8 x 8, one a thread.
 // Four groups of 64 threads take a quarter of K each.
@@ -214,7 +368,7 @@ template <typename T> struct NsArgs {
     const double* A;
     double* X;
     T *Y, *Z, *W, *Y2, *Z2;    // N rows of ld
-    double* part;              // one a CTA
+    float* part;               // one a CTA
     unsigned* bar;             // 4, zero at launch
     unsigned long long* norm;  // zero at launch
     int* status;               // 1 converged, 0 failed, -1 a barrier wait ran out (preset)
@@ -293,7 +447,7 @@ template <typename T>
 __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     using C = NsTile<T>;
     __shared__ __align__(16) T smem[C::S * (C::P + C::KC) + 4 * C::S * C::S];
-    __shared__ double sh[kNsThreads / 32];
+    __shared__ float sh[kNsThreads / 32];
     __shared__ int abort_sh;
     unsigned gen = 0;
     const int N = a.N, ld = a.ld, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -333,7 +487,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     auto put = [&](T* M, int m, int n, T v) { __stcg(M + (size_t)m * ld + n, v); };
     // sum over the CTAs in a fixed order: every CTA decides alike
     auto total = [&]() {
-        double s = 0.0;
+        float s = 0.f;
         if (warp == 0) {
             for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + b);
 #pragma unroll
@@ -353,12 +507,12 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
             break;
         }
         if (it > 0) {
-            double h = 0.0;
+            float h = 0.f;
             for (int t = blockIdx.x; t < tiles; t += gridDim.x)
                 grid_product<T>(N, ld, Z, Y, t / nt, t % nt, smem, [&](int m, int n, T v) {
                     const T d = m == n ? T(1) : T(0);
-                    const double x = (double)(d - v);
-                    h += x * x;
+                    const float x = (float)(d - v);
+                    h = fmaf(x, x, h);
                     put(a.W, m, n, T(0.5) * (T(2) * d + (d - v)));
                 });
             h = block_sum(h, sh);
@@ -384,30 +538,26 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         Z2 = t;
     }
     // ||(A/c)^{-1/2}||_F^2 >= lambda_max / lambda_min: reject ill-conditioned A
-    double f = 0.0;
+    float f = 0.f;
     const double s = 1.0 / sqrt(c);
     for (size_t e = me; e < (size_t)N * N; e += all) {
         const double z = 0.5 * ((double)__ldcg(Z + (e / N) * ld + e % N) + (double)__ldcg(Z + (e % N) * ld + e / N));
-        f += z * z;
+        f = fmaf((float)z, (float)z, f);
         if (ok) a.X[e] = s * z;
     }
     f = block_sum(f, sh);
     if (tid == 0) __stcg(a.part + blockIdx.x, f);
     if (!grid_barrier(a.bar, gen, &abort_sh)) return;
     f = total();
-    if (me == 0) *a.status = ok && f < 1e12 ? 1 : 0;
+    if (me == 0) *a.status = ok && f < 1e12f ? 1 : 0;
 }
 
-template <typename T, int NB>
-cudaError_t ns_one(int N, const double* A, double* X, int* d_status, cudaStream_t s) {
-    constexpr int R = 16 * NB, P = R + (sizeof(T) == 4 ? 4 : 1);
-    constexpr size_t sm = 5 * sizeof(T) * R * P;
-    const void* fn = (const void*)ns_one_kernel<T, NB>;
-    if (sm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e) return e;
-    }
-    ns_one_kernel<T, NB><<<1, kNsThreads, sm, s>>>(N, A, X, d_status);
+template <int RB> cudaError_t ns_cluster(int N, const double* A, double* X, int* d_status, cudaStream_t s) {
+    using C = NsCl<RB>;
+    constexpr size_t sm = C::FLOATS * sizeof(float);
+    cudaError_t e = cudaFuncSetAttribute((const void*)ns_cluster_kernel<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e) return e;
+    ns_cluster_kernel<RB><<<kNsCluster, C::THREADS, sm, s>>>(N, A, X, d_status);
     return cudaGetLastError();
 }
 
@@ -422,12 +572,13 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, c
     int* d_status = reinterpret_cast<int*>(ctl);
     cudaError_t e;
     int h = 0;
-    const bool one = sizeof(T) == 4 ? N <= 64 : N <= 16;
-    if (one) {
-        if (sizeof(T) == 8 || N <= 16) e = ns_one<T, 1>(N, A, X, d_status, s);
-        else if (N <= 32) e = ns_one<float, 2>(N, A, X, d_status, s);
-        else if (N <= 48) e = ns_one<float, 3>(N, A, X, d_status, s);
-        else e = ns_one<float, 4>(N, A, X, d_status, s);
+    const bool small = N <= (sizeof(T) == 4 ? 64 : 16);
+    if (small) {
+        if (N <= 16) {
+            ns_one_kernel<T><<<1, kNsThreads, 0, s>>>(N, A, X, d_status);
+            e = cudaGetLastError();
+        } else if (N <= 32) e = ns_cluster<4>(N, A, X, d_status, s);
+        else e = ns_cluster<8>(N, A, X, d_status, s);
         if (e) return e;
     } else {
         if ((e = cudaMemsetAsync(ctl, 0xff, sizeof(int), s))) return e;        // status -1
@@ -445,7 +596,7 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, c
         a.status = d_status;
         a.bar = reinterpret_cast<unsigned*>(ctl + 16);
         a.norm = reinterpret_cast<unsigned long long*>(ctl + 32);
-        a.part = reinterpret_cast<double*>(ctl + 64);
+        a.part = reinterpret_cast<float*>(ctl + 64);
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
