@@ -25,20 +25,20 @@
 // square root's), localised 2.3e-7, 1.9e-7 -> 6e-8, 6e-8; orbitals rotated 4.1e-7 -> 7e-8.
 //
 // Kernels: the warp-role Gram of tc_gemm.cu with nine products (diagonal tiles load
-// and cut their rows once), and a rotation persistent over tiles of 128 points x
-// 128 targets, 32 orbitals a step, with A's slices in TMEM: from shared memory both
+// and cut their rows once), and combine_ws_kernel of tc_combine.cuh with three
+// accumulators of 128 targets: A's slices are in TMEM, since from shared memory both
 // operands of a 128 x 128 tile take all its bandwidth, and the cut's writes come on top.
 //
 // Measured, 72^3 x 256 (launches, alone): Gram 1043 -> 271 us (nine products over
 // three tiles of four: 165 us at the dense FP16 rate; bound by shared memory:
 // operands, rows and slices are 1.9k of its 128-byte cycles a step of 1.1 us),
-// rotation 653 -> 243 us (196 us at the FP16 rate; 420 us with a CTA-wide barrier a
-// step and A's slices in shared memory).  Row maxima come with the rounding to FP32.
+// rotation 653 -> 225 us (196 us at the FP16 rate).  Row maxima come with the rounding to FP32.
 #include <algorithm>
 #include <atomic>
 
 #include "f32x2.cuh"
 #include "lace_internal.cuh"
+#include "tc_combine.cuh"
 #include "tc_util.cuh"
 
 #include <cuda_fp16.h>
@@ -58,14 +58,6 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(kIdescF16), "r"(accumulate));
 }
-// The same with A in TMEM (a point a lane, two orbitals a 32-bit column).
-__device__ __forceinline__ void mma_f16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(tmem_d),
-        "r"(tmem_a), "l"(bdesc), "r"(kIdescF16), "r"(accumulate));
-}
 // The products by order into accumulators of 128 columns; mma(acc, i, j, first)
 // multiplies slices a_i b_j.  GRAM: all nine, a2 b2 apart from the low ones.
 template <bool GRAM, class Mma> __device__ __forceinline__ void mma_orders(uint32_t acc, uint32_t first, Mma mma) {
@@ -79,12 +71,6 @@ template <bool GRAM, class Mma> __device__ __forceinline__ void mma_orders(uint3
     mma(low, 1, 2, 1u);
     mma(low, 2, 1, 1u);
     if (GRAM) mma(low, 2, 2, 1u);
-}
-// 8 FP32 accumulator columns of this warp's 32 TMEM lanes.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
-                 : "r"(taddr));
 }
 // Two FP32 values rounded to FP16, x0 in the low half.
 __device__ __forceinline__ uint32_t f16x2_rn(float x0, float x1) {
@@ -354,15 +340,7 @@ __global__ void __launch_bounds__(GX_THREADS, 1)
 }
 
 // ------------------------------------------------------------------ rotation
-constexpr int CX_N = TC_N, CX_BK = 32, CX_BSTAGES = 4, CX_ASTAGES = 5, CX_CUT_WARPS = 16;
-constexpr int CX_THREADS = CX_CUT_WARPS * 32 + 64;
-constexpr int CX_A32_BYTES = CX_BK * TC_M * 4;              // 16 KB: 32 orbitals x 128 points
-constexpr int CX_B_TILE = CX_N * CX_BK * 2, CX_B_BYTES = 3 * CX_B_TILE;  // 24 KB: three slices of 128 targets
-constexpr int CX_SMEM_BYTES = CX_BSTAGES * CX_B_BYTES + CX_ASTAGES * CX_A32_BYTES + 1024;
-// TMEM columns: three accumulators, then two stages of A's slices
-constexpr int CX_A_COLS = CX_BK / 2, CX_A_AT = 3 * CX_N, CX_A_STAGE = 3 * CX_A_COLS;
-static_assert(CX_SMEM_BYTES <= 227 * 1024 - 256, "one CTA an SM");
-static_assert(CX_A_AT + 2 * CX_A_STAGE <= 512 && CX_BK == 8 * (CX_CUT_WARPS / 4), "TMEM columns; 8 orbitals a thread");
+constexpr int CX_N = TC_N;
 
 // Slices of the coefficients, [slice][npad][kpad] FP16 (targets by rows, zero
 // padded): column n of coef[k][n] 2^-e_k (the rows of A are scaled by 2^e_k),
@@ -403,204 +381,16 @@ __global__ void coef_cut_kernel(int Kc, int N, const double* __restrict__ coef, 
     }
 }
 
-__device__ __forceinline__ void tmem_st4(uint32_t taddr, const uint32_t* v) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-                 "r"(v[3])
-                 : "memory");
-}
-
-// Warp roles: warps 0-15 cut the FP32 rows into A's slices in TMEM (warp w: points
-// 32 (w % 4).., orbitals 8 (w / 4).. of a step) and write the results, warp 16
-// copies, warp 17 issues the MMAs.  Hand-offs by mbarriers: full_a/full_b
-// (copies landed), empty_a (a stage of rows is cut), cut_bar (slices are in TMEM), mma_bar
-// (the MMAs are done with a slice stage), empty_b (and with their coefficients),
-// drained_bar (a tile's sums are in registers; its stores run under the next tile's MMAs).
-__global__ void __launch_bounds__(CX_THREADS, 1)
-    combine_exact_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_c, int N, size_t K,
-                         int kpad, int npad, const float* __restrict__ scale_a, const float* __restrict__ scale_out, bool add,
-                         float* __restrict__ Out, size_t ldo, int* __restrict__ err) {
-    extern __shared__ unsigned char tc_smem_raw[];
-    __shared__ uint64_t full_a[CX_ASTAGES], empty_a[CX_ASTAGES], full_b[CX_BSTAGES], empty_b[CX_BSTAGES];
-    __shared__ uint64_t cut_bar[2], mma_bar[2], drained_bar;
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ volatile int abort_sh;
-    __shared__ int last_a[CX_ASTAGES], last_b[CX_BSTAGES];
-    unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* bst = smem;                           // coefficient slices
-    unsigned char* a32 = bst + CX_BSTAGES * CX_B_BYTES;  // FP32 rows
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nsteps = kpad / CX_BK;
-    const int rtiles = (int)((K + TC_M - 1) / TC_M), ntiles = npad / CX_N;
-    const long long tiles = (long long)rtiles * ntiles;
-    const int my_tiles = (int)((tiles - 1 - (long long)blockIdx.x) / (int)gridDim.x + 1);  // gridDim.x <= tiles
-    const int total = my_tiles * nsteps;  // this CTA's steps over all its tiles
-    // step g is orbital step g % nsteps of tile g / nsteps of this CTA (targets
-    // fastest: the tiles of the same points run side by side)
-    auto tile_of_step = [&](int g, int& rt, int& nt) {
-        const long long tile = (long long)blockIdx.x + (long long)(g / nsteps) * (int)gridDim.x;
-        rt = (int)(tile / ntiles);
-        nt = (int)(tile % ntiles);
-    };
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < CX_ASTAGES; ++s) {
-            mbar_init(&full_a[s], 1);
-            mbar_init(&empty_a[s], CX_CUT_WARPS);
-            last_a[s] = -1;
-        }
-        for (int s = 0; s < CX_BSTAGES; ++s) {
-            mbar_init(&full_b[s], 1);
-            mbar_init(&empty_b[s], 1);
-            last_b[s] = -1;
-        }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(&cut_bar[s], CX_CUT_WARPS);
-            mbar_init(&mma_bar[s], 1);
-        }
-        mbar_init(&drained_bar, CX_CUT_WARPS);
-        abort_sh = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+// Three FP16 slices, their eight products by order in three accumulators.
+struct ExactSlices {
+    static constexpr int SLICES = 3, ACCS = 3;
+    static constexpr bool SCALED = true;
+    static constexpr uint32_t FORMAT = 0;  // F16
+    static __device__ __forceinline__ void cut(f2 x, uint32_t* s) { cut2(x, s[0], s[1], s[2]); }
+    template <class Mma> static __device__ __forceinline__ void products(uint32_t acc, uint32_t first, Mma mma) {
+        mma_orders<false>(acc, first, mma);
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_sh)),
-                     "r"(512)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base_sh;
-    int committed = 0;  // MMA thread: steps committed
-
-    if (warp == CX_CUT_WARPS) {
-        if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_c)) : "memory");
-            for (int g = 0; g < total; ++g) {
-                const int sa = g % CX_ASTAGES, sb = g % CX_BSTAGES;
-                int rt, nt;
-                tile_of_step(g, rt, nt);
-                if (g >= CX_ASTAGES && !mbar_wait_or_abort(&empty_a[sa], (uint32_t)(g / CX_ASTAGES - 1) & 1, &abort_sh)) break;
-                mbar_expect_tx(&full_a[sa], CX_A32_BYTES);
-                tma_load_2d(a32 + sa * CX_A32_BYTES, &map_a, rt * TC_M, (g % nsteps) * CX_BK, &full_a[sa]);
-                last_a[sa] = g;
-                if (g >= CX_BSTAGES && !mbar_wait_or_abort(&empty_b[sb], (uint32_t)(g / CX_BSTAGES - 1) & 1, &abort_sh)) break;
-                mbar_expect_tx(&full_b[sb], CX_B_BYTES);
-#pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    tma_load_2d(bst + sb * CX_B_BYTES + q * CX_B_TILE, &map_c, (g % nsteps) * CX_BK, q * npad + nt * CX_N,
-                                &full_b[sb]);
-                last_b[sb] = g;
-            }
-        }
-    } else if (warp == CX_CUT_WARPS + 1) {
-        if (lane == 0) {
-            for (int g = 0; g < total; ++g) {
-                const int b = g & 1, sb = g % CX_BSTAGES, step = g % nsteps;
-                if (!mbar_wait_or_abort(&full_b[sb], (uint32_t)(g / CX_BSTAGES) & 1, &abort_sh) ||
-                    !mbar_wait_or_abort(&cut_bar[b], (uint32_t)(g >> 1) & 1, &abort_sh))
-                    break;
-                // a tile starts once the last one's sums are read
-                if (g > 0 && step == 0 && !mbar_wait_or_abort(&drained_bar, (uint32_t)(g / nsteps - 1) & 1, &abort_sh)) break;
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t a = tmem + CX_A_AT + b * CX_A_STAGE, bb = smem_u32(bst + sb * CX_B_BYTES);
-#pragma unroll
-                for (int kk = 0; kk < CX_BK / 16; ++kk)
-                    mma_orders<false>(tmem, (step == 0 && kk == 0) ? 0u : 1u, [&](uint32_t acc, int i, int j, uint32_t first) {
-                        mma_f16_ta(acc, a + i * CX_A_COLS + kk * 8, sw64_desc(bb + kk * 32 + j * CX_B_TILE), first);
-                    });
-                mma_commit(&mma_bar[b]);
-                mma_commit(&empty_b[sb]);
-                committed = g + 1;
-            }
-        }
-    } else {
-        const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
-        const int ar = (warp & 3) * 32 + lane, kq = (warp >> 2) * 8, cb = (warp >> 2) * 32;
-        // the sums of the tile that ends with step g -> Out (32 targets of one point a thread)
-        auto finish_tile = [&](int g, bool more) {
-            if (!mbar_wait_or_abort(&mma_bar[g & 1], (uint32_t)(g >> 1) & 1, &abort_sh)) return false;
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float x[32];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-                uint32_t v[3][8];
-#pragma unroll
-                for (int o = 0; o < 3; ++o) tmem_ld8(tlane + o * CX_N + cb + 8 * h, v[o]);
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-                    x[8 * h + j] = __uint_as_float(v[0][j]) + (__uint_as_float(v[1][j]) + __uint_as_float(v[2][j]));
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (more && lane == 0) mbar_arrive(&drained_bar);
-            int rt, nt;
-            tile_of_step(g, rt, nt);
-            const size_t r = (size_t)rt * TC_M + ar;
-            const int n0 = nt * CX_N + cb;
-            if (r < K) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (n0 + j < N) {
-                        float* o = Out + (size_t)(n0 + j) * ldo + r;
-                        const float y = x[j] * __ldg(scale_out + n0 + j);
-                        *o = add ? *o + y : y;
-                    }
-            }
-            return true;
-        };
-        bool ok = true;
-        for (int g = 0; g < total; ++g) {
-            const int sa = g % CX_ASTAGES, b = g & 1, step = g % nsteps;
-            const float4 c0 = __ldg(reinterpret_cast<const float4*>(scale_a + step * CX_BK + kq));
-            const float4 c1 = __ldg(reinterpret_cast<const float4*>(scale_a + step * CX_BK + kq + 4));
-            if (!mbar_wait_or_abort(&full_a[sa], (uint32_t)(g / CX_ASTAGES) & 1, &abort_sh)) { ok = false; break; }
-            // the MMAs of step g - 2 are done with slice stage b
-            if (g >= 2 && !mbar_wait_or_abort(&mma_bar[b], (uint32_t)((g >> 1) - 1) & 1, &abort_sh)) { ok = false; break; }
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const float* src = reinterpret_cast<const float*>(a32 + sa * CX_A32_BYTES) + kq * TC_M + ar;
-            uint32_t s1[4], s2[4], s3[4];
-            cut2(mk2(src[0 * TC_M], src[1 * TC_M]) * mk2(c0.x, c0.y), s1[0], s2[0], s3[0]);
-            cut2(mk2(src[2 * TC_M], src[3 * TC_M]) * mk2(c0.z, c0.w), s1[1], s2[1], s3[1]);
-            cut2(mk2(src[4 * TC_M], src[5 * TC_M]) * mk2(c1.x, c1.y), s1[2], s2[2], s3[2]);
-            cut2(mk2(src[6 * TC_M], src[7 * TC_M]) * mk2(c1.z, c1.w), s1[3], s2[3], s3[3]);
-            const uint32_t ta = tlane + CX_A_AT + b * CX_A_STAGE + (warp >> 2) * 4;
-            tmem_st4(ta, s1);
-            tmem_st4(ta + CX_A_COLS, s2);
-            tmem_st4(ta + 2 * CX_A_COLS, s3);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&empty_a[sa]);
-                mbar_arrive(&cut_bar[b]);
-            }
-            // the tile before (this step's slices are written: only its MMAs wait)
-            if (g > 0 && step == 0 && !finish_tile(g - 1, true)) { ok = false; break; }
-        }
-        if (ok) finish_tile(total - 1, false);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (abort_sh) {
-        // copies still landing, MMAs still running (bounded waits)
-        if (warp == CX_CUT_WARPS && lane == 0) {
-            for (int s = 0; s < CX_ASTAGES; ++s)
-                if (last_a[s] >= 0) mbar_wait(&full_a[s], (uint32_t)(last_a[s] / CX_ASTAGES) & 1);
-            for (int s = 0; s < CX_BSTAGES; ++s)
-                if (last_b[s] >= 0) mbar_wait(&full_b[s], (uint32_t)(last_b[s] / CX_BSTAGES) & 1);
-        }
-        if (warp == CX_CUT_WARPS + 1 && lane == 0 && committed > 0)
-            mbar_wait(&mma_bar[(committed - 1) & 1], (uint32_t)((committed - 1) >> 1) & 1);
-        if (threadIdx.x == 0) atomicExch(err, 1);
-    }
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-    }
-}
+};
 
 // ------------------------------------------------------------------ row maxima
 // out[row] = bits of the largest |x| of the row (zeroed before); Tin = double:
@@ -718,7 +508,7 @@ cudaError_t gram_exact(int M, int N, size_t K, const float* A, const unsigned* m
 }
 
 size_t combine_exact_scratch_bytes(int N, int Kc) {
-    const size_t kpad = ((size_t)Kc + CX_BK - 1) / CX_BK * CX_BK, npad = ((size_t)N + CX_N - 1) / CX_N * CX_N;
+    const size_t kpad = ((size_t)Kc + CW_BK - 1) / CW_BK * CW_BK, npad = ((size_t)N + CX_N - 1) / CX_N * CX_N;
     return 3 * kpad * npad * sizeof(__half) + (npad + kpad) * sizeof(float);
 }
 
@@ -726,14 +516,14 @@ cudaError_t combine_exact(int N, size_t K, int Kc, const float* A, const unsigne
                           bool add, float* Out, size_t ldo, void* scratch, int* d_err, cudaStream_t s, int* launches) {
     if (N <= 0 || K == 0) return cudaSuccess;
     if (!exact_ok(K, A) || Kc <= 0) return cudaErrorInvalidValue;
-    const int kpad = (Kc + CX_BK - 1) / CX_BK * CX_BK, npad = (N + CX_N - 1) / CX_N * CX_N;
+    const int kpad = (Kc + CW_BK - 1) / CW_BK * CW_BK, npad = (N + CX_N - 1) / CX_N * CX_N;
     __half* slices = static_cast<__half*>(scratch);
     float* scale_a = reinterpret_cast<float*>(slices + (size_t)3 * kpad * npad);
     float* scale_out = scale_a + kpad;
     CUtensorMap map_a, map_c;
-    if (!make_map(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), A, (size_t)Kc, K, K, TC_M, CX_BK,
+    if (!make_map(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), A, (size_t)Kc, K, K, TC_M, CW_BK,
                   CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !make_map(&map_c, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, slices, (size_t)3 * npad, (size_t)kpad, (size_t)kpad, CX_BK, CX_N,
+        !make_map(&map_c, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, slices, (size_t)3 * npad, (size_t)kpad, (size_t)kpad, CW_BK, CX_N,
                   CU_TENSOR_MAP_SWIZZLE_64B))
         return cudaErrorInvalidValue;
     static std::atomic<unsigned long long> attr_done{0};
@@ -742,15 +532,15 @@ cudaError_t combine_exact(int N, size_t K, int Kc, const float* A, const unsigne
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaError_t e;
     if (dev >= 64 || !(attr_done.load() & (1ull << dev))) {
-        if ((e = cudaFuncSetAttribute(combine_exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CX_SMEM_BYTES))) return e;
+        if ((e = cudaFuncSetAttribute(combine_ws_kernel<ExactSlices, CX_N, float>, cudaFuncAttributeMaxDynamicSharedMemorySize, CombineShape<ExactSlices, CX_N>::SMEM))) return e;
         if (dev < 64) attr_done.fetch_or(1ull << dev);
     }
     if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s))) return e;
     coef_cut_kernel<<<npad, 128, 0, s>>>(Kc, N, Coef, ldcoef, kpad, npad, max_a, slices, scale_a, scale_out);
-    const long long tiles = (long long)((K + TC_M - 1) / TC_M) * (npad / CX_N);
-    const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>(tiles, sms));
-    combine_exact_kernel<<<grid, CX_THREADS, CX_SMEM_BYTES, s>>>(map_a, map_c, N, K, kpad, npad, scale_a, scale_out, add, Out, ldo,
-                                                                 d_err);
+    bool resident;
+    const unsigned grid = combine_grid<ExactSlices, CX_N>(K, kpad, npad, sms, &resident);
+    combine_ws_kernel<ExactSlices, CX_N, float><<<grid, CW_THREADS, CombineShape<ExactSlices, CX_N>::SMEM, s>>>(
+        map_a, map_c, N, K, kpad, npad, scale_a, scale_out, resident, add ? 1.f : 0.f, Out, ldo, d_err);
     *launches += 2;
     return cudaGetLastError();
 }

@@ -17,10 +17,8 @@
 //   copies; the roles hand off through mbarriers.  The MMAs accumulate a few
 //   steps per TMEM accumulator (two alternating), which the split warps drain
 //   into compensated FP32 sums.
-// * tc_combine_tma_kernel (the combination, default): persistent over output
-//   tiles of 128 grid points x 256 targets; the FP32 A tiles and the pre-split
-//   coefficient tiles arrive by TMA (the latter directly in the 128-byte
-//   swizzled layout), the threads transpose-split A; FP32 or FP64 output.
+// * combine_ws_kernel of tc_combine.cuh (the combination, default): persistent over
+//   output tiles of 128 grid points x 128 or 256 targets; FP32 or FP64 output.
 // * tc_gram_kernel / tc_combine_kernel: the same contractions with the
 //   operands loaded through registers (used when no tensor map can be made).
 // Every mbarrier wait is bounded; on a timeout the CTA records an error,
@@ -34,6 +32,7 @@
 #include <algorithm>
 
 #include "lace_internal.cuh"
+#include "tc_combine.cuh"
 #include "tc_util.cuh"
 
 namespace lace {
@@ -671,204 +670,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
-// The combination with its operands brought in by the Tensor Memory
-// Accelerator, persistent over output tiles: each CTA takes tiles (128 grid
-// points x 256 targets) round-robin and runs their 64-orbital steps as one
-// pipeline of TC_STAGES-deep copies: per step, the FP32 A tile [64 k][128 r]
-// (row-major, rows past Kc and columns past K arrive as zeros) and the
-// pre-split Coef^T hi/lo tiles [256 n][64 k], which TMA writes directly in
-// the 128-byte swizzled K-major layout the MMA reads.  All 512 threads
-// transpose-split A into the BF16 hi/lo tiles (one BF16 stage: the split of a
-// step waits for the MMAs of the step before, and a stage's copies are
-// replaced only after its MMAs are done); after a tile's last MMA all 16
-// warps read the accumulators (warp w: lanes 32 (w % 4).., columns 64 (w / 4)..)
-// and write Out.  Bounded waits throughout; on a timeout the CTA records an
-// error, waits (bounded) for its copies and MMAs in flight, frees its tensor
-// memory and returns.
-constexpr int CT_STAGES = 2;
-constexpr int CT_A32_BYTES = TC_BK * TC_M * 4;                 // 32 KB: 64 k x 128 r FP32
-constexpr int CT_STAGE_BYTES = CT_A32_BYTES + 2 * CB_B_BYTES;  // + Coef^T hi, lo (32 KB each)
-constexpr int CT_SMEM_BYTES = CT_STAGES * CT_STAGE_BYTES + 2 * CB_A_BYTES + 1024;
-
-template <typename TO>
-__global__ void __launch_bounds__(TC_THREADS, 1)
-    tc_combine_tma_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_hi,
-                          const __grid_constant__ CUtensorMap map_lo, int N, size_t K, int kpad, float beta,
-                          TO* __restrict__ Out, size_t ldo, int* __restrict__ err) {
-    extern __shared__ unsigned char tc_smem_raw[];
-    __shared__ uint64_t full[CT_STAGES];
-    __shared__ uint64_t mma_bar;
-    __shared__ uint32_t tmem_base_sh;
-    __shared__ int abort_sh;
-    unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
-    unsigned char* abf = smem + CT_STAGES * CT_STAGE_BYTES;  // A^T hi, lo (swizzled K-major, 128 rows r)
-    const int warp = threadIdx.x >> 5;
-    const int nsteps = kpad / TC_BK;
-    const int rtiles = (int)((K + TC_M - 1) / TC_M), ntiles = (N + CB_N - 1) / CB_N;
-    const int tiles = rtiles * ntiles;
-    const int my_tiles = blockIdx.x < tiles ? (tiles - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
-    const int total = my_tiles * nsteps;  // this CTA's steps over all its tiles
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < CT_STAGES; ++s) mbar_init(&full[s], 1);
-        mbar_init(&mma_bar, 1);
-        abort_sh = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_a)) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_hi)) : "memory");
-        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&map_lo)) : "memory");
+// The combination's slices for combine_ws_kernel (tc_combine.cuh).
+struct Bf16Slices {
+    static constexpr int SLICES = 2, ACCS = 1;
+    static constexpr bool SCALED = false;
+    static constexpr uint32_t FORMAT = 1;  // BF16
+    static __device__ __forceinline__ void cut(f2 x, uint32_t* s) {
+        float a, b;
+        unpk2(x, a, b);
+        s[0] = bf16x2_rn(a, b);
+        s[1] = bf16x2_rn(a - __uint_as_float(s[0] << 16), b - __uint_as_float(s[0] & 0xffff0000u));
     }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_u32(&tmem_base_sh)),
-                     "r"(CB_N)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    template <class Mma> static __device__ __forceinline__ void products(uint32_t acc, uint32_t first, Mma mma) {
+        mma(acc, 0, 0, first);
+        mma(acc, 0, 1, 1u);
+        mma(acc, 1, 0, 1u);
     }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_base_sh;
-
-    // thread 0: global step g (tile g / nsteps of this CTA, orbital step g % nsteps) into stage g % CT_STAGES
-    int issued = 0;
-    auto issue = [&](int g) {
-        const int s = g % CT_STAGES;
-        const int tile = (int)blockIdx.x + (g / nsteps) * (int)gridDim.x;
-        const int rt = tile % rtiles, nt = tile / rtiles;
-        const int k0 = (g % nsteps) * TC_BK;
-        unsigned char* st = smem + s * CT_STAGE_BYTES;
-        mbar_expect_tx(&full[s], CT_STAGE_BYTES);
-        tma_load_2d(st, &map_a, rt * TC_M, k0, &full[s]);
-        tma_load_2d(st + CT_A32_BYTES, &map_hi, k0, nt * CB_N, &full[s]);
-        tma_load_2d(st + CT_A32_BYTES + CB_B_BYTES, &map_lo, k0, nt * CB_N, &full[s]);
-    };
-    if (threadIdx.x == 0)
-        for (; issued < CT_STAGES && issued < total; ++issued) issue(issued);
-    // this thread's transpose-split share: grid point ar, k quads aq + 4j
-    const int ar = threadIdx.x & (TC_M - 1), aq = threadIdx.x >> 7;
-    int g = 0, committed = 0;
-    for (; g < total; ++g) {
-        const int s = g % CT_STAGES, step = g % nsteps;
-        bool ok = mbar_wait(&full[s], (uint32_t)(g / CT_STAGES) & 1);
-        if (g > 0) ok = ok && mbar_wait(&mma_bar, (uint32_t)(g - 1) & 1);
-        if (!ok) abort_sh = 1;
-        __syncthreads();
-        if (abort_sh) break;
-        // the MMAs of step g - 1 are done: its stage may be refilled
-        if (threadIdx.x == 0 && g > 0 && issued < total) issue(issued++);
-        if (g > 0 && step == 0) {
-            // the previous tile is complete: accumulators -> Out
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int tile = (int)blockIdx.x + ((g - 1) / nsteps) * (int)gridDim.x;
-            const int rt = tile % rtiles, nt = tile / rtiles;
-            const size_t r = (size_t)rt * TC_M + (warp & 3) * 32 + (threadIdx.x & 31);
-            const int cb = (warp >> 2) * 64;
-#pragma unroll 1
-            for (int c0 = cb; c0 < cb + 64; c0 += 16) {
-                if (nt * CB_N + c0 >= N) break;
-                uint32_t v[16];
-                const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                    "[%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-                      "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-                      "=r"(v[14]), "=r"(v[15])
-                    : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                if (r < K) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int n = nt * CB_N + c0 + j;
-                        if (n < N) {
-                            TO* o = Out + (size_t)n * ldo + r;
-                            *o = beta == 0.f ? (TO)__uint_as_float(v[j]) : (TO)(beta * (float)*o + __uint_as_float(v[j]));
-                        }
-                    }
-                }
-            }
-            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        }
-        // A^T: FP32 [64 k][128 r] -> BF16 hi/lo, K-major rows r
-        const float* a32 = reinterpret_cast<const float*>(smem + s * CT_STAGE_BYTES);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int kq = (aq + 4 * j) * 4;
-            const float4 v = make_float4(a32[(kq + 0) * TC_M + ar], a32[(kq + 1) * TC_M + ar],
-                                         a32[(kq + 2) * TC_M + ar], a32[(kq + 3) * TC_M + ar]);
-            uint2 h, l;
-            split4(v, h, l);
-            const uint32_t off = sw128_off(ar, kq);
-            *reinterpret_cast<uint2*>(abf + off) = h;
-            *reinterpret_cast<uint2*>(abf + CB_A_BYTES + off) = l;
-        }
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t a_hi = smem_u32(abf), a_lo = a_hi + CB_A_BYTES;
-            const uint32_t b_hi = smem_u32(smem + s * CT_STAGE_BYTES + CT_A32_BYTES), b_lo = b_hi + CB_B_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < TC_BK / 16; ++kk) {
-                const uint32_t ko = kk * 32;
-                const uint32_t first = (step == 0 && kk == 0) ? 0u : 1u;
-                mma_bf16_n256(tmem, sw128_desc(a_hi + ko), sw128_desc(b_hi + ko), first);
-                mma_bf16_n256(tmem, sw128_desc(a_hi + ko), sw128_desc(b_lo + ko), 1u);
-                mma_bf16_n256(tmem, sw128_desc(a_lo + ko), sw128_desc(b_hi + ko), 1u);
-            }
-            mma_commit(&mma_bar);
-        }
-        committed = g + 1;
-    }
-    if (threadIdx.x == 0) {
-        if (abort_sh) {
-            for (int t = g; t < issued; ++t) mbar_wait(&full[t % CT_STAGES], (uint32_t)(t / CT_STAGES) & 1);
-            if (committed > 0) mbar_wait(&mma_bar, (uint32_t)(committed - 1) & 1);
-        } else if (total > 0 && !mbar_wait(&mma_bar, (uint32_t)(total - 1) & 1)) {
-            abort_sh = 1;
-        }
-    }
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (abort_sh) {
-        if (threadIdx.x == 0) atomicExch(err, 1);
-    } else if (total > 0) {
-        // the last tile
-        const int tile = (int)blockIdx.x + ((total - 1) / nsteps) * (int)gridDim.x;
-        const int rt = tile % rtiles, nt = tile / rtiles;
-        const size_t r = (size_t)rt * TC_M + (warp & 3) * 32 + (threadIdx.x & 31);
-        const int cb = (warp >> 2) * 64;
-#pragma unroll 1
-        for (int c0 = cb; c0 < cb + 64; c0 += 16) {
-            if (nt * CB_N + c0 >= N) break;
-            uint32_t v[16];
-            const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
-                "[%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (r < K) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const int n = nt * CB_N + c0 + j;
-                    if (n < N) {
-                        TO* o = Out + (size_t)n * ldo + r;
-                        *o = beta == 0.f ? (TO)__uint_as_float(v[j]) : (TO)(beta * (float)*o + __uint_as_float(v[j]));
-                    }
-                }
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(CB_N) : "memory");
-    }
-}
+};
 
 }  // namespace
 
@@ -880,7 +698,6 @@ bool make_tile_map(CUtensorMap* m, const float* base, size_t rows, size_t cols, 
                     CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
-
 }  // namespace
 
 size_t tc_combine_scratch_bytes(int N, int Kc) {
@@ -889,49 +706,70 @@ size_t tc_combine_scratch_bytes(int N, int Kc) {
     return 2 * kpad * npad * sizeof(__nv_bfloat16);
 }
 
+namespace {
+
+template <int NT, typename TO>
+cudaError_t combine_ws(const CUtensorMap& map_a, int N, size_t K, int kpad, int npad, const __nv_bfloat16* slices, float beta,
+                       TO* Out, size_t ldo, int* d_err, bool* done, cudaStream_t s) {
+    constexpr int SMEM = CombineShape<Bf16Slices, NT>::SMEM;
+    CUtensorMap map_c;
+    *done = make_map(&map_c, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, slices, (size_t)2 * npad, (size_t)kpad, (size_t)kpad, CW_BK,
+                     NT, CU_TENSOR_MAP_SWIZZLE_64B);
+    if (!*done) return cudaSuccess;
+    static std::atomic<unsigned long long> attr_done{0};  // one per instance
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (dev >= 64 || !(attr_done.load() & (1ull << dev))) {
+        cudaError_t e = cudaFuncSetAttribute(combine_ws_kernel<Bf16Slices, NT, TO>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM);
+        if (e) return e;
+        if (dev < 64) attr_done.fetch_or(1ull << dev);
+    }
+    bool resident;
+    const unsigned grid = combine_grid<Bf16Slices, NT>(K, kpad, npad, sms, &resident);
+    combine_ws_kernel<Bf16Slices, NT, TO><<<grid, CW_THREADS, SMEM, s>>>(map_a, map_c, N, K, kpad, npad, nullptr, nullptr,
+                                                                         resident, beta, Out, ldo, d_err);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
 template <typename TO>
 cudaError_t tc_combine(int N, size_t K, int Kc, const float* A, size_t lda, const double* Coef, int ldcoef,
                        double beta, TO* Out, size_t ldo, void* scratch, int* d_err, int* h_err, cudaStream_t s,
                        int* launches) {
     if (N <= 0 || K == 0) return cudaSuccess;
-    const int kpad = (Kc + TC_BK - 1) / TC_BK * TC_BK;
-    const int npad = (N + CB_N - 1) / CB_N * CB_N;
+    // rows that TMA can read: 32 orbitals a step, tiles of 128 targets where
+    // these are all and 256 beyond (72^3 x 256: 199 us against 257, for a cut and
+    // its hand-offs of half as many steps); others: 64 and 256
+    CUtensorMap map_a;
+    const bool tma = Kc > 0 && K <= 0x7fffffffull &&
+                     make_map(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), A, (size_t)Kc, K, lda, TC_M, CW_BK,
+                              CU_TENSOR_MAP_SWIZZLE_NONE);
+    const int bk = tma ? CW_BK : TC_BK, nt = tma && N <= TC_N ? TC_N : CB_N;
+    const int kpad = (Kc + bk - 1) / bk * bk, npad = (N + nt - 1) / nt * nt;
     __nv_bfloat16* hiT = static_cast<__nv_bfloat16*>(scratch);
     __nv_bfloat16* loT = hiT + (size_t)kpad * npad;
-    static std::atomic<unsigned long long> attr_done{0};  // one per output type
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && !(attr_done.load() & (1ull << dev))) {
-        cudaError_t e =
-            cudaFuncSetAttribute(tc_combine_kernel<TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM_BYTES);
-        if (!e)
-            e = cudaFuncSetAttribute(tc_combine_tma_kernel<TO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     CT_SMEM_BYTES);
-        if (e) return e;
-        attr_done.fetch_or(1ull << dev);
-    }
     cudaMemsetAsync(d_err, 0, sizeof(int), s);
     const int tot = kpad * npad;
     coef_split_kernel<<<(tot + 255) / 256, 256, 0, s>>>(Kc, N, Coef, ldcoef, kpad, npad, hiT, loT);
-    // TMA-fed persistent kernel: A as [Kc][K] FP32 in boxes of 64 k x 128 r;
-    // Coef^T hi/lo as [npad][kpad] BF16 in boxes of 256 n x 64 k, written by
-    // the copy in the 128-byte swizzled layout
-    CUtensorMap map_a, map_hi, map_lo;
-    const bool tma = K <= 0x7fffffffull &&
-                     make_map(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), A, (size_t)Kc, K, lda, TC_M,
-                              TC_BK, CU_TENSOR_MAP_SWIZZLE_NONE) &&
-                     make_map(&map_hi, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, hiT, (size_t)npad, (size_t)kpad,
-                              (size_t)kpad, TC_BK, CB_N, CU_TENSOR_MAP_SWIZZLE_128B) &&
-                     make_map(&map_lo, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, loT, (size_t)npad, (size_t)kpad,
-                              (size_t)kpad, TC_BK, CB_N, CU_TENSOR_MAP_SWIZZLE_128B);
-    if (tma) {
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const long long tiles = (long long)((K + TC_M - 1) / TC_M) * (npad / CB_N);
-        const unsigned grid = (unsigned)std::max<long long>(1, std::min<long long>(tiles, sms));
-        tc_combine_tma_kernel<TO><<<grid, TC_THREADS, CT_SMEM_BYTES, s>>>(map_a, map_hi, map_lo, N, K, kpad,
-                                                                          (float)beta, Out, ldo, d_err);
-    } else {
+    cudaError_t e = cudaSuccess;
+    bool done = false;
+    if (tma)
+        e = nt == TC_N ? combine_ws<TC_N>(map_a, N, K, kpad, npad, hiT, (float)beta, Out, ldo, d_err, &done, s)
+                       : combine_ws<CB_N>(map_a, N, K, kpad, npad, hiT, (float)beta, Out, ldo, d_err, &done, s);
+    if (e) return e;
+    if (!done) {
+        if (tma) return cudaErrorInvalidValue;
+        static std::atomic<unsigned long long> attr_done{0};  // one per output type
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (dev >= 64 || !(attr_done.load() & (1ull << dev))) {
+            if ((e = cudaFuncSetAttribute(tc_combine_kernel<TO>, cudaFuncAttributeMaxDynamicSharedMemorySize, CB_SMEM_BYTES)))
+                return e;
+            if (dev < 64) attr_done.fetch_or(1ull << dev);
+        }
         dim3 grid((unsigned)((K + TC_M - 1) / TC_M), npad / CB_N);
         tc_combine_kernel<TO><<<grid, TC_THREADS, CB_SMEM_BYTES, s>>>(N, K, Kc, kpad, A, lda, hiT, loT,
                                                                       (float)beta, Out, ldo, d_err);
