@@ -563,15 +563,12 @@ template <int RB> cudaError_t ns_cluster(int N, const double* A, double* X, int*
 
 // X = A^{-1/2}; work: five N x ld matrices of T, then the control words.
 template <typename T>
-cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s, int* launches) {
-    *ok = 0;
+cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s, int* launches) {
     const int ld = sizeof(T) == 4 ? (N + 3) / 4 * 4 : N;
     const size_t mat = ((size_t)N * ld * sizeof(T) + 15) / 16 * 16;
     unsigned char* w = reinterpret_cast<unsigned char*>(((uintptr_t)work + 15) & ~(uintptr_t)15);
     unsigned char* ctl = w + 5 * mat;
-    int* d_status = reinterpret_cast<int*>(ctl);
     cudaError_t e;
-    int h = 0;
     const bool small = N <= (sizeof(T) == 4 ? 64 : 16);
     if (small) {
         if (N <= 16) {
@@ -581,7 +578,7 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, c
         else e = ns_cluster<8>(N, A, X, d_status, s);
         if (e) return e;
     } else {
-        if ((e = cudaMemsetAsync(ctl, 0xff, sizeof(int), s))) return e;        // status -1
+        if ((e = cudaMemsetAsync(d_status, 0xff, sizeof(int), s))) return e;        // status -1
         if ((e = cudaMemsetAsync(ctl + 16, 0, 32, s))) return e;               // barrier, norm
         NsArgs<T> a;
         a.N = N;
@@ -610,20 +607,18 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* ok, c
         if ((e = cudaLaunchCooperativeKernel(fn, dim3(ctas), dim3(kNsThreads), args, 0, s))) return e;
     }
     *launches += 1;
-    if ((e = cudaMemcpyAsync(&h, d_status, sizeof(int), cudaMemcpyDeviceToHost, s))) return e;
-    if ((e = cudaStreamSynchronize(s))) return e;
-    if (h < 0) return cudaErrorLaunchTimeout;  // a barrier wait ran out
-    *ok = h == 1;
     return cudaSuccess;
 }
 
 }  // namespace
 
-cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s, int* launches) {
-    return inv_sqrt<double>(N, A, X, work, ok, s, launches);
+cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
+                         int* launches) {
+    return inv_sqrt<double>(N, A, X, work, d_status, s, launches);
 }
-cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s, int* launches) {
-    return inv_sqrt<float>(N, A, X, work, ok, s, launches);
+cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
+                               int* launches) {
+    return inv_sqrt<float>(N, A, X, work, d_status, s, launches);
 }
 
 }  // namespace lace

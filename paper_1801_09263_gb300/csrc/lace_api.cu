@@ -167,7 +167,7 @@ lace_status ensure_orbital_buffers(lace_ctx* c, int n_occ, int n_extra) {
     const size_t wk = std::max(gemm_rows_work_elems(n_p, n_p, ng), (size_t)1);
     CK(c->work.ensure(wk * sizeof(double)), "alloc work");
     CK(c->rowmax.ensure(sizeof(unsigned) * 4 * (size_t)n_p), "alloc row maxima");
-    CK(c->flag.ensure(64), "alloc flag");
+    CK(c->flag.ensure((kFlagSlots + kStatusSlots) * sizeof(int)), "alloc flag");
     CK(c->exd.ensure((8 + 2 * kSumBlocks) * sizeof(double)), "alloc exd");  // [0] E_x, [1] ACE energy, sum scratch
     CK(c->counts.ensure(sizeof(int) * (2 * (size_t)n_occ + 2)), "alloc counts");
     return LACE_OK;
@@ -288,24 +288,33 @@ lace_status orbital_combine(lace_ctx* c, int N, size_t K, int Kc, const T* A, co
     return LACE_OK;
 }
 
+// X = A^{-1/2} with its status in word k, which inv_sqrt_result reads after the
+// next synchronisation (what runs until then works on whatever X holds).
+lace_status inv_sqrt_queue(lace_ctx* c, int n, const double* A, double* X, bool mixed, int k, const char* where, Launch& L) {
+    int* d = c->flag.as<int>() + kFlagSlots + k;
+    *c->status(k) = -1;
+    CK(mixed ? inv_sqrt_spd_mixed(n, A, X, c->m(MS_NSWORK), d, c->stream, &L.n)
+             : inv_sqrt_spd(n, A, X, c->m(MS_NSWORK), d, c->stream, &L.n),
+       where);
+    CK(cudaMemcpyAsync(c->status(k), d, sizeof(int), cudaMemcpyDeviceToHost, c->stream), where);
+    return LACE_OK;
+}
+lace_status inv_sqrt_result(lace_ctx* c, int k, const char* where, const char* not_pd) {
+    if (*c->status(k) < 0) CK(cudaErrorLaunchTimeout, where);  // a barrier wait ran out
+    return *c->status(k) == 1 ? LACE_OK : fail(c, LACE_ERR_NOT_PD, not_pd);
+}
+
 // Loewdin coefficients: X = S^{-1/2}, S = dV src src^T (FP64 Newton-Schulz;
-// mixed path: FP32 Newton-Schulz and one FP64 first-order refinement).
+// mixed path: FP32 Newton-Schulz and one FP64 first-order Loewdin step on X^T S X);
+// the status is in word k.
 template <typename T>
-lace_status lowdin_coeffs(lace_ctx* c, const T* src, const unsigned* mx, int n, double* X, Launch& L) {
+lace_status lowdin_coeffs(lace_ctx* c, const T* src, const unsigned* mx, int n, double* X, int k, Launch& L) {
     double* S = c->m(MS_A);
-    {
-        lace_status st = orbital_gram<T>(c, n, n, c->g.ng, src, mx, src, mx, c->g.dv, S, n, L, "loewdin overlap");
-        if (st) return st;
-    }
-    int ok = 0;
-    if (c->prec == LACE_FP64) {
-        CK(inv_sqrt_spd(n, S, X, c->m(MS_NSWORK), &ok, c->stream, &L.n), "loewdin inverse sqrt");
-    } else {
-        // FP32 Newton-Schulz, then one FP64 first-order Loewdin step on X^T S X
-        CK(inv_sqrt_spd_mixed(n, S, X, c->m(MS_NSWORK), &ok, c->stream, &L.n), "loewdin inverse sqrt");
-        if (ok) CK(lowdin_refine(n, X, S, c->m(MS_NSWORK), c->stream, &L.n), "loewdin refine");
-    }
-    if (!ok) return fail(c, LACE_ERR_NOT_PD, "overlap matrix is singular or ill-conditioned (inverse square root did not converge)");
+    lace_status st = orbital_gram<T>(c, n, n, c->g.ng, src, mx, src, mx, c->g.dv, S, n, L, "loewdin overlap");
+    if (st) return st;
+    const bool mixed = c->prec != LACE_FP64;
+    if ((st = inv_sqrt_queue(c, n, S, X, mixed, k, "loewdin inverse sqrt", L))) return st;
+    if (mixed) CK(lowdin_refine(n, X, S, c->m(MS_NSWORK), c->stream, &L.n), "loewdin refine");
     return LACE_OK;
 }
 
@@ -313,7 +322,7 @@ lace_status lowdin_coeffs(lace_ctx* c, const T* src, const unsigned* mx, int n, 
 template <typename T>
 lace_status lowdin_rows(lace_ctx* c, const T* src, const unsigned* mx, int n, T* dst, Launch& L) {
     double* X = c->m(MS_B);
-    lace_status st = lowdin_coeffs<T>(c, src, mx, n, X, L);
+    lace_status st = lowdin_coeffs<T>(c, src, mx, n, X, 1, L);
     if (st) return st;
     return orbital_combine<T>(c, n, c->g.ng, n, src, mx, X, n, false, dst, L, "loewdin combine");
 }
@@ -351,7 +360,7 @@ lace_status load_impl(lace_ctx* c, const double* d_phi64, int n_occ, int n_extra
     c->x_identity = !ortho;
     c->psi_occ_ready = false;
     if (ortho) {
-        lace_status st = lowdin_coeffs<T>(c, raw, max_occ(c), n_occ, X, L);
+        lace_status st = lowdin_coeffs<T>(c, raw, max_occ(c), n_occ, X, 0, L);
         if (st) return st;
     }
     if (n_extra > 0) {
@@ -447,11 +456,18 @@ lace_status load_common(lace_ctx* c, const double* phi, bool dev, int n_occ, int
     CK(cudaStreamSynchronize(c->stream), "load");
     if (c->hflags && tc_timed_out(c))
         return fail(c, LACE_ERR_TIMEOUT, "orthonormalisation: an mbarrier wait timed out");
+    for (int k = 0; ortho && k < (n_extra > 0 ? 2 : 1); ++k)
+        if ((st = inv_sqrt_result(c, k, "loewdin inverse sqrt",
+                                  "overlap matrix is singular or ill-conditioned (inverse square root did not converge)")))
+            return st;
     c->loaded = true;
     return LACE_OK;
 }
 
 // ------------------------------------------------------------------ SCDM
+// Orbitals sorted along the Z-order curve of their points (behind the points).
+int* pair_order(lace_ctx* c) { return reinterpret_cast<int*>(c->pivfull.as<long long>() + c->n_occ); }
+
 template <typename T>
 lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
     Launch L{c};
@@ -459,8 +475,9 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
     const int n = c->n_occ;
     T* raw = c->canon.as<T>();
     const double* X = c->m(MS_X);
-    CK(c->pivfull.ensure(sizeof(long long) * n), "alloc pivots");
+    CK(c->pivfull.ensure((sizeof(long long) + sizeof(int)) * n), "alloc pivots");
     long long* d_full = c->pivfull.as<long long>();
+    *c->status(2) = 0;
     if (!imposed) {
         int ncol = 0;
         const int m1 = (c->g.n[0] + stride - 1) / stride, m2 = (c->g.n[1] + stride - 1) / stride,
@@ -481,25 +498,14 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
             lace_status st = orbital_combine<T>(c, n, (size_t)ncol, n, tmp, max_occ(c), X, n, false, R, L, "subsample");
             if (st) return st;
         }
-        int timeout = 0;
-        CK(qrcp_pivots<T>(n, ncol, R, n, c->piv.as<int>(), c->aux.p, &timeout, c->wait_limit_ns, c->stream, &L.n),
+        CK(cudaMemsetAsync(c->piv.p, 0, sizeof(int) * n, c->stream), "qrcp");
+        CK(qrcp_pivots<T>(n, ncol, R, n, c->piv.as<int>(), c->aux.p, c->status(2), c->wait_limit_ns, c->stream, &L.n),
            "qrcp");
-        if (timeout) return fail(c, LACE_ERR_TIMEOUT, "pivoted QR: a grid barrier wait timed out");
-        std::vector<int> hp(n);
-        CK(cudaMemcpyAsync(hp.data(), c->piv.p, sizeof(int) * n, cudaMemcpyDeviceToHost, c->stream), "pivots");
-        CK(cudaStreamSynchronize(c->stream), "pivots");
-        c->pivots_host.resize(n);
-        for (int k = 0; k < n; ++k) {
-            const int cc = hp[k];
-            const int kz = cc % m3, jy = (cc / m3) % m2, ix = cc / (m3 * m2);
-            c->pivots_host[k] = ((long long)(ix * stride) * c->g.n[1] + (long long)(jy * stride)) * c->g.n[2] +
-                                (long long)(kz * stride);
-        }
+        CK(pivot_points(c->g, stride, n, c->piv.as<int>(), d_full, pair_order(c), c->stream, &L.n), "pivots");
     } else {
-        c->pivots_host.assign(imposed, imposed + n);
+        CK(cudaMemcpyAsync(d_full, imposed, sizeof(long long) * n, cudaMemcpyHostToDevice, c->stream), "pivots");
+        CK(pivot_points(c->g, 1, n, nullptr, d_full, pair_order(c), c->stream, &L.n), "pivots");
     }
-    CK(cudaMemcpyAsync(d_full, c->pivots_host.data(), sizeof(long long) * n, cudaMemcpyHostToDevice, c->stream),
-       "pivots");
     double* phic = c->m(MS_A);
     double* B = c->m(MS_B);
     double* Bmh = c->m(MS_LINV);
@@ -514,13 +520,16 @@ lace_status localize_impl(lace_ctx* c, int stride, const long long* imposed) {
     }
     // B = phi_C phi_C^T  (points x points)
     CK(small_gemm_f64(n, n, n, phic, n, false, phic, n, true, 1.0, 0.0, B, n, c->stream, &L.n), "scdm B");
-    int ok = 0;
-    if (c->prec == LACE_FP64) {
-        CK(inv_sqrt_spd(n, B, Bmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "scdm inverse sqrt");
-    } else {
-        CK(inv_sqrt_spd_mixed(n, B, Bmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "scdm inverse sqrt");
+    {
+        lace_status st = inv_sqrt_queue(c, n, B, Bmh, c->prec != LACE_FP64, 0, "scdm inverse sqrt", L);
+        if (st) return st;
+        c->pivots_host.resize(n);
+        CK(cudaMemcpyAsync(c->pivots_host.data(), d_full, sizeof(long long) * n, cudaMemcpyDeviceToHost, c->stream), "pivots");
+        CK(cudaStreamSynchronize(c->stream), "pivots");
+        if (*c->status(2)) return fail(c, LACE_ERR_TIMEOUT, "pivoted QR: a grid barrier wait timed out");
+        // (the orbitals stay as they are when the columns are dependent)
+        if ((st = inv_sqrt_result(c, 0, "scdm inverse sqrt", "selected columns are rank deficient"))) return st;
     }
-    if (!ok) return fail(c, LACE_ERR_NOT_PD, "selected columns are rank deficient");
     // U = phi_C^T B^{-1/2}  (orbitals x orbitals)
     CK(small_gemm_f64(n, n, n, phic, n, true, Bmh, n, false, 1.0, 0.0, U, n, c->stream, &L.n), "scdm U");
     // mixed path: restore exact orthogonality of U in FP64 (U <- U (I - (U^T U - I)/2))
@@ -559,9 +568,10 @@ lace_status align_impl(lace_ctx* c) {
         (st = orbital_gram<T>(c, n, n, ng, w, max_w(c), ref, max_ref(c), c->g.dv, Om, n, L, "alignment overlap")))
         return st;
     CK(small_gemm_f64(n, n, n, Om, n, true, Om, n, false, 1.0, 0.0, P, n, c->stream, &L.n), "alignment");
-    int ok = 0;
-    CK(inv_sqrt_spd(n, P, Pmh, c->m(MS_NSWORK), &ok, c->stream, &L.n), "alignment");
-    if (!ok) return fail(c, LACE_ERR_NOT_PD, "the orbitals are nearly orthogonal to the previous ones (no alignment)");
+    if ((st = inv_sqrt_queue(c, n, P, Pmh, false, 0, "alignment", L))) return st;
+    CK(cudaStreamSynchronize(c->stream), "alignment");
+    if ((st = inv_sqrt_result(c, 0, "alignment", "the orbitals are nearly orthogonal to the previous ones (no alignment)")))
+        return st;
     CK(small_gemm_f64(n, n, n, Om, n, false, Pmh, n, false, 1.0, 0.0, Q, n, c->stream, &L.n), "alignment");
     // the SCDM rotation now includes Q
     double* U = c->m(MS_U);
@@ -609,44 +619,15 @@ lace_status make_pairs(lace_ctx* c, bool use_S, double thr, Launch& L) {
     const size_t maxp = (size_t)n * (n + 1) / 2 + (size_t)n * ne;
     CK(c->pairs.ensure(sizeof(int2) * std::max<size_t>(maxp, 1)), "alloc pairs");
     CK(c->grids.ensure(sizeof(PairGrid) * std::max<size_t>((maxp + 1) / 2, 1)), "alloc grids");
-    long long np = 0;
-    CK(build_pair_list(n, ne, c->m(MS_S), thr, use_S, c->pairs.as<int2>(), c->counts.as<int>(), &np, c->stream, &L.n),
-       "pair list");
-    // Localised orbitals: order the pairs by the Z-order rank of their orbitals'
-    // SCDM points, so consecutive FFT grids touch nearby orbitals and their W
-    // and Psi planes stay in L2.  Each pair keeps (i, j) with i <= j.
+    // Localised orbitals: rows and columns of the list in the Z-order of their SCDM
+    // points, so consecutive FFT grids touch nearby orbitals and their W and Psi
+    // planes stay in L2.  Each pair keeps (i, j) with i <= j.
     const char* noord = getenv("LACE_NO_PAIR_ORDER");
-    if (c->localized && np > 1 && (int)c->pivots_host.size() == n && !(noord && noord[0] == '1')) {
-        std::vector<int2> hp(np);
-        CK(cudaMemcpyAsync(hp.data(), c->pairs.p, sizeof(int2) * np, cudaMemcpyDeviceToHost, c->stream), "pairs");
-        CK(cudaStreamSynchronize(c->stream), "pairs");
-        auto spread = [](uint64_t v) {  // interleave 21 bits with two zero bits
-            v &= 0x1fffff;
-            v = (v | v << 32) & 0x1f00000000ffffULL;
-            v = (v | v << 16) & 0x1f0000ff0000ffULL;
-            v = (v | v << 8) & 0x100f00f00f00f00fULL;
-            v = (v | v << 4) & 0x10c30c30c30c30c3ULL;
-            v = (v | v << 2) & 0x1249249249249249ULL;
-            return v;
-        };
-        std::vector<std::pair<uint64_t, int>> code(n);
-        for (int i = 0; i < n; ++i) {
-            const long long p = c->pivots_host[i];
-            const uint64_t z = p % c->g.n[2], y = (p / c->g.n[2]) % c->g.n[1], x = p / ((long long)c->g.n[2] * c->g.n[1]);
-            code[i] = {spread(x) << 2 | spread(y) << 1 | spread(z), i};
-        }
-        std::sort(code.begin(), code.end());
-        std::vector<int> rank(n + ne);
-        for (int r = 0; r < n; ++r) rank[code[r].second] = r;
-        for (int e = 0; e < ne; ++e) rank[n + e] = n + e;
-        std::stable_sort(hp.begin(), hp.end(), [&](const int2& a, const int2& b) {
-            const int a0 = std::min(rank[a.x], rank[a.y]), a1 = std::max(rank[a.x], rank[a.y]);
-            const int b0 = std::min(rank[b.x], rank[b.y]), b1 = std::max(rank[b.x], rank[b.y]);
-            return a0 != b0 ? a0 < b0 : a1 < b1;
-        });
-        CK(cudaMemcpyAsync(c->pairs.p, hp.data(), sizeof(int2) * np, cudaMemcpyHostToDevice, c->stream), "pairs");
-        CK(cudaStreamSynchronize(c->stream), "pairs");
-    }
+    const bool ordered = c->localized && (int)c->pivots_host.size() == n && !(noord && noord[0] == '1');
+    long long np = 0;
+    CK(build_pair_list(n, ne, c->m(MS_S), thr, use_S, ordered ? pair_order(c) : nullptr, c->pairs.as<int2>(),
+                       c->counts.as<int>(), c->status(3), &np, c->stream, &L.n),
+       "pair list");
     CK(pack_pair_grids(c->pairs.as<int2>(), np, n, c->grids.as<PairGrid>(), c->stream, &L.n), "pack pairs");
     c->n_pairs = np;
     return LACE_OK;
@@ -1018,7 +999,7 @@ lace_status lace_create(lace_ctx** out, int device, int precision) {
     c->stream = c->own_stream;
     for (auto& e : c->ev) cudaEventCreate(&e);
     void* hf = nullptr;  // pinned timeout flags (without them every tensor-core call waits for its own)
-    if (cudaHostAlloc(&hf, kFlagSlots * sizeof(int), cudaHostAllocDefault) == cudaSuccess) {
+    if (cudaHostAlloc(&hf, (kFlagSlots + kStatusSlots) * sizeof(int), cudaHostAllocDefault) == cudaSuccess) {
         c->hflags = static_cast<int*>(hf);
     } else {
         cudaGetLastError();

@@ -42,7 +42,8 @@ constexpr int kMatSlots = MS_NSWORK + 5 + 1;
 // chunks of a host ACE apply (the chunk energies sit in exd[2 .. 2 + kApplyChunks))
 constexpr int kApplyChunks = 4;
 // int slots of a context's device flag buffer (64 bytes)
-constexpr int kFlagSlots = 16;
+constexpr int kFlagSlots = 16;  // tensor-core timeout flags
+constexpr int kStatusSlots = 4;  // and behind them: inverse square roots (2), pivoted QR, pair count
 
 }  // namespace lace
 
@@ -106,8 +107,10 @@ struct lace_ctx {
     // timeout flags of the tensor-core calls of one API call: device slots
     // flag[2 .. tc_next), copied after each call into pinned hflags and read
     // at the API call's next synchronisation instead of one wait per call
-    int* hflags = nullptr;  // pinned, kFlagSlots ints
+    int* hflags = nullptr;  // pinned, kFlagSlots + kStatusSlots ints
     int tc_next = 2;
+    int status_host[lace::kStatusSlots] = {};  // the status words where no pinned ones could be had
+    int* status(int k) { return hflags ? hflags + lace::kFlagSlots + k : status_host + k; }
 
     // small-matrix slots inside `mat` (each n_p*n_p doubles, plus staging)
     size_t mslot = 0;

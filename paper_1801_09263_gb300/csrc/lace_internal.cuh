@@ -206,12 +206,13 @@ size_t combine_exact_scratch_bytes(int N, int Kc);
 cudaError_t small_gemm_f64(int M, int N, int K, const double* A, int lda, bool ta, const double* B, int ldb, bool tb,
                            double alpha, double beta, double* C, int ldc, cudaStream_t s, int* launches);
 // X = A^{-1/2} of a symmetric positive definite A by the coupled Newton-Schulz
-// iteration; returns cudaSuccess and *ok=0 if it does not converge.
+// iteration.  *d_status (read it after a synchronisation): 1 converged, 0 not (X is not
+// written), -1 a grid-barrier wait ran out of time.
 // (invsqrt.cu; work: 5 N^2 + 320 N + 320 doubles)
-cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s, int* launches);
+cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s, int* launches);
 // Mixed-precision variant: FP32 Newton-Schulz to ~1e-7, returns X0 ~ A^{-1/2}
 // (FP64, symmetric).  Pair it with lowdin_refine.
-cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* ok, cudaStream_t s,
+cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
                                int* launches);
 // F <- F (I - E/2), E = F^T G F - I (G = I when null): orthonormality to O(E^2).
 cudaError_t lowdin_refine(int N, double* F, const double* G, double* work, cudaStream_t s, int* launches);
@@ -229,9 +230,9 @@ cudaError_t symmetrize(int N, const double* A, double* B, int mode, bool neg, cu
 // SCDM pivoted QR (scdm.cu): selects npiv columns of R (nrow x ncol,
 // row-major, overwritten).  Pivots are column indices, ties to the lowest
 // index.  aux: caller scratch of qrcp_aux_bytes(nrow, ncol) bytes.
-// *h_timeout = 1 when a grid-barrier wait of the persistent kernel ran out of
-// time (the pivots are then invalid); wait_limit_ns bounds each such wait.
-// The persistent path waits for s.
+// *h_timeout != 0 (after a synchronisation of s): a grid-barrier wait of the
+// persistent kernel ran out of time (the pivots are then invalid); wait_limit_ns
+// bounds each such wait.
 template <typename T>
 cudaError_t qrcp_pivots(int nrow, int ncol, T* R, int npiv, int* d_piv, void* aux, int* h_timeout,
                         unsigned long long wait_limit_ns, cudaStream_t s, int* launches);
@@ -246,11 +247,17 @@ template <typename T>
 cudaError_t gather_columns(const T* psi, size_t ldpsi, int norb, const long long* d_full_idx, int npts, double* out,
                            cudaStream_t s, int* launches);
 
+// Grid points full[k] of the subsample columns piv[k] < ncol (piv == nullptr: full
+// is given), and order[0..n): the points' indices sorted along the Z-order curve.
+cudaError_t pivot_points(const GridGeom& g, int stride, int n, const int* piv, long long* full, int* order, cudaStream_t s,
+                         int* launches);
+
 // Screening (screen.cu): keep mask from S and the pair list.
-// Writes the kept (i, j) pairs, i <= j < n_occ with S_ij >= thr, row by row,
-// followed by all (i, n_occ + e).  Returns the count in *n_pairs (host).
-cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double thr, bool use_S, int2* d_pairs,
-                            int* d_counts, long long* n_pairs, cudaStream_t s, int* launches);
+// Writes the kept pairs (i, j), i <= j < n_occ with S_ij >= thr, row by row,
+// followed by all (i, n_occ + e); rows and columns run through order[] where
+// given.  Returns the count in *n_pairs, read through h_total (pinned).
+cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double thr, bool use_S, const int* order,
+                            int2* d_pairs, int* d_counts, int* h_total, long long* n_pairs, cudaStream_t s, int* launches);
 // Pack pairs two by two into complex FFT grids (an orbital shared by the two
 // pairs of a grid in both i slots).
 cudaError_t pack_pair_grids(const int2* d_pairs, long long n_pairs, int n_occ, PairGrid* d_grids, cudaStream_t s,

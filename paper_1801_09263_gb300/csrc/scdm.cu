@@ -493,6 +493,47 @@ __global__ void gather_columns_kernel(const T* __restrict__ psi, size_t ldpsi, i
     out[e] = (double)psi[(size_t)o * ldpsi + (size_t)idx[p]];
 }
 
+// Thread i: grid point of pivot i and its rank among all by the Z-order code
+// (coordinate bits interleaved), codes recomputed 256 at a time in shared
+// memory.
+__global__ void __launch_bounds__(256) pivot_points_kernel(int n1, int n2, int m1, int m2, int m3, int stride, int n,
+                                                           const int* __restrict__ piv, long long* __restrict__ full,
+                                                           int* __restrict__ order) {
+    __shared__ unsigned long long code[256];
+    auto spread = [](unsigned long long v) {  // two zero bits between 21 bits
+        v &= 0x1fffff;
+        v = (v | v << 32) & 0x1f00000000ffffULL;
+        v = (v | v << 16) & 0x1f0000ff0000ffULL;
+        v = (v | v << 8) & 0x100f00f00f00f00fULL;
+        v = (v | v << 4) & 0x10c30c30c30c30c3ULL;
+        return (v | v << 2) & 0x1249249249249249ULL;
+    };
+    auto point = [&](int k) -> long long {
+        if (!piv) return full[k];
+        const int c = min(max(piv[k], 0), m1 * m2 * m3 - 1);  // (invalid after a timeout)
+        return ((long long)(c / (m3 * m2) * stride) * n1 + (long long)(c / m3 % m2) * stride) * n2 + (long long)(c % m3) * stride;
+    };
+    auto code_of = [&](long long p) {
+        return spread((unsigned long long)(p / ((long long)n2 * n1))) << 2 | spread((unsigned long long)(p / n2 % n1)) << 1 |
+               spread((unsigned long long)(p % n2));
+    };
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    const long long mine = i < n ? point(i) : 0;
+    const unsigned long long c = code_of(mine);
+    int rank = 0;
+    for (int j0 = 0; j0 < n; j0 += 256) {
+        __syncthreads();
+        if (j0 + (int)threadIdx.x < n) code[threadIdx.x] = code_of(point(j0 + threadIdx.x));
+        __syncthreads();
+        const int m = min(256, n - j0);
+        for (int j = 0; j < m; ++j) rank += code[j] < c || (code[j] == c && j0 + j < i);
+    }
+    if (i < n) {
+        if (piv) full[i] = mine;
+        order[rank] = i;
+    }
+}
+
 }  // namespace
 
 static size_t align256(size_t b) { return (b + 255) / 256 * 256; }
@@ -632,11 +673,7 @@ cudaError_t qrcp_pivots(int nrow, int ncol, T* R, int npiv, int* d_piv, void* au
     }
     if (e) return e;
     if (ran) {
-        unsigned flag = 0;
-        if ((e = cudaMemcpyAsync(&flag, bar + 2, sizeof(unsigned), cudaMemcpyDeviceToHost, s))) return e;
-        if ((e = cudaStreamSynchronize(s))) return e;
-        *h_timeout = flag != 0u;
-        return cudaSuccess;
+        return cudaMemcpyAsync(h_timeout, bar + 2, sizeof(int), cudaMemcpyDeviceToHost, s);
     }
     for (int step = 0; step < npiv; ++step) {
         qr_update_kernel<T><<<nblocks, QR_THREADS, 0, s>>>(nrow, ncol, R, (size_t)ncol, q, step > 0, chosen, best);
@@ -655,6 +692,15 @@ cudaError_t gather_subsample(const GridGeom& g, int stride, const T* psi, int no
     *ncol_out = (int)ncol;
     dim3 grid((unsigned)std::min<size_t>((ncol + 255) / 256, 1024), norb);
     gather_subsample_kernel<T><<<grid, 256, 0, s>>>(g.n[0], g.n[1], g.n[2], stride, m1, m2, m3, psi, g.ng, out, ncol);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t pivot_points(const GridGeom& g, int stride, int n, const int* piv, long long* full, int* order, cudaStream_t s,
+                         int* launches) {
+    const int m1 = (g.n[0] + stride - 1) / stride, m2 = (g.n[1] + stride - 1) / stride,
+              m3 = (g.n[2] + stride - 1) / stride;
+    pivot_points_kernel<<<(n + 255) / 256, 256, 0, s>>>(g.n[1], g.n[2], m1, m2, m3, stride, n, piv, full, order);
     *launches += 1;
     return cudaGetLastError();
 }

@@ -13,14 +13,22 @@ namespace {
 
 constexpr int SC_THREADS = 256;
 
-// counts[i] = number of kept j in [i, n_occ) plus n_extra.
+// Pair of row r and column q of the list, its lower orbital first.
+__device__ __forceinline__ int2 pair_of(int r, int q, const int* __restrict__ order) {
+    const int i = order ? order[r] : r, j = order ? order[q] : q;
+    return make_int2(min(i, j), max(i, j));
+}
+__device__ __forceinline__ bool kept(int2 p, int n_occ, const double* __restrict__ S, double thr, int use_S) {
+    return !use_S || S[(size_t)p.x * n_occ + p.y] >= thr;
+}
+
+// counts[r] = number of kept pairs of row r with columns in [r, n_occ) plus n_extra.
 __global__ void count_kernel(int n_occ, int n_extra, const double* __restrict__ S, double thr, int use_S,
-                             int* __restrict__ counts) {
+                             const int* __restrict__ order, int* __restrict__ counts) {
     const int i = blockIdx.x;
     __shared__ int sh[SC_THREADS];
     int c = 0;
-    for (int j = i + threadIdx.x; j < n_occ; j += blockDim.x)
-        c += (!use_S || S[(size_t)i * n_occ + j] >= thr) ? 1 : 0;
+    for (int j = i + threadIdx.x; j < n_occ; j += blockDim.x) c += kept(pair_of(i, j, order), n_occ, S, thr, use_S) ? 1 : 0;
     sh[threadIdx.x] = c;
     __syncthreads();
     for (int o = blockDim.x / 2; o > 0; o >>= 1) {
@@ -42,9 +50,9 @@ __global__ void scan_kernel(int n, const int* __restrict__ counts, int* __restri
     }
 }
 
-// Row i writes its kept (i, j), j ascending, then (i, n_occ + e).
+// Row i writes its kept pairs, columns ascending, then those with the extras.
 __global__ void write_pairs_kernel(int n_occ, int n_extra, const double* __restrict__ S, double thr, int use_S,
-                                   const int* __restrict__ offs, int2* __restrict__ pairs) {
+                                   const int* __restrict__ order, const int* __restrict__ offs, int2* __restrict__ pairs) {
     const int i = blockIdx.x;
     __shared__ int base;
     __shared__ int warp_tot[SC_THREADS / 32];
@@ -53,14 +61,15 @@ __global__ void write_pairs_kernel(int n_occ, int n_extra, const double* __restr
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j0 = i; j0 < n_occ; j0 += blockDim.x) {
         const int j = j0 + threadIdx.x;
-        const bool keep = j < n_occ && (!use_S || S[(size_t)i * n_occ + j] >= thr);
+        const int2 p = j < n_occ ? pair_of(i, j, order) : make_int2(0, 0);
+        const bool keep = j < n_occ && kept(p, n_occ, S, thr, use_S);
         const unsigned ballot = __ballot_sync(0xffffffffu, keep);
         const int rank = __popc(ballot & ((1u << lane) - 1u));
         if (lane == 0) warp_tot[warp] = __popc(ballot);
         __syncthreads();
         int before = 0;
         for (int w = 0; w < warp; ++w) before += warp_tot[w];
-        if (keep) pairs[base + before + rank] = make_int2(i, j);
+        if (keep) pairs[base + before + rank] = p;
         __syncthreads();
         if (threadIdx.x == 0) {
             int t = 0;
@@ -69,7 +78,7 @@ __global__ void write_pairs_kernel(int n_occ, int n_extra, const double* __restr
         }
         __syncthreads();
     }
-    for (int e = threadIdx.x; e < n_extra; e += blockDim.x) pairs[base + e] = make_int2(i, n_occ + e);
+    for (int e = threadIdx.x; e < n_extra; e += blockDim.x) pairs[base + e] = make_int2(order ? order[i] : i, n_occ + e);
 }
 
 // Two pairs of one grid that share an occupied orbital both take it as i (a
@@ -161,17 +170,17 @@ cudaError_t neg_sum_squares(size_t m, const double* d_X, double* d_part, double*
     return fixed_sum(m, d_X, true, -1.0, d_part, d_out, s, launches);
 }
 
-cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double thr, bool use_S, int2* d_pairs,
-                            int* d_counts, long long* n_pairs, cudaStream_t s, int* launches) {
+cudaError_t build_pair_list(int n_occ, int n_extra, const double* d_S, double thr, bool use_S, const int* order,
+                            int2* d_pairs, int* d_counts, int* h_total, long long* n_pairs, cudaStream_t s, int* launches) {
     int* offs = d_counts + n_occ;  // caller provides 2*n_occ + 1 ints
-    count_kernel<<<n_occ, SC_THREADS, 0, s>>>(n_occ, n_extra, d_S, thr, use_S ? 1 : 0, d_counts);
+    count_kernel<<<n_occ, SC_THREADS, 0, s>>>(n_occ, n_extra, d_S, thr, use_S ? 1 : 0, order, d_counts);
     scan_kernel<<<1, 32, 0, s>>>(n_occ, d_counts, offs);
-    write_pairs_kernel<<<n_occ, SC_THREADS, 0, s>>>(n_occ, n_extra, d_S, thr, use_S ? 1 : 0, offs, d_pairs);
+    write_pairs_kernel<<<n_occ, SC_THREADS, 0, s>>>(n_occ, n_extra, d_S, thr, use_S ? 1 : 0, order, offs, d_pairs);
     *launches += 3;
-    int total = 0;
-    cudaMemcpyAsync(&total, offs + n_occ, sizeof(int), cudaMemcpyDeviceToHost, s);
+    *h_total = 0;
+    cudaMemcpyAsync(h_total, offs + n_occ, sizeof(int), cudaMemcpyDeviceToHost, s);
     cudaError_t e = cudaStreamSynchronize(s);
-    *n_pairs = total;
+    *n_pairs = *h_total;
     return e;
 }
 
