@@ -428,6 +428,17 @@ size_t f64_chunks(int M, int N, size_t K, bool sym) {
     return std::max<size_t>(1, std::min(want, (K + 255) / 256));
 }
 
+// Whether an FP64 Gram takes the 64-wide tiles of gemm_rows_kernel: their operands
+// are reused four times as often, 0.81 ms a tile on 48^3 against 0.066 ms a 16-wide one,
+// but the padding is theirs.  On 48^3, 64-wide and 16-wide: 128 x 128 3.37 and 4.25 ms, its
+// triangle 3.35 and 2.39; 192 x 192 7.30 and 9.57, triangle 4.78 and 5.45; 96 x 96 3.34 and
+// 2.39; a single tile does not fill the chip, 64 x 64 1.18 and 1.01.
+bool f64_wide(int M, int N, bool sym) {
+    const size_t tm = (size_t)(M + GR_BM - 1) / GR_BM, tn = (size_t)(N + GR_BN - 1) / GR_BN;
+    const size_t wide = sym ? tm * (tm + 1) / 2 : tm * tn;
+    return wide > 1 && 2 * f64_tiles(M, N, sym) > 25 * wide;
+}
+
 // ------------------------------------------------------------------ gemm_combine
 constexpr int GC_BR = 128, GC_BN = 64, GC_BK = 16, GC_THREADS = 256;
 
@@ -926,7 +937,7 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
     if (M <= 0 || N <= 0) return cudaSuccess;
     const bool sym = (A == B) && (lda == ldb) && (M == N);
     const size_t tot = (size_t)M * N;
-    if constexpr (sizeof(T) == 8) {
+    if constexpr (sizeof(T) == 8) if (!f64_wide(M, N, sym)) {
         const size_t n = std::min(f64_chunks(M, N, K, sym), work_elems / tot);
         if (n == 0) return cudaErrorInvalidValue;
         size_t kc = (K + n - 1) / n;
@@ -960,6 +971,8 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
             gemm_rows_kernel<T, true><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
         else
             gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
+    } else {
+        gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
     }
     if (nch_eff >= 32)
         reduce_chunks_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym,
