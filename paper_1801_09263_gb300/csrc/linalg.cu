@@ -11,6 +11,7 @@
 #include <type_traits>
 
 #include "f32x2.cuh"
+#include "chunk_sum.cuh"
 #include "lace_internal.cuh"
 
 namespace lace {
@@ -350,35 +351,6 @@ __global__ void __launch_bounds__(32 * GD_WARPS) gemm_rows_f64_kernel(int M, int
         if (m < M && n < N)
             out[(size_t)m * N + n] = (red[e] + red[GD_T * GD_T + e]) + (red[2 * GD_T * GD_T + e] + red[3 * GD_T * GD_T + e]);
     }
-}
-
-// Many chunks of a small product: one warp an output, the lanes over the
-// chunks, then across the lanes (a fixed order).  tile: rows of the tiles of a
-// symmetric product, of which only those on and above the diagonal hold values.
-__global__ void reduce_chunks_warp_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha,
-                                          bool sym, int tile, double* __restrict__ C, int ldc) {
-    const size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (idx >= (size_t)M * N) return;
-    const int lane = threadIdx.x & 31;
-    const int m = (int)(idx / N), n = (int)(idx % N);
-    const size_t src = (sym && n / tile < m / tile) ? (size_t)n * N + m : idx;
-    double s = 0.0;
-    for (int c = lane; c < nchunk; c += 32) s += work[(size_t)c * M * N + src];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) C[(size_t)m * ldc + n] = alpha * s;
-}
-
-__global__ void reduce_chunks_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha,
-                                     bool sym, int tile, double* __restrict__ C, int ldc) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)M * N) return;
-    const int m = (int)(idx / N), n = (int)(idx % N);
-    // symmetric products computed only the tiles above the diagonal: mirror the rest
-    const size_t src = (sym && n / tile < m / tile) ? (size_t)n * N + m : idx;
-    double s = 0.0;
-    for (int c = 0; c < nchunk; ++c) s += work[(size_t)c * M * N + src];
-    C[(size_t)m * ldc + n] = alpha * s;
 }
 
 int sm_count() {
@@ -945,13 +917,7 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
         const size_t nc = (K + kc - 1) / kc;
         gemm_rows_f64_kernel<<<dim3((unsigned)f64_tiles(M, N, sym), (unsigned)nc), 32 * GD_WARPS, 0, s>>>(
             M, N, K, A, lda, B, ldb, absval, sym, kc, work);
-        // (32 chunks and more: a thread summing them alone waits for each in turn)
-        if (nc >= 32)
-            reduce_chunks_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nc, work, alpha, sym,
-                                                                                 GD_T, C, ldc);
-        else
-            reduce_chunks_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nc, work, alpha, sym, GD_T, C,
-                                                                               ldc);
+        chunk_sum(M, N, nc, work, alpha, sym, GD_T, C, ldc, s);
         *launches += 2;
         return cudaGetLastError();
     }
@@ -974,12 +940,7 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
     } else {
         gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
     }
-    if (nch_eff >= 32)
-        reduce_chunks_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym,
-                                                                             GR_BM, C, ldc);
-    else
-        reduce_chunks_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym, GR_BM, C,
-                                                                           ldc);
+    chunk_sum(M, N, nch_eff, work, alpha, sym, GR_BM, C, ldc, s);
     *launches += 2;
     return cudaGetLastError();
 }

@@ -36,6 +36,7 @@
 #include <algorithm>
 #include <atomic>
 
+#include "chunk_sum.cuh"
 #include "f32x2.cuh"
 #include "lace_internal.cuh"
 #include "tc_combine.cuh"
@@ -430,25 +431,6 @@ size_t exact_chunks(int M, int N, size_t K, bool sym) {
     return std::max<size_t>(1, std::min(want, (K + 255) / 256));
 }
 
-__global__ void exact_reduce_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha, bool sym, bool warp,
-                                    double* __restrict__ C, int ldc) {
-    const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x, idx = warp ? t >> 5 : t;
-    if (idx >= (size_t)M * N) return;
-    const int lane = threadIdx.x & 31;
-    const int m = (int)(idx / N), n = (int)(idx % N);
-    const size_t src = (sym && n / TC_N < m / TC_M) ? (size_t)n * N + m : idx;
-    double s = 0.0;
-    if (warp) {
-        for (int c = lane; c < nchunk; c += 32) s += work[(size_t)c * M * N + src];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane) return;
-    } else {
-        for (int c = 0; c < nchunk; ++c) s += work[(size_t)c * M * N + src];
-    }
-    C[(size_t)m * ldc + n] = alpha * s;
-}
-
 }  // namespace
 
 bool exact_ok(size_t K, const void* a) { return K % 4 == 0 && K <= 0x7fffffffull && (uintptr_t)a % 16 == 0 && encode_tiled() != nullptr; }
@@ -499,10 +481,7 @@ cudaError_t gram_exact(int M, int N, size_t K, const float* A, const unsigned* m
     if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s))) return e;
     gram_exact_kernel<<<dim3((unsigned)exact_tiles(M, N, sym), 1, (unsigned)nch_eff), GX_THREADS, GX_SMEM_BYTES, s>>>(
         map_a, map_b, M, N, K, kchunk, (M + TC_M - 1) / TC_M, sym, max_a, max_b, work, d_err);
-    const size_t tot = (size_t)M * N;
-    const bool warp = nch_eff >= 16 && tot <= 128 * 128;
-    exact_reduce_kernel<<<(unsigned)(((warp ? 32 * tot : tot) + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, sym,
-                                                                                   warp, C, ldc);
+    chunk_sum(M, N, nch_eff, work, alpha, sym, TC_M, C, ldc, s);
     *launches += 2;
     return cudaGetLastError();
 }

@@ -31,6 +31,7 @@
 
 #include <algorithm>
 
+#include "chunk_sum.cuh"
 #include "lace_internal.cuh"
 #include "tc_combine.cuh"
 #include "tc_util.cuh"
@@ -476,36 +477,6 @@ __global__ void __launch_bounds__(TW_THREADS, 1)
     }
 }
 
-// Sum of the chunks in FP64 in a fixed order; for a symmetric product the
-// tiles below the diagonal were not computed and are read mirrored.
-__global__ void tc_reduce_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha, bool sym,
-                                 double* __restrict__ C, int ldc) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)M * N) return;
-    const int m = (int)(idx / N), n = (int)(idx % N);
-    const size_t src = (sym && n / TC_N < m / TC_M) ? (size_t)n * N + m : idx;
-    double s = 0.0;
-    for (int c = 0; c < nchunk; ++c) s += work[(size_t)c * M * N + src];
-    C[(size_t)m * ldc + n] = alpha * s;
-}
-
-// The same for small products of many chunks: one warp an output, the lanes
-// over the chunks, then across the lanes (a thread alone would wait for one
-// chunk after the other).
-__global__ void tc_reduce_warp_kernel(int M, int N, int nchunk, const double* __restrict__ work, double alpha, bool sym,
-                                      double* __restrict__ C, int ldc) {
-    const size_t idx = ((size_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (idx >= (size_t)M * N) return;
-    const int lane = threadIdx.x & 31;
-    const int m = (int)(idx / N), n = (int)(idx % N);
-    const size_t src = (sym && n / TC_N < m / TC_M) ? (size_t)n * N + m : idx;
-    double s = 0.0;
-    for (int c = lane; c < nchunk; c += 32) s += work[(size_t)c * M * N + src];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) C[(size_t)m * ldc + n] = alpha * s;
-}
-
 // ---------------------------------------------------------------------------
 // Combination over orbitals: Out[n][r] = beta Out[n][r] + sum_k Coef[k][n] A[k][r]
 // (xi = W L^{-T}; K_ACE psi = -xi X).  As an MMA: D[r][n] = sum_k A^T[r][k]
@@ -845,12 +816,7 @@ cudaError_t tc_gram(int M, int N, size_t K, const float* A, size_t lda, const fl
         auto kern = absval ? tc_gram_kernel<true> : tc_gram_kernel<false>;
         kern<<<grid, TC_THREADS, TC_SMEM_BYTES, s>>>(M, N, K, A, lda, B, ldb, kchunk, work, d_err);
     }
-    const size_t tot = (size_t)M * N;
-    if (nch_eff >= 16 && tot <= 128 * 128)
-        tc_reduce_warp_kernel<<<(unsigned)((tot * 32 + 127) / 128), 128, 0, s>>>(M, N, (int)nch_eff, work, alpha, mirrored,
-                                                                         C, ldc);
-    else
-        tc_reduce_kernel<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(M, N, (int)nch_eff, work, alpha, mirrored, C, ldc);
+    chunk_sum(M, N, nch_eff, work, alpha, mirrored, TC_M, C, ldc, s);
     *launches += 2;
     if (h_err) {
         cudaMemcpyAsync(h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
