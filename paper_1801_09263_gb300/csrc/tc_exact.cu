@@ -517,7 +517,7 @@ cudaError_t combine_exact(int N, size_t K, int Kc, const float* A, const unsigne
     if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s))) return e;
     coef_cut_kernel<<<npad, 128, 0, s>>>(Kc, N, Coef, ldcoef, kpad, npad, max_a, slices, scale_a, scale_out);
     bool resident;
-    const unsigned grid = combine_grid<ExactSlices, CX_N>(K, kpad, npad, sms, &resident);
+    const unsigned grid = combine_grid<ExactSlices, CX_N>(N, K, kpad, npad, sms, &resident);
     combine_ws_kernel<ExactSlices, CX_N, float><<<grid, CW_THREADS, CombineShape<ExactSlices, CX_N>::SMEM, s>>>(
         map_a, map_c, N, K, kpad, npad, scale_a, scale_out, resident, add ? 1.f : 0.f, Out, ldo, d_err);
     *launches += 2;

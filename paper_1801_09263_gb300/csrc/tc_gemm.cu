@@ -698,7 +698,7 @@ cudaError_t combine_ws(const CUtensorMap& map_a, int N, size_t K, int kpad, int 
         if (dev < 64) attr_done.fetch_or(1ull << dev);
     }
     bool resident;
-    const unsigned grid = combine_grid<Bf16Slices, NT>(K, kpad, npad, sms, &resident);
+    const unsigned grid = combine_grid<Bf16Slices, NT>(N, K, kpad, npad, sms, &resident);
     combine_ws_kernel<Bf16Slices, NT, TO><<<grid, CW_THREADS, SMEM, s>>>(map_a, map_c, N, K, kpad, npad, nullptr, nullptr,
                                                                          resident, beta, Out, ldo, d_err);
     return cudaGetLastError();

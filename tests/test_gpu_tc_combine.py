@@ -20,7 +20,8 @@ CELL = (7.0, 8.0, 9.0)
 
 
 @pytest.mark.parametrize("n_occ,n_apply,shape", [(1, 1, (16, 15, 18)), (70, 129, (16, 15, 18)), (65, 128, (16, 16, 16)),
-                                                 (128, 190, (16, 15, 18)), (129, 190, (16, 15, 18)), (300, 3, (20, 18, 16))])
+                                                 (128, 190, (16, 15, 18)), (129, 190, (16, 15, 18)), (300, 3, (20, 18, 16)),
+                                                 (290, 300, (16, 15, 18))])
 def test_apply_matches_cuda_cores(n_occ, n_apply, shape, monkeypatch):
     rng = np.random.default_rng(n_occ + n_apply)
     phi = rng.standard_normal((n_occ,) + shape)
