@@ -21,6 +21,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "cta_sums.cuh"
 #include "grid_sync.cuh"
 #include "lace_internal.cuh"
 
@@ -368,7 +369,7 @@ template <typename T> struct NsArgs {
     const double* A;
     double* X;
     T *Y, *Z, *W, *Y2, *Z2;    // N rows of ld
-    float* part;               // one a CTA
+    float* part;               // CtaSums::kRows x kNsMaxCtas
     unsigned* bar;             // 4, zero at launch
     unsigned long long* norm;  // zero at launch
     int* status;               // 1 converged, 0 failed, -1 a barrier wait ran out (preset)
@@ -485,19 +486,24 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     if (!grid_barrier(a.bar, gen, &abort_sh)) return;
     T *Y = a.Y, *Z = a.Z, *Y2 = a.Y2, *Z2 = a.Z2;
     auto put = [&](T* M, int m, int n, T v) { __stcg(M + (size_t)m * ld + n, v); };
-    // sum over the CTAs in a fixed order: every CTA decides alike
-    auto total = [&]() {
+    // v summed over the CTAs in a fixed order, so that every CTA decides alike; false: a
+    // barrier wait ran out
+    CtaSums sums;
+    auto total = [&](float& v) {
+        if (tid == 0) __stcg(a.part + sums.at(blockIdx.x, kNsMaxCtas), v);
+        if (!grid_barrier(a.bar, gen, &abort_sh)) return false;
         float s = 0.f;
         if (warp == 0) {
-            for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + b);
+            for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + sums.at(b, kNsMaxCtas));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             if (lane == 0) sh[0] = s;
         }
         __syncthreads();
-        s = sh[0];
+        v = sh[0];
         __syncthreads();
-        return s;
+        sums.next();
+        return true;
     };
     Stop<T> stop;
     bool ok = false;
@@ -516,9 +522,8 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
                     put(a.W, m, n, T(0.5) * (T(2) * d + (d - v)));
                 });
             h = block_sum(h, sh);
-            if (tid == 0) __stcg(a.part + blockIdx.x, h);
-            if (!grid_barrier(a.bar, gen, &abort_sh)) return;
-            const int st = stop.test(total(), N);
+            if (!total(h)) return;
+            const int st = stop.test(h, N);
             if (st != 0) {
                 ok = st > 0;
                 break;
@@ -546,9 +551,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         if (ok) a.X[e] = s * z;
     }
     f = block_sum(f, sh);
-    if (tid == 0) __stcg(a.part + blockIdx.x, f);
-    if (!grid_barrier(a.bar, gen, &abort_sh)) return;
-    f = total();
+    if (!total(f)) return;
     if (me == 0) *a.status = ok && f < 1e12f ? 1 : 0;
 }
 
