@@ -33,17 +33,20 @@ constexpr int kNsMaxIt = 160;
 constexpr int kNsMaxCtas = 304;
 
 // Convergence of h = ||I - Z Y||_F^2 = sum (1 - x_k)^2 over the eigenvalues of
-// Z Y.  FP64: below 1e-24 N, or below 1e-12 N and no longer falling by 4x (the
-// rounding floor).  FP32: the same at 1e-11 N and 1e-6 N; and once below 1e-6 N
+// Z Y.  FP64: once below 1e-24 N this step is the last, for the bound leaves |1 - x_k| at
+// up to 1e-12 and a step squares it to the rounding level (without it FP64 orbitals
+// of 48^3 x 32 were off by 4e-14 instead of 4e-15); or below 1e-12 N and no longer falling
+// by 4x (the rounding floor) without another.  FP32: below 1e-11 N, or the same floor
+// below 1e-6 N; and once below 1e-6 N
 // every |1 - x_k| < 0.016 and the iteration is in its quadratic regime
 // (1 - x -> ~(3/4)(1 - x)^2), so two more steps reach the floor.
 // h is summed in FP32 (FP64 runs at 1/64 of its rate, and a sum of the squares of
 // FP64 differences needs neither its digits nor its range).
 template <typename T> struct Stop {
     float prev;
-    int extra;
+    int extra;  // steps left after this one, once they are counted
     __device__ Stop() : prev(INFINITY), extra(-1) {}
-    // the last of the two extra steps is done
+    // the last step is done
     __device__ bool done() const { return extra == 0; }
     // 1: converged, 0: go on, -1: failed
     __device__ int test(float h, int n) {
@@ -53,7 +56,12 @@ template <typename T> struct Stop {
             return 0;
         }
         if (!(h < INFINITY)) return -1;
-        if (h < lo * n || (h < hi * n && h > 0.25f * prev)) return 1;
+        if (h < lo * n) {
+            if (sizeof(T) == 4) return 1;
+            extra = 0;
+            return 0;
+        }
+        if (h < hi * n && h > 0.25f * prev) return 1;
         if (sizeof(T) == 4 && h < hi * n) extra = 1;  // this step and one more
         prev = h;
         return 0;
