@@ -551,16 +551,23 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         Z2 = t;
     }
     // ||(A/c)^{-1/2}||_F^2 >= lambda_max / lambda_min: reject ill-conditioned A
+    auto sym = [&](size_t e) {
+        return 0.5 * ((double)__ldcg(Z + (e / N) * ld + e % N) + (double)__ldcg(Z + (e % N) * ld + e / N));
+    };
     float f = 0.f;
-    const double s = 1.0 / sqrt(c);
     for (size_t e = me; e < (size_t)N * N; e += all) {
-        const double z = 0.5 * ((double)__ldcg(Z + (e / N) * ld + e % N) + (double)__ldcg(Z + (e % N) * ld + e / N));
-        f = fmaf((float)z, (float)z, f);
-        if (ok) a.X[e] = s * z;
+        const float z = (float)sym(e);
+        f = fmaf(z, z, f);
     }
     f = block_sum(f, sh);
     if (!total(f)) return;
-    if (me == 0) *a.status = ok && f < 1e12f ? 1 : 0;
+    ok = ok && f < 1e12f;
+    const double s = 1.0 / sqrt(c);
+    if (ok)
+        for (size_t e = me; e < (size_t)N * N; e += all) a.X[e] = s * sym(e);
+    // (a CTA whose wait for the sum ran out has not written its share)
+    if (!grid_barrier(a.bar, gen, &abort_sh)) return;
+    if (me == 0) *a.status = ok ? 1 : 0;
 }
 
 template <int RB> cudaError_t ns_cluster(int N, const double* A, double* X, int* d_status, cudaStream_t s) {
