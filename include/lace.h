@@ -85,14 +85,15 @@ lace_status lace_destroy(lace_ctx* ctx);
 lace_status lace_set_stream(lace_ctx* ctx, void* stream);
 
 /* Time limit, in seconds (0 to 3600; default 2), of each bounded device
- * wait of this context's persistent pivoted-QR kernel (lace_localize): a
- * grid-barrier wait for the other CTAs of the launch.  A wait that runs out
- * sets an error flag and its CTA leaves the kernel (the others then run out
- * at their next barrier and leave too); lace_localize returns
- * LACE_ERR_TIMEOUT and the context stays usable, with its orbitals loaded
- * but not localised (localise again).  A short limit turns a stalled
- * launch into an error quickly; 0 makes every wait that has to wait at all
- * give up.
+ * wait of this context's persistent kernels, a grid-barrier wait for the other
+ * CTAs of the launch: the pivoted QR (lace_localize) and the inverse square
+ * roots of more than 64 rows (FP64: 16) of a load, a localisation and an
+ * alignment.  A wait that runs out sets an error status and its CTA leaves the
+ * kernel (the others then run out at their next barrier and leave too); the call
+ * returns LACE_ERR_TIMEOUT and the context stays usable, in the state of a call
+ * that failed: nothing loaded, orbitals loaded but not localised, or localised
+ * orbitals as they were (call again).  A short limit turns a stalled launch into
+ * an error quickly; 0 makes every wait that has to wait at all give up.
  * Returns LACE_ERR_ARG for a limit outside [0, 3600]. */
 lace_status lace_set_wait_limit(lace_ctx* ctx, double seconds);
 

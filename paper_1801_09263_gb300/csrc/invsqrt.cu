@@ -380,6 +380,7 @@ template <typename T> struct NsArgs {
     float* part;               // CtaSums::kRows x kNsMaxCtas
     unsigned* bar;             // 4, zero at launch
     unsigned long long* norm;  // zero at launch
+    unsigned long long limit_ns;  // of a barrier wait
     int* status;               // 1 converged, 0 failed, -1 a barrier wait ran out (preset)
 };
 
@@ -470,7 +471,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) atomicMax(a.norm, (unsigned long long)__double_as_longlong(s));  // (a NaN is the largest)
     }
-    if (!grid_barrier(a.bar, gen, &abort_sh)) return;
+    if (!grid_barrier(a.bar, gen, &abort_sh, a.limit_ns)) return;
     const double c = __longlong_as_double((long long)__ldcg(a.norm));
     if (!(c > 0.0) || !(c < INFINITY)) {
         if (me == 0) *a.status = 0;
@@ -491,7 +492,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
         __stcg(a.Y2 + e, T(0));  // (the padding of the rows stays zero)
         __stcg(a.Z + e, T(0));
     }
-    if (!grid_barrier(a.bar, gen, &abort_sh)) return;
+    if (!grid_barrier(a.bar, gen, &abort_sh, a.limit_ns)) return;
     T *Y = a.Y, *Z = a.Z, *Y2 = a.Y2, *Z2 = a.Z2;
     auto put = [&](T* M, int m, int n, T v) { __stcg(M + (size_t)m * ld + n, v); };
     // v summed over the CTAs in a fixed order, so that every CTA decides alike; false: a
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     CtaSums sums;
     auto total = [&](float& v) {
         if (tid == 0) __stcg(a.part + sums.at(blockIdx.x, kNsMaxCtas), v);
-        if (!grid_barrier(a.bar, gen, &abort_sh)) return false;
+        if (!grid_barrier(a.bar, gen, &abort_sh, a.limit_ns)) return false;
         float s = 0.f;
         if (warp == 0) {
             for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + sums.at(b, kNsMaxCtas));
@@ -542,7 +543,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
             if (t < tiles) grid_product<T>(N, ld, Y, a.W, bm, bn, smem, [&](int m, int n, T v) { put(Y2, m, n, v); });
             else grid_product<T>(N, ld, a.W, Z, bm, bn, smem, [&](int m, int n, T v) { put(Z2, m, n, v); });
         }
-        if (!grid_barrier(a.bar, gen, &abort_sh)) return;
+        if (!grid_barrier(a.bar, gen, &abort_sh, a.limit_ns)) return;
         T* t = Y;
         Y = Y2;
         Y2 = t;
@@ -566,7 +567,7 @@ __global__ void __launch_bounds__(kNsThreads) ns_grid_kernel(NsArgs<T> a) {
     if (ok)
         for (size_t e = me; e < (size_t)N * N; e += all) a.X[e] = s * sym(e);
     // (a CTA whose wait for the sum ran out has not written its share)
-    if (!grid_barrier(a.bar, gen, &abort_sh)) return;
+    if (!grid_barrier(a.bar, gen, &abort_sh, a.limit_ns)) return;
     if (me == 0) *a.status = ok ? 1 : 0;
 }
 
@@ -581,7 +582,8 @@ template <int RB> cudaError_t ns_cluster(int N, const double* A, double* X, int*
 
 // X = A^{-1/2}; work: five N x ld matrices of T, then the control words.
 template <typename T>
-cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s, int* launches) {
+cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, unsigned long long wait_limit_ns, int* d_status,
+                     cudaStream_t s, int* launches) {
     const int ld = sizeof(T) == 4 ? (N + 3) / 4 * 4 : N;
     const size_t mat = ((size_t)N * ld * sizeof(T) + 15) / 16 * 16;
     unsigned char* w = reinterpret_cast<unsigned char*>(((uintptr_t)work + 15) & ~(uintptr_t)15);
@@ -611,6 +613,7 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* d_sta
         a.status = d_status;
         a.bar = reinterpret_cast<unsigned*>(ctl + 16);
         a.norm = reinterpret_cast<unsigned long long*>(ctl + 32);
+        a.limit_ns = wait_limit_ns;
         a.part = reinterpret_cast<float*>(ctl + 64);
         int dev = 0, sms = 0, per_sm = 0;
         cudaGetDevice(&dev);
@@ -630,13 +633,13 @@ cudaError_t inv_sqrt(int N, const double* A, double* X, double* work, int* d_sta
 
 }  // namespace
 
-cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
-                         int* launches) {
-    return inv_sqrt<double>(N, A, X, work, d_status, s, launches);
+cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, unsigned long long wait_limit_ns, int* d_status,
+                         cudaStream_t s, int* launches) {
+    return inv_sqrt<double>(N, A, X, work, wait_limit_ns, d_status, s, launches);
 }
-cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
-                               int* launches) {
-    return inv_sqrt<float>(N, A, X, work, d_status, s, launches);
+cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, unsigned long long wait_limit_ns,
+                               int* d_status, cudaStream_t s, int* launches) {
+    return inv_sqrt<float>(N, A, X, work, wait_limit_ns, d_status, s, launches);
 }
 
 }  // namespace lace

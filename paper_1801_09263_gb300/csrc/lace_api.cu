@@ -293,14 +293,14 @@ lace_status orbital_combine(lace_ctx* c, int N, size_t K, int Kc, const T* A, co
 lace_status inv_sqrt_queue(lace_ctx* c, int n, const double* A, double* X, bool mixed, int k, const char* where, Launch& L) {
     int* d = c->flag.as<int>() + kFlagSlots + k;
     *c->status(k) = -1;
-    CK(mixed ? inv_sqrt_spd_mixed(n, A, X, c->m(MS_NSWORK), d, c->stream, &L.n)
-             : inv_sqrt_spd(n, A, X, c->m(MS_NSWORK), d, c->stream, &L.n),
+    CK(mixed ? inv_sqrt_spd_mixed(n, A, X, c->m(MS_NSWORK), c->wait_limit_ns, d, c->stream, &L.n)
+             : inv_sqrt_spd(n, A, X, c->m(MS_NSWORK), c->wait_limit_ns, d, c->stream, &L.n),
        where);
     CK(cudaMemcpyAsync(c->status(k), d, sizeof(int), cudaMemcpyDeviceToHost, c->stream), where);
     return LACE_OK;
 }
 lace_status inv_sqrt_result(lace_ctx* c, int k, const char* where, const char* not_pd) {
-    if (*c->status(k) < 0) CK(cudaErrorLaunchTimeout, where);  // a barrier wait ran out
+    if (*c->status(k) < 0) return fail(c, LACE_ERR_TIMEOUT, std::string(where) + ": a grid barrier wait timed out");
     return *c->status(k) == 1 ? LACE_OK : fail(c, LACE_ERR_NOT_PD, not_pd);
 }
 

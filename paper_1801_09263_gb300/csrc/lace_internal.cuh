@@ -207,13 +207,15 @@ cudaError_t small_gemm_f64(int M, int N, int K, const double* A, int lda, bool t
                            double alpha, double beta, double* C, int ldc, cudaStream_t s, int* launches);
 // X = A^{-1/2} of a symmetric positive definite A by the coupled Newton-Schulz
 // iteration.  *d_status (read it after a synchronisation): 1 converged, 0 not (X is not
-// written), -1 a grid-barrier wait ran out of time.
+// written), -1 a grid-barrier wait ran out of time (wait_limit_ns bounds each; parts of X
+// may be written).
 // (invsqrt.cu; work: 5 N^2 + 320 N + 320 doubles)
-cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s, int* launches);
+cudaError_t inv_sqrt_spd(int N, const double* A, double* X, double* work, unsigned long long wait_limit_ns, int* d_status,
+                         cudaStream_t s, int* launches);
 // Mixed-precision variant: FP32 Newton-Schulz to ~1e-7, returns X0 ~ A^{-1/2}
 // (FP64, symmetric).  Pair it with lowdin_refine.
-cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, int* d_status, cudaStream_t s,
-                               int* launches);
+cudaError_t inv_sqrt_spd_mixed(int N, const double* A, double* X, double* work, unsigned long long wait_limit_ns,
+                               int* d_status, cudaStream_t s, int* launches);
 // F <- F (I - E/2), E = F^T G F - I (G = I when null): orthonormality to O(E^2).
 cudaError_t lowdin_refine(int N, double* F, const double* G, double* work, cudaStream_t s, int* launches);
 // In-place lower Cholesky of A (N x N, lda); *ok = 0 when not positive definite.

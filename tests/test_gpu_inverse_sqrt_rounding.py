@@ -55,8 +55,8 @@ def just_passing(n, seed):
 @pytest.mark.parametrize("n", [4, 16, 17, 24, 40, 130])
 def test_fp64_inverse_sqrt_reaches_rounding(n):
     torch = pytest.importorskip("torch")
-    fn = B.load_library()._ZN4lace12inv_sqrt_spdEiPKdPdS2_PiP11CUstream_stS3_
-    fn.argtypes = [C.c_int] + [C.c_void_p] * 6
+    fn = B.load_library()._ZN4lace12inv_sqrt_spdEiPKdPdS2_yPiP11CUstream_stS3_
+    fn.argtypes = [C.c_int] + [C.c_void_p] * 3 + [C.c_ulonglong] + [C.c_void_p] * 3
     for seed in range(4):
         mat = just_passing(n, seed)
         a = torch.from_numpy(mat).cuda()
@@ -65,7 +65,8 @@ def test_fp64_inverse_sqrt_reaches_rounding(n):
         status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
         torch.cuda.synchronize()
         launches = C.c_int(0)
-        assert fn(n, a.data_ptr(), x.data_ptr(), work.data_ptr(), status.data_ptr(), None, C.addressof(launches)) == 0
+        assert fn(n, a.data_ptr(), x.data_ptr(), work.data_ptr(), 2 * 10**9, status.data_ptr(), None,
+                  C.addressof(launches)) == 0
         torch.cuda.synchronize()
         assert int(status.item()) == 1
         x = x.cpu().numpy()
