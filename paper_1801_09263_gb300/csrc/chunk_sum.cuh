@@ -35,8 +35,10 @@ __global__ void __launch_bounds__(32 * kSumWarps) chunk_sum_kernel(int M, int N,
     C[(size_t)m * ldc + n] = alpha * s;
 }
 
-cudaError_t chunk_sum(int M, int N, size_t nchunk, const double* work, double alpha, bool sym, int tile, double* C, int ldc,
-                      cudaStream_t s) {
+// Returns the error of its own launch or of one before it (reading clears it, so the
+// caller has to pass it on).
+[[nodiscard]] cudaError_t chunk_sum(int M, int N, size_t nchunk, const double* work, double alpha, bool sym, int tile, double* C,
+                                    int ldc, cudaStream_t s) {
     chunk_sum_kernel<<<(unsigned)(((size_t)M * N + 31) / 32), 32 * kSumWarps, 0, s>>>(M, N, (int)nchunk, work, alpha, sym, tile,
                                                                                       C, ldc);
     return cudaGetLastError();

@@ -917,9 +917,8 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
         const size_t nc = (K + kc - 1) / kc;
         gemm_rows_f64_kernel<<<dim3((unsigned)f64_tiles(M, N, sym), (unsigned)nc), 32 * GD_WARPS, 0, s>>>(
             M, N, K, A, lda, B, ldb, absval, sym, kc, work);
-        chunk_sum(M, N, nc, work, alpha, sym, GD_T, C, ldc, s);
         *launches += 2;
-        return cudaGetLastError();
+        return chunk_sum(M, N, nc, work, alpha, sym, GD_T, C, ldc, s);
     }
     // as many chunks as the workspace holds, up to the balanced count
     const size_t nch = std::min(n_chunks_for(M, N, K, sym), work_elems / ((size_t)M * N));
@@ -940,9 +939,8 @@ cudaError_t gemm_rows(int M, int N, size_t K, const T* A, size_t lda, const T* B
     } else {
         gemm_rows_kernel<T, false><<<grid, GR_THREADS, 0, s>>>(M, N, K, A, lda, B, ldb, absval, sym, kchunk, work);
     }
-    chunk_sum(M, N, nch_eff, work, alpha, sym, GR_BM, C, ldc, s);
     *launches += 2;
-    return cudaGetLastError();
+    return chunk_sum(M, N, nch_eff, work, alpha, sym, GR_BM, C, ldc, s);
 }
 
 template <typename T>
@@ -995,18 +993,21 @@ cudaError_t lowdin_refine(int N, double* F, const double* G, double* work, cudaS
     double* E = work + nn;
     double* F2 = work + 2 * nn;
     const double* rhs = F;
+    cudaError_t e;
     if (G) {
-        small_gemm_f64(N, N, N, G, N, false, F, N, false, 1.0, 0.0, GF, N, s, launches);
+        if ((e = small_gemm_f64(N, N, N, G, N, false, F, N, false, 1.0, 0.0, GF, N, s, launches))) return e;
         rhs = GF;
     }
-    small_gemm_f64(N, N, N, F, N, true, rhs, N, false, -0.5, 0.0, E, N, s, launches);
-    small_gemm_f64(N, N, N, F, N, false, E, N, false, 1.0, 0.0, F2, N, s, launches);
+    if ((e = small_gemm_f64(N, N, N, F, N, true, rhs, N, false, -0.5, 0.0, E, N, s, launches)) ||
+        (e = small_gemm_f64(N, N, N, F, N, false, E, N, false, 1.0, 0.0, F2, N, s, launches)))
+        return e;
     axpby_kernel<<<(int)((nn + 255) / 256), 256, 0, s>>>((int)nn, F2, 1.5, F);
     *launches += 1;
     return cudaGetLastError();
 }
 
 cudaError_t cholesky_lower(int N, double* A, int lda, int* d_flag, int* ok, cudaStream_t s, int* launches) {
+    cudaError_t e;
     cudaMemsetAsync(d_flag, 0, sizeof(int), s);
     for (int k0 = 0; k0 < N; k0 += CH_NB) {
         const int nb = std::min(CH_NB, N - k0);
@@ -1019,15 +1020,15 @@ cudaError_t cholesky_lower(int N, double* A, int lda, int* d_flag, int* ok, cuda
             // A22 -= L21 L21^T
             double* L21 = A + (size_t)(k0 + nb) * lda + k0;
             double* A22 = A + (size_t)(k0 + nb) * lda + k0 + nb;
-            small_gemm_f64(rem, rem, nb, L21, lda, false, L21, lda, true, -1.0, 1.0, A22, lda, s, launches);
+            if ((e = small_gemm_f64(rem, rem, nb, L21, lda, false, L21, lda, true, -1.0, 1.0, A22, lda, s, launches))) return e;
         }
     }
     zero_upper_kernel<<<(N * N + 255) / 256, 256, 0, s>>>(N, A, lda);
     *launches += 1;
-    if (!ok) return cudaGetLastError();  // deferred: the caller reads d_flag (0 = positive definite)
+    if ((e = cudaGetLastError()) || !ok) return e;  // !ok: the caller reads d_flag (0 = positive definite)
     int h = 0;
     cudaMemcpyAsync(&h, d_flag, sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaError_t e = cudaStreamSynchronize(s);
+    e = cudaStreamSynchronize(s);
     *ok = (h == 0);
     return e;
 }
@@ -1044,14 +1045,17 @@ cudaError_t trtri_lower(int N, const double* L, int ldl, double* X, int ldx, cud
     // unused upper-right area is not safe; so two steps with a small staging
     // area at the end of X's allocation (caller provides ldx*N + CH_NB*N).
     double* stage = X + (size_t)N * ldx;
+    cudaError_t e;
     for (int bi = 1; bi < nblk; ++bi) {
         const int i0 = bi * CH_NB;
         const int nb = std::min(CH_NB, N - i0);
         // stage[nb x i0] = L[i0:i0+nb, 0:i0] * X[0:i0, 0:i0]
-        small_gemm_f64(nb, i0, i0, L + (size_t)i0 * ldl, ldl, false, X, ldx, false, 1.0, 0.0, stage, i0, s, launches);
+        e = small_gemm_f64(nb, i0, i0, L + (size_t)i0 * ldl, ldl, false, X, ldx, false, 1.0, 0.0, stage, i0, s, launches);
+        if (e) return e;
         // X[i0:i0+nb, 0:i0] = -X_ii * stage
-        small_gemm_f64(nb, i0, nb, X + (size_t)i0 * ldx + i0, ldx, false, stage, i0, false, -1.0, 0.0,
-                       X + (size_t)i0 * ldx, ldx, s, launches);
+        e = small_gemm_f64(nb, i0, nb, X + (size_t)i0 * ldx + i0, ldx, false, stage, i0, false, -1.0, 0.0,
+                           X + (size_t)i0 * ldx, ldx, s, launches);
+        if (e) return e;
     }
     return cudaGetLastError();
 }

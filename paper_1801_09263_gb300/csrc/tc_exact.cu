@@ -481,9 +481,8 @@ cudaError_t gram_exact(int M, int N, size_t K, const float* A, const unsigned* m
     if ((e = cudaMemsetAsync(d_err, 0, sizeof(int), s))) return e;
     gram_exact_kernel<<<dim3((unsigned)exact_tiles(M, N, sym), 1, (unsigned)nch_eff), GX_THREADS, GX_SMEM_BYTES, s>>>(
         map_a, map_b, M, N, K, kchunk, (M + TC_M - 1) / TC_M, sym, max_a, max_b, work, d_err);
-    chunk_sum(M, N, nch_eff, work, alpha, sym, TC_M, C, ldc, s);
     *launches += 2;
-    return cudaGetLastError();
+    return chunk_sum(M, N, nch_eff, work, alpha, sym, TC_M, C, ldc, s);
 }
 
 size_t combine_exact_scratch_bytes(int N, int Kc) {

@@ -816,14 +816,11 @@ cudaError_t tc_gram(int M, int N, size_t K, const float* A, size_t lda, const fl
         auto kern = absval ? tc_gram_kernel<true> : tc_gram_kernel<false>;
         kern<<<grid, TC_THREADS, TC_SMEM_BYTES, s>>>(M, N, K, A, lda, B, ldb, kchunk, work, d_err);
     }
-    chunk_sum(M, N, nch_eff, work, alpha, mirrored, TC_M, C, ldc, s);
     *launches += 2;
-    if (h_err) {
-        cudaMemcpyAsync(h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s);
-        cudaError_t e = cudaStreamSynchronize(s);
-        if (e) return e;
-    }
-    return cudaGetLastError();
+    cudaError_t e = chunk_sum(M, N, nch_eff, work, alpha, mirrored, TC_M, C, ldc, s);
+    if (e || !h_err) return e;
+    if ((e = cudaMemcpyAsync(h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s))) return e;
+    return cudaStreamSynchronize(s);
 }
 
 template cudaError_t tc_combine<float>(int, size_t, int, const float*, size_t, const double*, int, double, float*,
