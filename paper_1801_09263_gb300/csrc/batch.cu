@@ -65,8 +65,8 @@ cudaError_t ace_build_deferred(lace_ctx* c, cudaStream_t s, int* launches) {
     double* LinvT = c->m(MS_LINVT);
     int* f = c->flag.as<int>();
     cudaError_t e;
-    const bool aligned = ng % 4 == 0 && (uintptr_t)psi % 16 == 0 && (uintptr_t)W % 16 == 0;
-    if (aligned) {
+    const bool tc = ace_on_tc(n, ng), aligned = ng % 4 == 0 && (uintptr_t)psi % 16 == 0 && (uintptr_t)W % 16 == 0;
+    if (aligned && tc) {
         e = tc_gram(n, n, ng, psi, ng, W, ng, c->g.dv, M, n, c->work.as<double>(), c->work.bytes / sizeof(double),
                     f + 0, nullptr, s, launches);
     } else {
@@ -80,7 +80,9 @@ cudaError_t ace_build_deferred(lace_ctx* c, cudaStream_t s, int* launches) {
     if ((e = cudaMemcpyAsync(c->m(MS_L), A, sizeof(double) * n * n, cudaMemcpyDeviceToDevice, s))) return e;
     if ((e = trtri_lower(n, A, n, Linv, n, s, launches))) return e;
     if ((e = transpose_f64(n, Linv, LinvT, s, launches))) return e;
-    return tc_combine(n, ng, n, W, ng, LinvT, n, 0.0, c->xi.as<float>(), ng, c->work.p, f + 2, nullptr, s, launches);
+    if (tc) return tc_combine(n, ng, n, W, ng, LinvT, n, 0.0, c->xi.as<float>(), ng, c->work.p, f + 2, nullptr, s, launches);
+    if ((e = cudaMemsetAsync(f + 2, 0, sizeof(int), s))) return e;
+    return gemm_combine<float>(n, ng, n, W, ng, LinvT, n, 0.0, c->xi.as<float>(), ng, s, launches);
 }
 
 }  // namespace

@@ -715,18 +715,6 @@ lace_status exchange_finish(lace_ctx* c) {
 }
 
 // ------------------------------------------------------------------ ACE
-// Whether an ACE contraction or combination with this many rows (the longer side)
-// takes the tensor cores: few short rows are faster on the CUDA cores, whose chain
-// of launches and pipeline fills is shorter.  ACE build + apply, CUDA cores and
-// tensor cores: 32^3 x 16 128 and 164 us, 32^3 x 64 239 and 271, 48^3 x 16 196 and 218;
-// 48^3 x 32 234 and 241, 40^3 x 64 282 and 288, 48^3 x 64 342 and 327, 64^3 x 16 299 and
-// 297.  LACE_NO_TC=0 takes them at every size.
-bool ace_on_tc(size_t rows, size_t K) {
-    if (tc_off()) return false;
-    const char* e = getenv("LACE_NO_TC");
-    return (e && e[0] == '0') || K >= (1u << 17) || rows * K >= 3000000;
-}
-
 // Dense contraction over the grid for the ACE matrices: tcgen05 3xBF16 on the
 // mixed path (LACE_NO_TC=1 selects the CUDA-core FP32 kernel), FP64 otherwise.
 // The tensor-core kernel reads rows with 16-byte loads, so grids whose point
@@ -736,7 +724,7 @@ lace_status ace_contract(lace_ctx* c, int M, int N, const T* A, const T* B, doub
     const size_t ng = c->g.ng;
     if constexpr (std::is_same<T, float>::value) {
         const bool aligned = ng % 4 == 0 && (uintptr_t)A % 16 == 0 && (uintptr_t)B % 16 == 0;
-        if (aligned && ace_on_tc(std::max(M, N), ng)) {
+        if (aligned && ace_on_tc(c->n_p, ng)) {
             CK(c->work.ensure(std::max(c->work.bytes, tc_gram_work_elems(M, N, ng) * sizeof(double))), "alloc work");
             TcFlag f = tc_flag(c);
             CK(tc_gram(M, N, ng, A, ng, B, ng, alpha, C, N, c->work.as<double>(), c->work.bytes / sizeof(double),
@@ -763,7 +751,7 @@ template <typename T, typename TO>
 lace_status ace_combine(lace_ctx* c, int N, int Kc, const T* A, const double* Coef, TO* Out, Launch& L) {
     const size_t ng = c->g.ng;
     if constexpr (std::is_same<T, float>::value) {
-        if (ace_on_tc(std::max(N, Kc), ng)) {
+        if (ace_on_tc(c->n_p, ng)) {
             CK(c->work.ensure(std::max(c->work.bytes, tc_combine_scratch_bytes(N, Kc))), "alloc work");
             TcFlag f = tc_flag(c);
             CK(tc_combine(N, ng, Kc, A, ng, Coef, N, 0.0, Out, ng, c->work.p, f.d, f.h, c->stream, &L.n),
@@ -867,6 +855,12 @@ lace_status copy_orbitals_out(lace_ctx* c, const T* src, size_t count, double* h
 namespace lace {
 
 lace_status ctx_fail(lace_ctx* c, lace_status st, const std::string& msg) { return fail(c, st, msg); }
+
+bool ace_on_tc(int n_p, size_t ng) {
+    if (tc_off()) return false;
+    const char* e = getenv("LACE_NO_TC");
+    return (e && e[0] == '0') || ng >= (1u << 17) || (size_t)n_p * ng >= 3000000;
+}
 
 bool ctx_mergeable(lace_ctx* c) {
     return c && c->prec == LACE_MIXED && c->loaded && c->g.n[0] == c->g.n[1] && c->g.n[1] == c->g.n[2] &&

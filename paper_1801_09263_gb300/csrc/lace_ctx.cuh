@@ -120,6 +120,15 @@ struct lace_ctx {
 namespace lace {
 // Shared with the other translation units (defined in lace_api.cu).
 lace_status ctx_fail(lace_ctx* c, lace_status st, const std::string& msg);
+// Whether the contractions and combinations of an ACE projector of n_p orbitals take
+// the tensor cores (mixed precision): few short rows are faster on the CUDA cores,
+// whose chain of launches and pipeline fills is shorter.  ACE build + apply, CUDA cores
+// and tensor cores: 32^3 x 16 128 and 164 us, 32^3 x 64 239 and 271, 48^3 x 16 196 and 218;
+// 48^3 x 32 234 and 241, 40^3 x 64 282 and 288, 48^3 x 64 342 and 327, 64^3 x 16 299 and
+// 297.  The projector alone decides, for its builds, whole or in a batch, and for every
+// block that it is applied to: the two differ in accuracy (2e-7 and 8e-6 of the
+// largest value).  LACE_NO_TC=0 takes them at every size, LACE_NO_TC=1 at none.
+bool ace_on_tc(int n_p, size_t ng);
 // lace_load_orbitals from FP64 device memory (borrowed for the call)
 lace_status ctx_load_dev64(lace_ctx* c, const double* d_phi, int n_occ, int n_extra, int ortho);
 // device pointer of PSI / W / XI (working precision, [n_p][ng]) after the state checks
