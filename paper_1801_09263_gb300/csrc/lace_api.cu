@@ -924,8 +924,8 @@ lace_status ctx_orbitals(lace_ctx* c, int which, const void** src) {
 // Device bytes a context holds after loading n_occ + n_extra orbitals on an
 // n[0] x n[1] x n[2] grid, localising them (stride 2), screening, applying the
 // exchange, building ACE and applying it to n_apply host functions: the
-// buffers of the calls above at their largest (the tables excepted, which
-// are far smaller than one orbital).
+// buffers of the calls above at their largest (a few KB of axis tables, counters
+// and lists excepted).
 size_t predict_ctx_bytes(int prec, const int n[3], int n_occ, int n_extra, int n_apply, size_t fft_budget) {
     const size_t ng = (size_t)n[0] * n[1] * n[2], eb = prec == LACE_FP64 ? 8 : 4;
     const size_t n_p = (size_t)n_occ + n_extra, na = (size_t)std::max(n_apply, 0);
@@ -959,7 +959,8 @@ size_t predict_ctx_bytes(int prec, const int n[3], int n_occ, int n_extra, int n
     b += mslot * kMatSlots * sizeof(double) + work + qrcp_aux_bytes(n_occ, (int)ncol);
     b += maxp * 8 + (maxp + 1) / 2 * sizeof(PairGrid);
     b += std::max(batch * ng * 2 * eb, 2 * na * ng * eb) + batch * n[0] * 2 * sizeof(double);
-    b += 2 * na * ng * sizeof(double) + ng * (sizeof(float) + sizeof(double));
+    b += 2 * na * ng * sizeof(double) + ng * (sizeof(float) + sizeof(double));  // ... and K(G) tables
+    if (prec != LACE_FP64 && lanes_ok(n)) b += ng * sizeof(float);               // in the order of the lane passes
     return b;
 }
 
