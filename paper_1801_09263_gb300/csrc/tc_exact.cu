@@ -82,7 +82,7 @@ __device__ __forceinline__ uint32_t f16x2_rn(float x0, float x1) {
 
 // Power of two that brings a row with this largest magnitude (FP32 bits) to
 // below 256, and its inverse's exponent: scale = 2^(134 - E), E the biased
-// exponent.  Rows of zeros, infinities or NaN: 1 (they stay what they are).
+// exponent.  Rows without a finite value but zero: 1.
 __host__ __device__ __forceinline__ int row_exponent(unsigned maxbits) {
     const int e = (int)(maxbits >> 23) & 0xff;
     if (e == 0 || e == 255) return 0;
@@ -394,15 +394,17 @@ struct ExactSlices {
 };
 
 // ------------------------------------------------------------------ row maxima
-// out[row] = bits of the largest |x| of the row (zeroed before); Tin = double:
-// the row is also rounded to FP32 into dst (the load's conversion).
+// out[row] = bits of the largest finite |x| of the row (zeroed before; infinities
+// and NaN reach the results at their own points whatever the scale, and must not set
+// that of the other points); Tin = double: the row is also rounded to FP32 into
+// dst (the load's conversion).
 template <typename Tin>
 __global__ void row_max_kernel(const Tin* __restrict__ src, float* __restrict__ dst, size_t n, unsigned* __restrict__ out) {
     const size_t row = blockIdx.y, q4 = n / 4;
     const Tin* s = src + row * n;
     float* d = dst + row * n;
     float m = 0.f;
-    auto use = [&](float x) { m = fmaxf(m, fabsf(x)); if (x != x) m = INFINITY; };
+    auto use = [&](float x) { m = fabsf(x) < INFINITY ? fmaxf(m, fabsf(x)) : m; };
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < q4; q += (size_t)gridDim.x * blockDim.x) {
         float4 v;
         if constexpr (sizeof(Tin) == 8) {
