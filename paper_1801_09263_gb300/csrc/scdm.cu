@@ -121,34 +121,29 @@ __global__ void __launch_bounds__(QR_THREADS) qr_select_kernel(int nrow, int nbl
     }
 }
 
-// Persistent pivoted QR: one cooperative launch runs every step, one CTA of
+// Persistent pivoted QR in FP64: one cooperative launch runs every step, one CTA of
 // 512 threads (16 warps) per SM.  A group of wpt warps owns 32-column tiles
 // (lane = column); warp w of the group holds rows w*RPW .. w*RPW+RPW-1 of a
-// tile.  The matrix stays on chip across the steps where it fits: the first
-// NREG tiles of a group live in registers, the next nsm tiles in shared
-// memory, and only the rest is streamed from and back to global memory
-// every step.  A step forms q.r (partial sums exchanged through shared
-// memory behind the group's named barrier), updates the column, forms its
-// exact new norm and the group's argmax; each CTA then publishes its best
-// column's values, so one grid-wide barrier per step suffices: after it,
-// every CTA picks the global winner and reads the winner's published column
-// as the next q.  Block winners and published columns are double-buffered by
-// step parity.
-constexpr int QC_THREADS = 512, QC_WARPS = 16, QC_MAXROWS = 1024;
+// tile.  The first nsm tiles of a group stay in shared memory across the steps,
+// and only the rest is streamed from and back to global memory every step.  A
+// step forms q.r (partial sums exchanged through shared memory behind the
+// group's named barrier), updates the column, forms its exact new norm and the
+// group's argmax; each CTA then publishes its best column's values, so one
+// grid-wide barrier per step suffices: after it, every CTA picks the global
+// winner and reads the winner's published column as the next q.  Block winners
+// and published columns are double-buffered by step parity.
+constexpr int QC_THREADS = 512, QC_WARPS = 16, RPW = 32, QC_MAXROWS = QC_WARPS * RPW;
+static_assert(QC_MAXROWS <= QC_THREADS, "a published row a thread");
 
 __device__ __forceinline__ void best_merge(double& v, int& i, double v2, int i2) {
     if (better(v2, i2, v, i)) { v = v2; i = i2; }
 }
 
-template <typename T> struct Vec4 {
-    T a, b, c, d;
+struct Vec4 {
+    double a, b, c, d;
 };
 // four consecutive shared-memory values as 16-byte loads (16-byte aligned p)
-__device__ __forceinline__ Vec4<float> load4(const float* p) {
-    const float4 v = *reinterpret_cast<const float4*>(p);
-    return {v.x, v.y, v.z, v.w};
-}
-__device__ __forceinline__ Vec4<double> load4(const double* p) {
+__device__ __forceinline__ Vec4 load4(const double* p) {
     const double2 v0 = *reinterpret_cast<const double2*>(p), v1 = *reinterpret_cast<const double2*>(p + 2);
     return {v0.x, v0.y, v1.x, v1.y};
 }
@@ -158,12 +153,11 @@ __device__ __forceinline__ void group_bar(int id, int nthreads) {
 }
 
 // q . v over this warp's RPW rows, four independent partial sums
-template <typename T, int RPW>
-__device__ __forceinline__ T dot_rows(const T* v, const T* qs, int rbase) {
-    T p0 = T(0), p1 = T(0), p2 = T(0), p3 = T(0);
+__device__ __forceinline__ double dot_rows(const double* v, const double* qs, int rbase) {
+    double p0 = 0.0, p1 = 0.0, p2 = 0.0, p3 = 0.0;
 #pragma unroll
     for (int j = 0; j < RPW; j += 4) {
-        const Vec4<T> q4 = load4(qs + rbase + j);
+        const Vec4 q4 = load4(qs + rbase + j);
         p0 += q4.a * v[j];
         p1 += q4.b * v[j + 1];
         p2 += q4.c * v[j + 2];
@@ -173,12 +167,11 @@ __device__ __forceinline__ T dot_rows(const T* v, const T* qs, int rbase) {
 }
 
 // v -= q dot over the warp's rows, and the new squared norm of v
-template <typename T, int RPW>
-__device__ __forceinline__ T update_rows(T* v, const T* qs, int rbase, T dot) {
-    T n0 = T(0), n1 = T(0), n2 = T(0), n3 = T(0);
+__device__ __forceinline__ double update_rows(double* v, const double* qs, int rbase, double dot) {
+    double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;
 #pragma unroll
     for (int j = 0; j < RPW; j += 4) {
-        const Vec4<T> q4 = load4(qs + rbase + j);
+        const Vec4 q4 = load4(qs + rbase + j);
         v[j] -= q4.a * dot;
         v[j + 1] -= q4.b * dot;
         v[j + 2] -= q4.c * dot;
@@ -191,9 +184,8 @@ __device__ __forceinline__ T update_rows(T* v, const T* qs, int rbase, T dot) {
     return (n0 + n1) + (n2 + n3);
 }
 
-template <typename T, int RPW>
-__device__ __forceinline__ T norm_rows(const T* v) {
-    T n0 = T(0), n1 = T(0), n2 = T(0), n3 = T(0);
+__device__ __forceinline__ double norm_rows(const double* v) {
+    double n0 = 0.0, n1 = 0.0, n2 = 0.0, n3 = 0.0;
 #pragma unroll
     for (int j = 0; j < RPW; j += 4) {
         n0 += v[j] * v[j];
@@ -214,19 +206,17 @@ __device__ __forceinline__ void tile_argmax(double cv, int ci, double& best, int
     best_merge(best, bidx, cv, ci);
 }
 
-template <typename T, int RPW, int NREG>
 __global__ void __launch_bounds__(QC_THREADS, 1)
-    qr_persistent_kernel(int nrow, int ncol, T* __restrict__ R, int npiv, int wpt, int nsm,
-                         Best* __restrict__ block_best, T* __restrict__ pub, unsigned char* __restrict__ chosen,
+    qr_persistent_kernel(int nrow, int ncol, double* __restrict__ R, int npiv, int wpt, int nsm,
+                         Best* __restrict__ block_best, double* __restrict__ pub, unsigned char* __restrict__ chosen,
                          int* __restrict__ piv, unsigned* bar, unsigned long long limit_ns) {
     extern __shared__ __align__(16) unsigned char qr_smem_raw[];
     const int ngroups = QC_WARPS / wpt;
-    const int kres_max = NREG + nsm;                 // resident tiles per group at most
-    T* stiles = reinterpret_cast<T*>(qr_smem_raw);  // [ngroups][nsm][wpt][RPW][32]
-    T* pdot = stiles + (size_t)ngroups * nsm * wpt * RPW * 32;  // [kres_max][QC_WARPS][32]
-    T* pnrm = pdot + (size_t)kres_max * QC_WARPS * 32;            // [kres_max][QC_WARPS][32]
-    __shared__ __align__(16) T qs[QC_MAXROWS + RPW];
-    __shared__ T part[QC_WARPS * 32];
+    double* stiles = reinterpret_cast<double*>(qr_smem_raw);  // [ngroups][nsm][wpt][RPW][32]
+    double* pdot = stiles + (size_t)ngroups * nsm * wpt * RPW * 32;  // [nsm][QC_WARPS][32]
+    double* pnrm = pdot + (size_t)nsm * QC_WARPS * 32;            // [nsm][QC_WARPS][32]
+    __shared__ __align__(16) double qs[QC_MAXROWS + RPW];
+    __shared__ double part[QC_WARPS * 32];
     __shared__ double gv[QC_WARPS];
     __shared__ int gi[QC_WARPS];
     __shared__ int wsel[QC_WARPS];
@@ -239,14 +229,13 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
     const int ntiles = (ncol + 31) / 32;
     const int ggroup = blockIdx.x * ngroups + group, total_groups = gridDim.x * ngroups;
     const int ktot = ggroup < ntiles ? (ntiles - ggroup + total_groups - 1) / total_groups : 0;
-    const int kres = min(ktot, kres_max);  // this group's resident tiles
+    const int kres = min(ktot, nsm);  // this group's resident tiles
     const int rbase = wig * RPW;
     const int rows_pad = wpt * RPW;
-    T vr[NREG > 0 ? NREG : 1][RPW];
     // chosen columns among this lane's resident tiles (bit k: resident tile k),
     // kept in a register so that a step reads no global flag for them
     unsigned cmask = 0u;
-    for (int r = threadIdx.x; r < QC_MAXROWS + RPW; r += blockDim.x) qs[r] = T(0);
+    for (int r = threadIdx.x; r < QC_MAXROWS + RPW; r += blockDim.x) qs[r] = 0.0;
     __syncthreads();
     for (int step = 0; step < npiv; ++step) {
         double best = -2.0;
@@ -254,55 +243,34 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
         // resident tiles: all dot partials, one barrier, all updates and norm
         // partials, one barrier, then the argmax over the tiles
         if (step == 0) {
-#pragma unroll
-            for (int k = 0; k < NREG; ++k) {
-                if (k < kres) {
-                    const int c = (ggroup + k * total_groups) * 32 + lane;
-#pragma unroll
-                    for (int j = 0; j < RPW; ++j)
-                        vr[k][j] = (c < ncol && rbase + j < nrow) ? R[(size_t)(rbase + j) * ncol + c] : T(0);
-                    pnrm[(k * QC_WARPS + warp) * 32 + lane] = norm_rows<T, RPW>(vr[k]);
-                }
-            }
-            for (int k = NREG; k < kres; ++k) {
+            for (int k = 0; k < kres; ++k) {
                 const int c = (ggroup + k * total_groups) * 32 + lane;
-                T* st = stiles + ((((size_t)group * nsm + (k - NREG)) * wpt + wig) * RPW) * 32 + lane;
-                T v[RPW];
+                double* st = stiles + ((((size_t)group * nsm + k) * wpt + wig) * RPW) * 32 + lane;
+                double v[RPW];
 #pragma unroll
                 for (int j = 0; j < RPW; ++j) {
-                    v[j] = (c < ncol && rbase + j < nrow) ? R[(size_t)(rbase + j) * ncol + c] : T(0);
+                    v[j] = (c < ncol && rbase + j < nrow) ? R[(size_t)(rbase + j) * ncol + c] : 0.0;
                     st[j * 32] = v[j];
                 }
-                pnrm[(k * QC_WARPS + warp) * 32 + lane] = norm_rows<T, RPW>(v);
+                pnrm[(k * QC_WARPS + warp) * 32 + lane] = norm_rows(v);
             }
         } else {
-#pragma unroll
-            for (int k = 0; k < NREG; ++k)
-                if (k < kres) pdot[(k * QC_WARPS + warp) * 32 + lane] = dot_rows<T, RPW>(vr[k], qs, rbase);
-            for (int k = NREG; k < kres; ++k) {
-                const T* st = stiles + ((((size_t)group * nsm + (k - NREG)) * wpt + wig) * RPW) * 32 + lane;
-                T v[RPW];
+            for (int k = 0; k < kres; ++k) {
+                const double* st = stiles + ((((size_t)group * nsm + k) * wpt + wig) * RPW) * 32 + lane;
+                double v[RPW];
 #pragma unroll
                 for (int j = 0; j < RPW; ++j) v[j] = st[j * 32];
-                pdot[(k * QC_WARPS + warp) * 32 + lane] = dot_rows<T, RPW>(v, qs, rbase);
+                pdot[(k * QC_WARPS + warp) * 32 + lane] = dot_rows(v, qs, rbase);
             }
             if (kres > 0) group_bar(1 + group, wpt * 32);
-#pragma unroll
-            for (int k = 0; k < NREG; ++k) {
-                if (k < kres) {
-                    T dot = T(0);
-                    for (int w = 0; w < wpt; ++w) dot += pdot[(k * QC_WARPS + group * wpt + w) * 32 + lane];
-                    pnrm[(k * QC_WARPS + warp) * 32 + lane] = update_rows<T, RPW>(vr[k], qs, rbase, dot);
-                }
-            }
-            for (int k = NREG; k < kres; ++k) {
-                T* st = stiles + ((((size_t)group * nsm + (k - NREG)) * wpt + wig) * RPW) * 32 + lane;
-                T dot = T(0);
+            for (int k = 0; k < kres; ++k) {
+                double* st = stiles + ((((size_t)group * nsm + k) * wpt + wig) * RPW) * 32 + lane;
+                double dot = 0.0;
                 for (int w = 0; w < wpt; ++w) dot += pdot[(k * QC_WARPS + group * wpt + w) * 32 + lane];
-                T v[RPW];
+                double v[RPW];
 #pragma unroll
                 for (int j = 0; j < RPW; ++j) v[j] = st[j * 32];
-                pnrm[(k * QC_WARPS + warp) * 32 + lane] = update_rows<T, RPW>(v, qs, rbase, dot);
+                pnrm[(k * QC_WARPS + warp) * 32 + lane] = update_rows(v, qs, rbase, dot);
 #pragma unroll
                 for (int j = 0; j < RPW; ++j) st[j * 32] = v[j];
             }
@@ -310,7 +278,7 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
         if (kres > 0) group_bar(1 + group, wpt * 32);
         if (wig == 0) {
             for (int k = 0; k < kres; ++k) {
-                T tot = T(0);
+                double tot = 0.0;
                 for (int w = 0; w < wpt; ++w) tot += pnrm[(k * QC_WARPS + group * wpt + w) * 32 + lane];
                 const int c = (ggroup + k * total_groups) * 32 + lane;
                 const bool live = c < ncol && !((cmask >> k) & 1u);
@@ -318,26 +286,26 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
             }
         }
         // the rest: streamed from and back to global memory, one tile at a time
-        for (int tile = ggroup + kres_max * total_groups; tile < ntiles; tile += total_groups) {
+        for (int tile = ggroup + nsm * total_groups; tile < ntiles; tile += total_groups) {
             const int c = tile * 32 + lane;
             const bool live = c < ncol && !chosen[c];
-            T v[RPW];
+            double v[RPW];
             const bool full = rbase + RPW <= nrow;
             if (full) {
 #pragma unroll
-                for (int j = 0; j < RPW; ++j) v[j] = live ? R[(size_t)(rbase + j) * ncol + c] : T(0);
+                for (int j = 0; j < RPW; ++j) v[j] = live ? R[(size_t)(rbase + j) * ncol + c] : 0.0;
             } else {
 #pragma unroll
                 for (int j = 0; j < RPW; ++j)
-                    v[j] = (live && rbase + j < nrow) ? R[(size_t)(rbase + j) * ncol + c] : T(0);
+                    v[j] = (live && rbase + j < nrow) ? R[(size_t)(rbase + j) * ncol + c] : 0.0;
             }
             if (step > 0) {
-                part[warp * 32 + lane] = dot_rows<T, RPW>(v, qs, rbase);
+                part[warp * 32 + lane] = dot_rows(v, qs, rbase);
                 group_bar(1 + group, wpt * 32);
-                T dot = T(0);
+                double dot = 0.0;
                 for (int w = 0; w < wpt; ++w) dot += part[(group * wpt + w) * 32 + lane];
                 group_bar(1 + group, wpt * 32);
-                part[warp * 32 + lane] = update_rows<T, RPW>(v, qs, rbase, dot);
+                part[warp * 32 + lane] = update_rows(v, qs, rbase, dot);
                 if (live) {
                     if (full) {
 #pragma unroll
@@ -349,11 +317,11 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
                     }
                 }
             } else {
-                part[warp * 32 + lane] = norm_rows<T, RPW>(v);
+                part[warp * 32 + lane] = norm_rows(v);
             }
             group_bar(1 + group, wpt * 32);
             if (wig == 0) {
-                T tot = T(0);
+                double tot = 0.0;
                 for (int w = 0; w < wpt; ++w) tot += part[(group * wpt + w) * 32 + lane];
                 tile_argmax(live ? (double)tot : (c < ncol ? -1.0 : -2.0), c < ncol ? c : 0x7fffffff, best, bidx);
             }
@@ -372,53 +340,32 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
         // publish this CTA's candidate column (its current residual values) and,
         // in slot rows_pad, the inverse of its FP64 norm
         {
-            T* out = pub + ((size_t)(step & 1) * gridDim.x + blockIdx.x) * (rows_pad + 4);
+            double* out = pub + ((size_t)(step & 1) * gridDim.x + blockIdx.x) * (rows_pad + 4);
             const int cb = mybest_sh;
             if (cb >= 0) {
                 const int tile = cb / 32, cl = cb % 32;
                 const int kk = tile / total_groups, gg = tile % total_groups - blockIdx.x * ngroups;
-                T x = T(0);
-                if (kk < NREG) {
-                    // the lane holding the column, in each warp of its group
-                    if (group == gg && lane == cl) {
-#pragma unroll
-                        for (int k = 0; k < NREG; ++k)
-                            if (k == kk) {
-#pragma unroll
-                                for (int j = 0; j < RPW; ++j) out[rbase + j] = vr[k][j];
-                            }
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < rows_pad) x = out[threadIdx.x];
-                } else if (kk < kres_max) {
-                    const T* st = stiles + (((size_t)gg * nsm + (kk - NREG)) * wpt) * RPW * 32 + cl;
+                double x = 0.0;
+                if (kk < nsm) {
+                    const double* st = stiles + (((size_t)gg * nsm + kk) * wpt) * RPW * 32 + cl;
                     if (threadIdx.x < rows_pad) {
                         x = st[(size_t)threadIdx.x * 32];
                         out[threadIdx.x] = x;
                     }
                 } else {
                     if (threadIdx.x < rows_pad) {
-                        x = threadIdx.x < nrow ? R[(size_t)threadIdx.x * ncol + cb] : T(0);
+                        x = threadIdx.x < nrow ? R[(size_t)threadIdx.x * ncol + cb] : 0.0;
                         out[threadIdx.x] = x;
                     }
                 }
-                const int r2 = threadIdx.x + QC_THREADS;
-                T x2 = T(0);
-                if (r2 < rows_pad) {
-                    if (kk < NREG) x2 = out[r2];
-                    else if (kk < kres_max)
-                        x2 = stiles[((((size_t)gg * nsm + (kk - NREG)) * wpt) * RPW + r2) * 32 + cl];
-                    else x2 = r2 < nrow ? R[(size_t)r2 * ncol + cb] : T(0);
-                    if (kk >= NREG) out[r2] = x2;
-                }
-                double s2 = (double)x * (double)x + (double)x2 * (double)x2;
+                double s2 = x * x;
                 for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
                 if (lane == 0) red[warp] = s2;
                 __syncthreads();
                 if (threadIdx.x == 0) {
                     double t = 0.0;
                     for (int w = 0; w < QC_WARPS; ++w) t += red[w];
-                    out[rows_pad] = (T)(t > 0.0 ? 1.0 / sqrt(t) : 0.0);
+                    out[rows_pad] = t > 0.0 ? 1.0 / sqrt(t) : 0.0;
                 }
             }
         }
@@ -452,9 +399,9 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
         __syncthreads();
         const int p = pivot_sh;
         {
-            const T* col = pub + ((size_t)(step & 1) * gridDim.x + winner_sh) * (rows_pad + 4);
+            const double* col = pub + ((size_t)(step & 1) * gridDim.x + winner_sh) * (rows_pad + 4);
             const double inv = (double)col[rows_pad];
-            for (int r = threadIdx.x; r < nrow; r += blockDim.x) qs[r] = (T)((double)col[r] * inv);
+            for (int r = threadIdx.x; r < nrow; r += blockDim.x) qs[r] = col[r] * inv;
         }
         if (threadIdx.x == 0) {
             chosen[p] = 1;
@@ -462,7 +409,7 @@ __global__ void __launch_bounds__(QC_THREADS, 1)
         }
         {
             const int tile = p / 32, gg = tile % total_groups, kk = tile / total_groups;
-            if (gg / ngroups == (int)blockIdx.x && group == gg % ngroups && lane == p % 32 && kk < kres_max)
+            if (gg / ngroups == (int)blockIdx.x && group == gg % ngroups && lane == p % 32 && kk < nsm)
                 cmask |= 1u << kk;
         }
         __syncthreads();
@@ -551,10 +498,9 @@ size_t qrcp_aux_bytes(int nrow, int ncol) {
            std::max(pub_bytes(nrow), qrr::buf_bytes(nrow, ncol));
 }
 
-// The persistent kernel for one (T, RPW, NREG); *ran = false when the rows
-// do not fit its warp layout or the device cannot co-schedule it.
-template <typename T, int RPW, int NREG>
-static cudaError_t qr_persistent_launch(int nrow, int ncol, T* R, int npiv, Best* best, T* pub,
+// The persistent FP64 kernel; *ran = false when the rows do not fit its warp layout
+// or the device cannot co-schedule it.
+static cudaError_t qr_persistent_launch(int nrow, int ncol, double* R, int npiv, Best* best, double* pub,
                                         unsigned char* chosen, int* d_piv, unsigned* bar,
                                         unsigned long long limit_ns, cudaStream_t s, int* launches, bool* ran) {
     *ran = false;
@@ -566,9 +512,9 @@ static cudaError_t qr_persistent_launch(int nrow, int ncol, T* R, int npiv, Best
     int wpt = 2;  // >= 2 keeps the named-barrier ids (1 + group) within 1..8
     while (wpt * RPW < nrow) wpt *= 2;
     if (!coop || wpt > QC_WARPS || nrow > QC_MAXROWS || sms > 304 || 2 * sms > nblocks_cap(ncol) ||
-        (size_t)2 * sms * (wpt * RPW + 4) * sizeof(T) > pub_bytes(nrow))
+        (size_t)2 * sms * (wpt * RPW + 4) * sizeof(double) > pub_bytes(nrow))
         return cudaSuccess;
-    const void* fn = (const void*)qr_persistent_kernel<T, RPW, NREG>;
+    const void* fn = (const void*)qr_persistent_kernel;
     cudaFuncAttributes fa{};
     cudaError_t e;
     if ((e = cudaFuncGetAttributes(&fa, fn))) return e;
@@ -577,21 +523,17 @@ static cudaError_t qr_persistent_launch(int nrow, int ncol, T* R, int npiv, Best
         return e;
     const int ngroups = QC_WARPS / wpt;
     const int ntiles = (ncol + 31) / 32;
-    // no more CTAs than it takes to hold every tile in registers: a small
-    // matrix then syncs fewer CTAs per step and leaves SMs to other work
-    const int ctas = std::min(sms, std::max(1, (ntiles + ngroups * std::max(NREG, 1) - 1) / (ngroups * std::max(NREG, 1))));
+    // no more CTAs than tiles: a small matrix then syncs fewer CTAs per step and
+    // leaves SMs to other work
+    const int ctas = std::min(sms, std::max(1, (ntiles + ngroups - 1) / ngroups));
     const int total_groups = ctas * ngroups;
     const int max_k = (ntiles + total_groups - 1) / total_groups;
-    const size_t tile_bytes = (size_t)wpt * RPW * 32 * sizeof(T);  // one tile slot of one group
-    const size_t red_bytes = (size_t)2 * QC_WARPS * 32 * sizeof(T);  // dot and norm partials of one tile slot
+    const size_t tile_bytes = (size_t)wpt * RPW * 32 * sizeof(double);  // one tile slot of one group
+    const size_t red_bytes = (size_t)2 * QC_WARPS * 32 * sizeof(double);  // dot and norm partials of one tile slot
     const size_t budget = (size_t)std::max(0, optin - (int)fa.sharedSizeBytes - 1024);
-    if constexpr (NREG > 0) {
-        if (budget < NREG * red_bytes) return cudaSuccess;
-    }
-    int nsm = std::max(0, max_k - NREG);
-    nsm = (int)std::min<size_t>((size_t)nsm, (budget - NREG * red_bytes) / (ngroups * tile_bytes + red_bytes));
-    nsm = std::min(nsm, 30 - NREG);  // the per-lane chosen mask has 32 bits
-    const size_t dyn = (size_t)ngroups * nsm * tile_bytes + (size_t)(NREG + nsm) * red_bytes;
+    int nsm = (int)std::min<size_t>((size_t)max_k, budget / (ngroups * tile_bytes + red_bytes));
+    nsm = std::min(nsm, 30);  // the per-lane chosen mask has 32 bits
+    const size_t dyn = (size_t)ngroups * nsm * tile_bytes + (size_t)nsm * red_bytes;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, QC_THREADS, dyn))) return e;
     if (per_sm < 1) return cudaSuccess;
@@ -668,8 +610,7 @@ cudaError_t qrcp_pivots(int nrow, int ncol, T* R, int npiv, int* d_piv, void* au
         };
         e = nrow <= 256 ? go(qr_rounds_launch<8>) : nrow <= 512 ? go(qr_rounds_launch<16>) : go(qr_rounds_launch<32>);
     } else {
-        e = qr_persistent_launch<T, 32, 0>(nrow, ncol, R, npiv, best, pub, chosen, d_piv, bar, wait_limit_ns, s,
-                                          launches, &ran);
+        e = qr_persistent_launch(nrow, ncol, R, npiv, best, pub, chosen, d_piv, bar, wait_limit_ns, s, launches, &ran);
     }
     if (e) return e;
     if (ran) {
