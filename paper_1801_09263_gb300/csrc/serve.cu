@@ -68,7 +68,7 @@ class PairMerger {
         }
     }
 
-    // A REBUILD of grid size n started / left before its exchange step.
+    // A REBUILD of grid size n is to run / left before its exchange step.
     void starting(int n) {
         std::lock_guard<std::mutex> lk(mu_);
         keys_[n].expected++;
@@ -127,7 +127,7 @@ class PairMerger {
     struct Key {
         std::vector<Entry*> pending;
         bool leading = false;
-        int expected = 0;  // REBUILDs of this size started and not yet joined
+        int expected = 0;  // REBUILDs of this size announced and not yet joined
         std::mutex launch_mu;
         cudaStream_t s = nullptr;
         DevBuf refs, sys;
@@ -211,6 +211,17 @@ struct GpuExec {
         return (size_t)b;
     }
 
+    // a REBUILD that can join merged launches counts as expected there until it
+    // joins (or leaves before its exchange step)
+    void announce(const lace_serve::SystemDesc& d, lace_serve::Request& r) const {
+        r.announced = r.kind == lace_serve::REQ_REBUILD ? merge_key(d) : 0;
+        if (r.announced) merger->starting(r.announced);
+    }
+    void withdraw(const lace_serve::SystemDesc&, lace_serve::Request& r) const {
+        if (r.announced) merger->abandoned(r.announced);
+        r.announced = 0;
+    }
+
     int run(const lace_serve::SystemDesc& d, Handle& h, lace_serve::Request& r) {
         const lace_status st = run_calls(d, h, r);
         if (st != LACE_OK) {
@@ -229,8 +240,6 @@ struct GpuExec {
             lace_set_stream(h->ctx, nullptr);
             return st;
         }
-        // a REBUILD that can join merged launches counts as expected there
-        // until it joins (or leaves before its exchange step)
         struct Expect {
             PairMerger* m;
             int key;
@@ -238,8 +247,7 @@ struct GpuExec {
             ~Expect() {
                 if (key && !joined) m->abandoned(key);
             }
-        } expect{merger, merge_key(d)};
-        if (expect.key) merger->starting(expect.key);
+        } expect{merger, r.announced};
         lace_status st = LACE_OK;
         if (!h) h = new SysState();
         if (!h->ctx) {

@@ -18,6 +18,9 @@
 //   void release(Handle&);                                // free the system's memory
 //   int merge_key(const SystemDesc&);                     // REBUILDs of systems with one nonzero key can
 //                                                         // share their pair-convolution launches (0: never)
+//   void announce(const SystemDesc&, Request&);           // optional, with withdraw: the request will run, called for
+//                                                         // all requests of a group before any of them runs
+//   void withdraw(const SystemDesc&, Request&);           // it will, but only after others have
 #pragma once
 
 #include <algorithm>
@@ -62,6 +65,7 @@ struct Request {
     long long n_pairs = 0;
     double e_block = 0.0;  // APPLY: sum_j <data_j| K_ACE |data_j> (set by the executor)
     int rebuild_due = 0;   // APPLY: the inner loop has converged on this projector (see Scheduler)
+    int announced = 0;     // for the executor: what it was announced as
     std::string err;       // what failed (empty when result == 0)
 };
 
@@ -242,6 +246,16 @@ class Scheduler {
 
     static constexpr int kMaxGroup = 8;
 
+    // Executors without the two calls need none.
+    template <class E> static auto announce(E& e, const SystemDesc& d, Request& r, int) -> decltype(e.announce(d, r)) {
+        return e.announce(d, r);
+    }
+    template <class E> static void announce(E&, const SystemDesc&, Request&, long) {}
+    template <class E> static auto withdraw(E& e, const SystemDesc& d, Request& r, int) -> decltype(e.withdraw(d, r)) {
+        return e.withdraw(d, r);
+    }
+    template <class E> static void withdraw(E&, const SystemDesc&, Request&, long) {}
+
     struct Pick {
         std::shared_ptr<Request> r;
         size_t growth;
@@ -342,6 +356,9 @@ class Scheduler {
             rebuilds_running_ += rebuild;  // a group takes one rebuild slot
             if (group.size() > 1) groups_++, grouped_ += (long long)group.size();
             lk.unlock();
+            // all are announced before the first runs: a thread may take longer to start
+            // than a request to its pair convolutions, which then would not wait for it
+            for (size_t k = 0; k < group.size(); ++k) announce(exec_, sys[k]->d, *group[k].r, 0);
             // the companions on threads of their own, the first request here
             std::vector<int> st(group.size(), S_OK);
             std::vector<size_t> held(group.size(), 0);
@@ -354,7 +371,10 @@ class Scheduler {
                 try {
                     helpers.emplace_back(run_one, k);
                 } catch (...) {
-                    run_one(k);  // no thread to be had: one after the other (the merge is then skipped)
+                    // no thread to be had: one after the other, and none waits for those to come
+                    for (size_t j = k; j < group.size(); ++j) withdraw(exec_, sys[j]->d, *group[j].r, 0);
+                    withdraw(exec_, sys[0]->d, *group[0].r, 0);
+                    run_one(k);
                 }
             }
             run_one(0);
