@@ -713,12 +713,19 @@ cudaError_t tc_combine(int N, size_t K, int Kc, const float* A, size_t lda, cons
     if (N <= 0 || K == 0) return cudaSuccess;
     // rows that TMA can read: 32 orbitals a step, tiles of 128 targets where
     // these are all and 256 beyond (72^3 x 256: 199 us against 257, for a cut and
-    // its hand-offs of half as many steps); others: 64 and 256
+    // its hand-offs of half as many steps); others: 64 and 256.  Up to 64 targets
+    // of so many orbitals that the coefficients of 128 are not resident (an ACE apply
+    // to a small block): tiles of 64, whose coefficients are up to 576 orbitals (96^3 x 299
+    // on 6: 478 -> 340 us, on 64 484 -> 391; copied again for every tile they
+    // were slower than the kernel before, 408 us on 6).  Where 128 are resident the wider
+    // tile is as fast (72^3 x 256 on 64: 152 and 151 us, 96^3 x 160 221 and 232).
     CUtensorMap map_a;
     const bool tma = Kc > 0 && K <= 0x7fffffffull &&
                      make_map(&map_a, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, sizeof(float), A, (size_t)Kc, K, lda, TC_M, CW_BK,
                               CU_TENSOR_MAP_SWIZZLE_NONE);
-    const int bk = tma ? CW_BK : TC_BK, nt = tma && N <= TC_N ? TC_N : CB_N;
+    const bool few = tma && sizeof(TO) == 8 && N <= 64 &&
+                     (Kc + CW_BK - 1) / CW_BK > CombineShape<Bf16Slices, TC_N>::BSTAGES;
+    const int bk = tma ? CW_BK : TC_BK, nt = few ? 64 : tma && N <= TC_N ? TC_N : CB_N;
     const int kpad = (Kc + bk - 1) / bk * bk, npad = (N + nt - 1) / nt * nt;
     __nv_bfloat16* hiT = static_cast<__nv_bfloat16*>(scratch);
     __nv_bfloat16* loT = hiT + (size_t)kpad * npad;
@@ -727,7 +734,9 @@ cudaError_t tc_combine(int N, size_t K, int Kc, const float* A, size_t lda, cons
     coef_split_kernel<<<(tot + 255) / 256, 256, 0, s>>>(Kc, N, Coef, ldcoef, kpad, npad, hiT, loT);
     cudaError_t e = cudaSuccess;
     bool done = false;
-    if (tma)
+    if constexpr (sizeof(TO) == 8)
+        if (few) e = combine_ws<64>(map_a, N, K, kpad, npad, hiT, (float)beta, Out, ldo, d_err, &done, s);
+    if (tma && !few)
         e = nt == TC_N ? combine_ws<TC_N>(map_a, N, K, kpad, npad, hiT, (float)beta, Out, ldo, d_err, &done, s)
                        : combine_ws<CB_N>(map_a, N, K, kpad, npad, hiT, (float)beta, Out, ldo, d_err, &done, s);
     if (e) return e;
