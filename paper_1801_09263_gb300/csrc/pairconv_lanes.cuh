@@ -652,8 +652,22 @@ struct OncePerDevice {
     }
 };
 
-template <int N> bool launch_cube(int pass, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
-    constexpr int NT = plane_threads(N, N), RG = regs_at(NT, plane_ctas(N, N));
+// Threads of a plane pass whose launch does not fill the SMs (the exchange of a few
+// pairs): a CTA's chain of stages is all that counts then, and a thread a butterfly
+// of most stages makes it shortest, with two CTAs an SM up to 384 threads and one beyond.
+// Pass A and C of one grid, us: 48^3 8.2 and 9.1 -> 6.1 and 7.3 (128 -> 288 threads), 64^3 9.2
+// and 10.5 -> 6.7 and 7.7, 96^3 13.2 and 14.7 -> 9.8 and 11.4; of five grids at
+// 48^3 (240 CTAs) 8.6 and 11.1 -> 6.7 and 9.0.  Launches that do not fit at once are
+// slower with it (48^3, eight grids: 12.6 -> 14.4), and below 40 points an axis the
+// stages have no more items than the narrow CTA has threads.
+constexpr int wide_threads(int n) {
+    const int t = n < 40 ? 0 : (n * n / 8 + 31) / 32 * 32;
+    return t > 768 ? 768 : t;
+}
+constexpr int wide_ctas(int n) { return wide_threads(n) <= 384 ? 2 : 1; }
+
+template <int N, int NT, int CTAS> void launch_cube_as(int pass, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
+    constexpr int RG = regs_at(NT, CTAS);
     constexpr size_t sm = plane_smem(N, N);
     static OncePerDevice once;
     once.run([&] {
@@ -662,6 +676,19 @@ template <int N> bool launch_cube(int pass, int nb, const ConvArgs<float>& P, in
     });
     if (pass == 0) cube_a<N, NT, RG><<<dim3(nb, N), NT, sm, s>>>(P, g0);
     else cube_c<N, NT, RG><<<dim3(nb, N), NT, sm, s>>>(P, g0);
+}
+template <int N> bool launch_cube(int pass, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
+    constexpr int NT = plane_threads(N, N), WIDE = wide_threads(N);
+    if constexpr (WIDE > NT) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if ((long long)nb * N <= (long long)wide_ctas(N) * sms) {
+            launch_cube_as<N, WIDE, wide_ctas(N)>(pass, nb, P, g0, s);
+            return true;
+        }
+    }
+    launch_cube_as<N, NT, plane_ctas(N, N)>(pass, nb, P, g0, s);
     return true;
 }
 template <int N> bool launch_slab(int M, int nb, const ConvArgs<float>& P, int g0, cudaStream_t s) {
