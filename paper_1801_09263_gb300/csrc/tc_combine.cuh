@@ -32,7 +32,13 @@ constexpr int CW_A_COLS = CW_BK / 2;            // TMEM columns of a slice of A
 // products, SCALED (powers of two on rows and targets).
 template <class S, int NT> struct CombineShape {
     static constexpr int B_TILE = NT * CW_BK * 2, B_BYTES = S::SLICES * B_TILE;
-    static constexpr int ASTAGES = 5;
+    // Stages of rows: an even number, so that a stage passes between steps of one set of
+    // cut warps (below).  With five, a set could wait for a stage whose rows of the other
+    // set's step had not landed: a wait knows only the parity of a phase, took the phase
+    // before last for the awaited one, and the stage was read with other rows and freed early
+    // (rows landing out of order by two steps, so under load from other streams).  Six are as
+    // fast as five were, four up to 4% slower (80^3 x 512 -> 128: 454, 462, 488 us).
+    static constexpr int ASTAGES = 6;
     static constexpr int BSTAGES = (227 * 1024 - 1536 - ASTAGES * CW_A32_BYTES) / B_BYTES;
     static constexpr int SMEM = BSTAGES * B_BYTES + ASTAGES * CW_A32_BYTES + 1024;
     // TMEM columns: the accumulators, then up to four stages of A's slices
@@ -43,7 +49,7 @@ template <class S, int NT> struct CombineShape {
         (1u << 4) | (S::FORMAT << 7) | (S::FORMAT << 10) | ((uint32_t)(NT >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
     static_assert(SMEM <= 227 * 1024 - 512, "one CTA an SM");
     static_assert(TSTAGES >= 2 && TSTAGES % 2 == 0 && CW_BK == 16 * (CW_CUT_WARPS / 8), "slice stages; 16 orbitals a thread");
-    static_assert(ASTAGES > CW_AHEAD, "rows ahead");
+    static_assert(ASTAGES > CW_AHEAD && ASTAGES % 2 == 0, "rows ahead; the steps of a set alone in a stage");
 };
 
 // D (FP32) += A B^T with A in TMEM (a point a lane, two orbitals a 32-bit column).

@@ -715,8 +715,8 @@ cudaError_t tc_combine(int N, size_t K, int Kc, const float* A, size_t lda, cons
     // these are all and 256 beyond (72^3 x 256: 199 us against 257, for a cut and
     // its hand-offs of half as many steps); others: 64 and 256.  Up to 64 targets
     // of so many orbitals that the coefficients of 128 are not resident (an ACE apply
-    // to a small block): tiles of 64, whose coefficients are up to 576 orbitals (96^3 x 299
-    // on 6: 478 -> 340 us, on 64 484 -> 391; copied again for every tile they
+    // to a small block): tiles of 64, whose coefficients are up to 512 orbitals (96^3 x 299
+    // on 6: 478 -> 340 us, on 64 484 -> 389; copied again for every tile they
     // were slower than the kernel before, 408 us on 6).  Where 128 are resident the wider
     // tile is as fast (72^3 x 256 on 64: 152 and 151 us, 96^3 x 160 221 and 232).
     CUtensorMap map_a;

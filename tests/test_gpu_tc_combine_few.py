@@ -1,7 +1,7 @@
 """Tensor-core combinations to few targets: tiles of 64 where 128 would not be resident.
 
-Around the line (288 and 289 orbitals, 64 and 65 targets), past the orbitals whose coefficients
-are resident in tiles of 64 (576 and 577), one target, point counts with and without a
+Around the line (256 and 257 orbitals; 64 and 65 targets), past the orbitals whose coefficients
+are resident in tiles of 64 (512 and 513), one target, point counts with and without a
 remainder of 128; against FP64.
 
 Tolerance: two BF16 slices hold an operand to 2^-17 and the dropped product of the low slices
@@ -18,7 +18,7 @@ from paper_1801_09263_gb300 import binding as B
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_orb", [288, 289, 299, 576, 577, 1030])
+@pytest.mark.parametrize("n_orb", [256, 257, 288, 289, 299, 512, 513, 576, 577, 1030])
 @pytest.mark.parametrize("n_targets", [1, 6, 63, 64, 65])
 @pytest.mark.parametrize("points", [128 * 160, 128 * 153 + 4])
 def test_few_targets_match_fp64(n_orb, n_targets, points):
