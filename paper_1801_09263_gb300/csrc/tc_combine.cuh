@@ -190,10 +190,16 @@ __global__ void __launch_bounds__(CW_THREADS, 1)
                         mma_ta<C::IDESC>(acc, a + i * CW_A_COLS + kk * 8, sw64_desc(bb + kk * 32 + j * C::B_TILE), first);
                     });
                 mma_commit(&mma_bar[b]);
-                mma_commit(&empty_b[sb]);
+                if (!resident) mma_commit(&empty_b[sb]);
                 if (step == nsteps - 1) mma_commit(&tile_bar);
                 committed = g + 1;
             }
+            // The commits of a step may arrive in any order: none may be on its way when
+            // the CTA leaves (the others are waited for by the next users of their stages).
+            for (int g = max(0, committed - C::TSTAGES); g < committed; ++g)
+                mbar_wait(&mma_bar[g % C::TSTAGES], (uint32_t)(g / C::TSTAGES) & 1);
+            for (int g = max(0, committed - C::BSTAGES); g < committed && !resident; ++g)
+                mbar_wait(&empty_b[g % C::BSTAGES], (uint32_t)(g / C::BSTAGES) & 1);
         }
     } else {
         const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
@@ -283,15 +289,13 @@ __global__ void __launch_bounds__(CW_THREADS, 1)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (abort_sh) {
-        // copies still landing, MMAs still running (bounded waits)
+        // copies still landing (bounded waits; the MMAs are done)
         if (warp == CW_CUT_WARPS && lane == 0) {
             for (int s = 0; s < C::ASTAGES; ++s)
                 if (last_a[s] >= 0) mbar_wait(&full_a[s], (uint32_t)(last_a[s] / C::ASTAGES) & 1);
             for (int s = 0; s < C::BSTAGES; ++s)
                 if (last_b[s] >= 0) mbar_wait(&full_b[s], (uint32_t)(last_b[s] / C::BSTAGES) & 1);
         }
-        if (warp == CW_CUT_WARPS + 1 && lane == 0 && committed > 0)
-            mbar_wait(&mma_bar[(committed - 1) % C::TSTAGES], (uint32_t)((committed - 1) / C::TSTAGES) & 1);
         if (threadIdx.x == 0) atomicExch(err, 1);
     }
     __syncthreads();
